@@ -378,7 +378,7 @@ static int align_up(int v, int a) { return (v + a - 1) / a * a; }
 // while the plain variant leaves the GPU short of blocks.
 static bool tune_eligible(const cc_ctx *c, int tkind, const long long *blocks, int v)
 {
-    if (tkind == TK_TAUMIX && TAU_VAR_S[v] > 1) return blocks[0] < 16ll * c->nsm;
+    if (tkind == TK_TAUMIX && v == TAU_VAR_SMALL) return blocks[0] < 16ll * c->nsm;
     if (tkind == TK_MK && MK_VAR_SLICE[v] > 1) return blocks[0] < 8ll * c->nsm;
     return true;
 }
@@ -472,7 +472,7 @@ static int ensure_level(cc_ctx *c, LevelAlloc &a, int need, int nsets)
         const long long worst = std::min<long long>(2 * (long long)c->n + 64, 0x3fffffff);
         int cap = align_up(std::max<int>(need, (int)std::max<long long>(64, worst)), 64);
         size_t nd = (size_t)cap + PAD_TAIL;
-        size_t bytes = nd * 8 * 7 + (nd * 11 + 4) * 4 + nd * 64 + 4096;
+        size_t bytes = nd * 8 * 7 + (nd * 11 + 4) * 4 + nd * 88 + 4096;
         if (cudaMalloc(&a.block, bytes) != cudaSuccess) {
             cudaGetLastError();
             return fail(c, CC_E_NOMEM, "device allocation failed (level buffer)");
@@ -497,6 +497,7 @@ static int ensure_level(cc_ctx *c, LevelAlloc &a, int need, int nsets)
         a.info_cap = (int)nd;
         a.F.pq = (float4 *)q; q += nd * 32;
         a.F.vq = (float4 *)q; q += nd * 32;
+        a.F.hp = (float4 *)q; q += nd * 24;
         a.F.maxes = (float *)q;
         a.F.cap = (int)nd;
         a.cap = cap;
@@ -1818,7 +1819,7 @@ int cc_timestep_graph(cc_ctx *c, const int32_t *set, int64_t n_set, double h, in
     Level UL = u.L;
     UL.tile_off = u.tau_off[TAU_VAR_128];  // 128-wide tiles
     launch_init_parent(u.L, nullptr, c->stream);
-    launch_tau_hook(UL, (int)(nt * (nt + 1) / 2), P, TAU_VAR_128, c->d_ctr, nullptr, 0, c->d_near_ij,
+    launch_tau_hook(UL, (int)(nt * (nt + 1) / 2), P, c->d_ctr, nullptr, 0, c->d_near_ij,
                     c->d_near_tau, c->near_cap, c->stream);
     DevCounters h1;
     CC_CUDA(c, cudaMemcpyAsync(&h1, c->d_ctr, sizeof(h1), cudaMemcpyDeviceToHost, c->stream));
@@ -1838,7 +1839,7 @@ int cc_timestep_graph(cc_ctx *c, const int32_t *set, int64_t n_set, double h, in
         void *ss = (void *)(de + 2 * ne);
         CC_TRY(reset_call_counters(c));
         launch_init_parent(u.L, nullptr, c->stream);
-        launch_tau_hook(UL, (int)(nt * (nt + 1) / 2), P, TAU_VAR_128, c->d_ctr, de, ne, c->d_near_ij,
+        launch_tau_hook(UL, (int)(nt * (nt + 1) / 2), P, c->d_ctr, de, ne, c->d_near_ij,
                         c->d_near_tau, c->near_cap, c->stream);
         int bits = 0;
         while (bits < 31 && (1ll << bits) <= c->n) ++bits;

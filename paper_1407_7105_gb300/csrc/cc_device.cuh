@@ -32,6 +32,9 @@ constexpr float SLACK = 2e-6f;
 struct MixedTauParams {
     float eta, etah, eps2, G;
     float hq;  // eta/etah (h, or h/eta when eta multiplies the min): the pre-test's q = hq |dv|/r
+    // tau_pair_bounds' constants (mixed_tau_params): c^2, T, V of the bounds
+    // below; pb_c2 < 0: the bounds are off
+    float pb_c2, pb_r3, pb_v;
 };
 
 // The h-independent part of the decision: everything except T/h.  The
@@ -215,6 +218,68 @@ __device__ __forceinline__ bool tau_groups_apart(const GroupBox &A, const GroupB
     const float vt = vm * 1.0001f + 4.f * pad_v;
     vthr2 = vt * vt;
     return true;
+}
+
+// The same two bounds for single pairs of the groups, as three comparisons on
+// r~^2 and |dv~|^2 (no square root, no division): with T_ff/h = etah
+// sqrt(r^3/mu), f(r, v) as above and mu <= mu_max,
+//   (3) r >= c v,  c = M (2 + eta) / (2 etah (1 - D)):  the first term of the
+//       flyby's denominator takes the share 1 - D of its numerator, and q =
+//       hq v/r <= hq/c;
+//   (1) r >= r_min, r_min^3 = mu_max T^2, T = M/(etah (1 - 0.75 M hq/c)):
+//       free fall at that q;
+//   (2) v >= v_thr = V mu_max/r_min^2, V = M eta/(2 etah D): the flyby's second
+//       term takes the share D.
+// M = 1.02 covers the FP32 rounding and the high parts': r_min >= 1.02e3 c_x
+// and v_thr >= 1.02e3 c_v (c_x = 7.1 u max|x_i|, c_v likewise) put the
+// relative error of r~ and v~ below 1e-3 + 4.5u, of r^2 v below 4e-3.
+// The kernel forms p = r~^2 - r_min^2 and w = v~^2 - v_thr^2 by starting
+// their sums at -r_min^2 (+ eps^2) and -v_thr^2, and asks for w >= 0 and p -
+// c^2 w >= 0: that is (3) with r_min^2 - c^2 v_thr^2 to spare (r_min is
+// raised until it is not negative), and it implies (1).  Returns false when
+// the bounds cannot be used (the caller then leaves every pair open); the
+// caller has seen that all |x|, |v| are below TAU_WILD, so no sum overflows.
+constexpr float TAU_WILD = 1e15f;
+struct PairBounds {
+    float p0, w0;  // eps^2 - r_min^2, -v_thr^2
+};
+
+__device__ __forceinline__ bool tau_pair_bounds(float amax, float vabs, float mu_max, const MixedTauParams &Q,
+                                                PairBounds &b)
+{
+    const float mu = mu_max * 1.0001f;
+    const float r3 = mu * Q.pb_r3;
+    // r_min by exp2(log2/3): the approximations' error is far inside 5e-4
+    float rmin = 1.0005f * exp2f(__log2f(r3) * (1.f / 3.f));
+    rmin = fmaxf(rmin, fmaxf(1.02e3f * 7.1f * U32 * amax, 1e-15f));
+    float vt = fmaxf(1.0001f * Q.pb_v * mu / (rmin * rmin), fmaxf(1.02e3f * 7.1f * U32 * vabs, 1e-15f));
+    const float w2 = vt * vt, p2 = fmaxf(rmin * rmin, 1.0001f * Q.pb_c2 * w2);
+    b.p0 = Q.eps2 - p2;
+    b.w0 = -w2;
+    return Q.pb_c2 >= 0.f && r3 > 1e-36f && r3 < 1e36f && w2 < 1e30f && p2 < 1e30f;
+}
+
+// the FP32 constants of a split at threshold P.h
+inline MixedTauParams mixed_tau_params(const TauParams &P)
+{
+    MixedTauParams Q;
+    const double etah = P.eta_outside ? P.eta_in * P.eta / P.h : P.eta_in / P.h;
+    const double hq = P.eta_outside ? P.h / P.eta : P.h;  // h/eta_in in the units of T: eta_in/etah
+    Q.eta = (float)P.eta_in;
+    Q.etah = (float)etah;
+    Q.eps2 = (float)P.eps2;
+    Q.G = (float)P.G;
+    Q.hq = (float)hq;
+    // D: a 3 % tighter (3) at the usual eta; more where eta is not small
+    const double M = 1.02, D = fmax(1.0 / 32, 0.75 * P.eta_in / (2.0 + P.eta_in));
+    const double c = M * (2.0 + P.eta_in) / (2.0 * etah * (1.0 - D));
+    const double q = hq / c, T = M / (etah * (1.0 - 0.75 * M * q));
+    Q.pb_c2 = (float)(c * c * 1.0001);
+    Q.pb_r3 = (float)(T * T * 1.0001);
+    Q.pb_v = (float)(M * P.eta_in / (2.0 * etah * D) * 1.0001);
+    // (q >= 4/(3M) has no free-fall bound; constants outside the float range)
+    if (!(0.75 * M * q < 0.95) || !(Q.pb_c2 < 1e30f) || !(Q.pb_r3 < 1e36f) || !(Q.pb_v < 1e36f)) Q.pb_c2 = -1.f;
+    return Q;
 }
 
 __device__ __forceinline__ int tau_decide_fp32(float dx0, float dx1, float dx2, float dv0, float dv1, float dv2,

@@ -43,9 +43,11 @@ struct Level {
 //   pq[2k] = (x_hi, y_hi, z_hi, G m),  pq[2k+1] = (x_lo, y_lo, z_lo, 0)
 //   vq[2k] = (vx_hi, vy_hi, vz_hi, 0), vq[2k+1] = (vx_lo, vy_lo, vz_lo, 0)
 // with hi = fl32(x), lo = fl32(x - hi); maxes = max |x|, max |v| of the
-// level (float bit patterns, for the error bounds)
+// level (float bit patterns, for the error bounds).  hp holds the high parts
+// once more for the tau kernel's packed pair loop, two bodies together:
+//   hp[3p], [3p+1], [3p+2] = (x x' y y') (z z' vx vx') (vy vy' vz vz'), k = 2p, 2p+1
 struct FFView {
-    float4 *pq, *vq;
+    float4 *pq, *vq, *hp;
     float *maxes;
     int cap;
 };
@@ -287,21 +289,22 @@ extern unsigned long long g_launches;
 
 // cc_pair.cu
 void launch_init_parent(const Level &L, unsigned long long *edge_count, cudaStream_t s);
-// tunable launch shapes (variant index): tau tiles {64, 128, 64 in two
-// column slices}; FP64 kick tiles {32, 64, 128}; mixed kick (j-chunk in
+// tunable launch shapes (variant index): tau tiles {128, 256, 64, the first
+// and last in two column slices}; FP64 kick tiles {32, 64, 128}; mixed kick (j-chunk in
 // tiles of 128, column slices) {(1, 1), (4, 1), (1, 4)}
 constexpr int N_TAU_VAR = 3, N_K64_VAR = 3, N_MK_VAR = 3;
 // tau variants: tile edge T and column slices S per tile row (the FP64
-// kernel takes the first two)
-constexpr int TAU_VAR_T[N_TAU_VAR] = {64, 128, 64};
-constexpr int TAU_VAR_S[N_TAU_VAR] = {1, 1, 2};
-constexpr int N_TAU64_VAR = 2, TAU_VAR_128 = 1;
-static_assert(TAU_VAR_T[TAU_VAR_128] == 128 && TAU_VAR_S[TAU_VAR_128] == 1, "128-wide tau tiles");
+// kernels run on the 128-wide tiles)
+constexpr int TAU_VAR_T[N_TAU_VAR] = {128, 256, 64};
+constexpr int TAU_VAR_S[N_TAU_VAR] = {2, 1, 2};
+constexpr int TAU_VAR_SMALL = 2;  // the shape for sets with few tiles
+constexpr int N_TAU64_VAR = 2, TAU_VAR_128 = 0;
+static_assert(TAU_VAR_T[TAU_VAR_128] == 128, "128-wide tau tiles");
 constexpr int K64_VAR_T[N_K64_VAR] = {32, 64, 128};
 constexpr int MK_VAR_CHUNK[N_MK_VAR] = {1, 4, 1};
 constexpr int MK_VAR_SLICE[N_MK_VAR] = {1, 1, 4};
 constexpr int MK_TILE = 128;
-void launch_tau_hook(const Level &L, int ntiles, const TauParams &P, int variant, DevCounters *ctr,
+void launch_tau_hook(const Level &L, int ntiles, const TauParams &P, DevCounters *ctr,
                      int32_t *edges, long long edge_cap, int32_t *near_ij, double *near_tau, long long near_cap,
                      cudaStream_t s, const EdgeList *rec = nullptr);
 // first-half split from the parent split's edge records: the records that

@@ -44,6 +44,7 @@ __global__ void k_prep_ff(Level L, FFView F, float G, int with_v, int init_fores
         }
         F.pq[2 * k] = make_float4(hi[0], hi[1], hi[2], G * fl32(L.m[k]));
         F.pq[2 * k + 1] = make_float4(lo[0], lo[1], lo[2], 0.f);
+        const float xh[3] = {hi[0], hi[1], hi[2]};
         if (with_v) {
             const double vs[3] = {L.vx[k], L.vy[k], L.vz[k]};
 #pragma unroll
@@ -53,6 +54,12 @@ __global__ void k_prep_ff(Level L, FFView F, float G, int with_v, int init_fores
             }
             F.vq[2 * k] = make_float4(hi[0], hi[1], hi[2], 0.f);
             F.vq[2 * k + 1] = make_float4(lo[0], lo[1], lo[2], 0.f);
+            float *h = reinterpret_cast<float *>(F.hp) + (size_t)(k >> 1) * 12 + (k & 1);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                h[2 * c] = xh[c];
+                h[6 + 2 * c] = hi[c];
+            }
         }
     }
     // positive floats order like their bit patterns
@@ -112,26 +119,84 @@ void launch_prep_kick(const Level &L, const FFView &F, const int32_t *order, con
     CC_COUNT_LAUNCH(1);
 }
 
+// ------------------------------------------------------------ tau
+// One block per triangular tile (T x T pairs) of a set: each warp holds 32 R
+// rows (R per lane) against T/S columns of the tile (S > 1 splits the
+// columns over more warps, for sets with few tiles).
+//
+// What bounds it: the FP32 pipes.  The certificates are three comparisons a
+// pair (tau_pair_bounds: no square root; 13 FP32 operations against ~35 and
+// three reciprocal square roots for tau_quick_apart), formed for two columns
+// at a time with the packed FP32 instructions (add/fma .f32x2: one issue slot
+// for two pairs), so a pair costs ~10 issue slots; the comparisons' outcomes
+// are the sign bits of two sums, shifted into a 32-column mask per lane, so
+// there is no vote and no branch per column.  Pairs left open are queued per
+// warp and settled 32 at a time by the certified decision.
+// Measured (GB300): top level of the 16384-body Plummer sphere (1.34e8 pairs)
+// 252 -> 126 us, 65536-body fractal (2.1e9 pairs) 1798 -> 807 us, 40009 bodies
+// in no spatial order (8.0e8 pairs) 1790 -> 630 us, before -> after the
+// comparisons took the place of tau_quick_apart.  In a spatial order the
+// launch ends with the tiles on the diagonal, whose pairs are mostly edges:
+// four warps a 128-wide tile (S = 2) instead of two took the 16384-body level
+// from 196 to 126 us.
+// RAW: the set is a caller's FP64 arrays (L.x .. L.m, L.total bodies, no
+// float-float copy): columns and rows are rounded as they are loaded.
+constexpr int TAU_JG = 8;  // columns per group of the group certificates
 
-constexpr int TAU_JG = 8;  // columns per group of the group certificates (rows: a warp's 32)
-
-template <int T, int S>
+template <int T, int S, int R>
 struct __align__(16) MixedTauSmem {
-    float4 pq[2 * T];   // positions (hi, Gm), (lo) of the j-tile
-    float4 vq[2 * T];   // velocities (hi), (lo)
-    int32_t lp[2 * T];  // local union-find over the tile's particles
-    uint32_t q[T * S / 32][64];  // per warp: pairs waiting for the certified decision
-    uint32_t om[T * S / 32][T / S];       // per warp and column: lanes whose pair is still open
-    uint32_t cm[T * S / 32][T / S / 32];  // per warp and 32 columns: columns with open pairs
-    GroupBox jb[T / TAU_JG];               // boxes of the j-tile's TAU_JG-column groups
-    float gthr[T * S / 32][T / S / TAU_JG];  // per warp and column group: |dv~|^2 threshold, < 0: none
+    static constexpr int W = T * S / (32 * R);  // warps
+    float4 hp[3 * T / 2];                       // high parts of the j-tile, two bodies together (FFView::hp)
+    int32_t lp[2 * T];                          // local union-find over the tile's particles
+    uint32_t q[W][64];                          // per warp: pairs waiting for the certified decision
+    uint32_t ent[W][128];                       // per warp: edges waiting to be recorded, and their tau
+    double tau[W][128];
+    GroupBox jb[T / TAU_JG];                    // boxes of the j-tile's TAU_JG-column groups
+    float4 gq[W][T / S / TAU_JG];               // per warp and column group: p0, w0, what to do (TauKind), mu
     uint64_t bar;
 };
 
-// min / max over each aligned segment of W lanes
+enum TauKind : int { TAU_BOUNDS = 0, TAU_SPEED = 1, TAU_OPEN = 2 };
+
+// two packed FP32 values; the operations round each half as the scalar ones do
+__device__ __forceinline__ uint64_t pack2(float a, float b)
+{
+    uint64_t v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(a), "f"(b));
+    return v;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float &a, float &b)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
+{
+    uint64_t d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b)
+{
+    uint64_t d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
+{
+    uint64_t d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+
+// min / max over each aligned segment of W lanes (a whole warp: one
+// instruction)
 template <int W>
 __device__ __forceinline__ float warp_min(float v)
 {
+    if constexpr (W == 32) {
+        asm volatile("redux.sync.min.f32 %0, %0, 0xffffffff;" : "+f"(v));
+        return v;
+    }
 #pragma unroll
     for (int o = W / 2; o > 0; o >>= 1) v = fminf(v, __shfl_xor_sync(0xffffffffu, v, o));
     return v;
@@ -140,41 +205,61 @@ __device__ __forceinline__ float warp_min(float v)
 template <int W>
 __device__ __forceinline__ float warp_max(float v)
 {
+    if constexpr (W == 32) {
+        asm volatile("redux.sync.max.f32 %0, %0, 0xffffffff;" : "+f"(v));
+        return v;
+    }
 #pragma unroll
     for (int o = W / 2; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
     return v;
 }
 
-// box of the high parts held by the lanes with `on` in each aligned segment
-// of W lanes (p = (x, y, z, G m), v = (vx, vy, vz)); returns false if no
-// lane of the segment is on
+// widens box B to the boxes of all lanes of each aligned segment of W lanes
+// (a lane without a body brings an empty box: +-inf, Gm = 0)
 template <int W>
-__device__ __forceinline__ bool warp_group_box(bool on, float4 p, float4 v, GroupBox &B)
+__device__ __forceinline__ void warp_group_box(GroupBox &B)
 {
-    const float inf = __int_as_float(0x7f800000);
-    B.xlo[0] = warp_min<W>(on ? p.x : inf);
-    B.xlo[1] = warp_min<W>(on ? p.y : inf);
-    B.xlo[2] = warp_min<W>(on ? p.z : inf);
-    B.xhi[0] = warp_max<W>(on ? p.x : -inf);
-    B.xhi[1] = warp_max<W>(on ? p.y : -inf);
-    B.xhi[2] = warp_max<W>(on ? p.z : -inf);
-    B.vlo[0] = warp_min<W>(on ? v.x : inf);
-    B.vlo[1] = warp_min<W>(on ? v.y : inf);
-    B.vlo[2] = warp_min<W>(on ? v.z : inf);
-    B.vhi[0] = warp_max<W>(on ? v.x : -inf);
-    B.vhi[1] = warp_max<W>(on ? v.y : -inf);
-    B.vhi[2] = warp_max<W>(on ? v.z : -inf);
-    B.gm = warp_max<W>(on ? p.w : 0.f);
     float a = 0.f, b = 0.f;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
+        B.xlo[k] = warp_min<W>(B.xlo[k]);
+        B.xhi[k] = warp_max<W>(B.xhi[k]);
+        B.vlo[k] = warp_min<W>(B.vlo[k]);
+        B.vhi[k] = warp_max<W>(B.vhi[k]);
         a = fmaxf(a, fmaxf(fabsf(B.xlo[k]), fabsf(B.xhi[k])));
         b = fmaxf(b, fmaxf(fabsf(B.vlo[k]), fabsf(B.vhi[k])));
     }
+    B.gm = warp_max<W>(B.gm);
     B.amax = a;
     B.vabs = b;
-    const unsigned seg = (W == 32 ? 0xffffffffu : ((1u << W) - 1u)) << ((threadIdx.x & 31) & ~(W - 1));
-    return (__ballot_sync(0xffffffffu, on) & seg) != 0u;
+}
+
+__device__ __forceinline__ void box_empty(GroupBox &B)
+{
+    const float inf = __int_as_float(0x7f800000);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        B.xlo[k] = B.vlo[k] = inf;
+        B.xhi[k] = B.vhi[k] = -inf;
+    }
+    B.gm = 0.f;
+}
+
+// adds one body to box B; returns whether it is outside what the bounds
+// allow for (TAU_WILD, a mass that is not positive and finite, NaN)
+__device__ __forceinline__ bool box_add(GroupBox &B, const float s[6], float gm)
+{
+    bool in = gm > 0.f && gm < 1e30f;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        B.xlo[k] = fminf(B.xlo[k], s[k]);
+        B.xhi[k] = fmaxf(B.xhi[k], s[k]);
+        B.vlo[k] = fminf(B.vlo[k], s[3 + k]);
+        B.vhi[k] = fmaxf(B.vhi[k], s[3 + k]);
+        in = in && fabsf(s[k]) < TAU_WILD && fabsf(s[3 + k]) < TAU_WILD;
+    }
+    B.gm = fmaxf(B.gm, gm);
+    return !in;
 }
 
 // local union-find in shared memory (indices 0..2T-1, links to the smaller)
@@ -204,18 +289,64 @@ __device__ __forceinline__ bool luf_union(int32_t *p, int a, int b)
     return false;
 }
 
+// the high parts of body k and its G m
+template <bool RAW>
+__device__ __forceinline__ void tau_load_hi(const Level &L, const FFView &F, const MixedTauParams &Q, int k,
+                                            float s[6], float &gm)
+{
+    if constexpr (RAW) {
+        s[0] = fl32(L.x[k]); s[1] = fl32(L.y[k]); s[2] = fl32(L.z[k]);
+        s[3] = fl32(L.vx[k]); s[4] = fl32(L.vy[k]); s[5] = fl32(L.vz[k]);
+        gm = Q.G * fl32(L.m[k]);
+    } else {
+        const float4 p = F.pq[2 * k], v = F.vq[2 * k];
+        s[0] = p.x; s[1] = p.y; s[2] = p.z;
+        s[3] = v.x; s[4] = v.y; s[5] = v.z;
+        gm = p.w;
+    }
+}
+
+// the certified decision of one pair from its float-float differences
+template <bool RAW>
+__device__ __forceinline__ int tau_decide_pair(const Level &L, const FFView &F, const MixedTauParams &Q, int i, int j)
+{
+    constexpr float c11 = 11.f * U32 * U32;
+    if constexpr (RAW) {
+        const double *src[6] = {L.x, L.y, L.z, L.vx, L.vy, L.vz};
+        float d[6], big[2] = {0.f, 0.f};
+#pragma unroll
+        for (int c = 0; c < 6; ++c) {
+            float ih, il, jh, jl;
+            ff_split(src[c][i], ih, il);
+            ff_split(src[c][j], jh, jl);
+            d[c] = (jh - ih) + (jl - il);
+            big[c / 3] = fmaxf(big[c / 3], fmaxf(fabsf(ih), fabsf(jh)));
+        }
+        return tau_decide_fp32(d[0], d[1], d[2], d[3], d[4], d[5], Q.G * fl32(L.m[i]) + Q.G * fl32(L.m[j]),
+                               c11 * big[0], c11 * big[1], Q);
+    } else {
+        const float4 a0 = F.pq[2 * i], a1 = F.pq[2 * i + 1], b0 = F.vq[2 * i], b1 = F.vq[2 * i + 1];
+        const float4 p0 = F.pq[2 * j], p1 = F.pq[2 * j + 1], v0 = F.vq[2 * j], v1 = F.vq[2 * j + 1];
+        return tau_decide_fp32((p0.x - a0.x) + (p1.x - a1.x), (p0.y - a0.y) + (p1.y - a1.y),
+                               (p0.z - a0.z) + (p1.z - a1.z), (v0.x - b0.x) + (v1.x - b1.x),
+                               (v0.y - b0.y) + (v1.y - b1.y), (v0.z - b0.z) + (v1.z - b1.z), a0.w + p0.w,
+                               c11 * F.maxes[0], c11 * F.maxes[1], Q);
+    }
+}
+
 // Settles the warp's queued pairs sm.q[w][0..cnt), one per lane: the
 // certified FP32 decision on the float-float differences, the exact FP64
-// predicate when it is undecided, then the local union and the edge record
-// (one counter update per batch).  Out of line: the pair loop keeps only the
-// high parts and its queue in registers.
-template <int T, int S>
-__device__ __noinline__ uint2 tau_settle_batch(MixedTauSmem<T, S> &sm, int w, int cnt, int ibase, int j0, int joff,
+// predicate when it is undecided, then the local union; edges join the warp's
+// list of edges to record (ne of them so far).  Out of line: the pair loop
+// keeps only the high parts and its masks in registers.
+template <int T, int S, int R, bool RAW>
+__device__ __noinline__ uint2 tau_settle_batch(MixedTauSmem<T, S, R> &sm, int w, int cnt, int ne, int ibase, int j0,
+                                              int joff,
                                               const Level &L, const FFView &F, const TauParams &P,
                                               const MixedTauParams &Q, DevCounters *ctr, int32_t *near_ij,
                                               double *near_tau, long long near_cap, const EdgeList &E)
 {
-    // returns (edges, FP64 evaluations) of this lane's pair
+    // returns (lanes whose pair is an edge, FP64 evaluations of this lane's pair)
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
     const bool has = lane < cnt;
@@ -226,13 +357,7 @@ __device__ __noinline__ uint2 tau_settle_batch(MixedTauSmem<T, S> &sm, int w, in
     double tau = CUDART_NAN;
     if (has) {
         const int gi = ibase + ii, gj = j0 + kk;
-        const float4 a0 = F.pq[2 * gi], a1 = F.pq[2 * gi + 1], b0 = F.vq[2 * gi], b1 = F.vq[2 * gi + 1];
-        const float cX = 11.f * U32 * U32 * F.maxes[0], cV = 11.f * U32 * U32 * F.maxes[1];
-        const float4 jp0 = sm.pq[2 * kk], jp1 = sm.pq[2 * kk + 1], jv0 = sm.vq[2 * kk], jv1 = sm.vq[2 * kk + 1];
-        dec = tau_decide_fp32((jp0.x - a0.x) + (jp1.x - a1.x), (jp0.y - a0.y) + (jp1.y - a1.y),
-                              (jp0.z - a0.z) + (jp1.z - a1.z), (jv0.x - b0.x) + (jv1.x - b1.x),
-                              (jv0.y - b0.y) + (jv1.y - b1.y), (jv0.z - b0.z) + (jv1.z - b1.z), a0.w + jp0.w, cX, cV,
-                              Q);
+        dec = tau_decide_pair<RAW>(L, F, Q, gi, gj);
         if (dec < 0) {
             // undecided: the exact FP64 predicate
             tau = tau_fp64(__dsub_rn(L.x[gi], L.x[gj]), __dsub_rn(L.y[gi], L.y[gj]), __dsub_rn(L.z[gi], L.z[gj]),
@@ -255,193 +380,290 @@ __device__ __noinline__ uint2 tau_settle_batch(MixedTauSmem<T, S> &sm, int w, in
     const unsigned eb = __ballot_sync(0xffffffffu, edge);
     if (eb == 0u) return make_uint2(0u, nfp64);
     if (edge && !luf_union(sm.lp, ii, joff + kk)) raise_err(ctr, DERR_UF_RETRY);
-    if (E.rec) {
-        // every edge is recorded (the decision at h/2 is left to the first
-        // half's pass); tau = the FP64 value or NaN
-        unsigned long long base = 0;
-        if (lane == 0) base = atomicAdd(E.count, (unsigned long long)__popc(eb));
-        base = __shfl_sync(0xffffffffu, base, 0);
-        const unsigned long long q = base + (unsigned)__popc(eb & lt);
-        if (edge && (long long)q < E.cap) {
-            EdgeRec r;
-            r.a = ibase + ii;
-            r.b = j0 + kk;
-            r.e = -1;
-            r.pad = 0;
-            r.tau = tau;
-            E.rec[q] = r;
-        }
+    if (edge && E.rec) {
+        const int q = ne + __popc(eb & lt);
+        sm.ent[w][q] = ent;
+        sm.tau[w][q] = tau;
     }
-    return make_uint2(edge ? 1u : 0u, nfp64);
+    return make_uint2(eb, nfp64);
 }
 
-// Block = T x S threads: thread (row r, slice s) takes pairs (r, k) of the
-// tile with k in the slice's T/S columns (S > 1 shortens each warp's chain
-// for sets with few tiles).  Parameters are grid constants: the out-of-line
-// settle takes them by reference without a copy.
-template <int T, int S>
-__global__ void __launch_bounds__(T * S, 1024 / (T * S))
+// Records the warp's ne listed edges (the decision at h/2 is left to the first
+// half's pass; tau = the FP64 value or NaN).  One counter update for up to
+// 128 of them: its round trip to L2 is longer than settling a batch, and in a
+// spatial order the tiles on the diagonal hold thousands of edges each.
+template <int T, int S, int R>
+__device__ __noinline__ void tau_record(MixedTauSmem<T, S, R> &sm, int w, int ne, int ibase, int j0, const EdgeList &E)
+{
+    const int lane = threadIdx.x & 31;
+    unsigned long long base = 0;
+    if (lane == 0) base = atomicAdd(E.count, (unsigned long long)ne);
+    base = __shfl_sync(0xffffffffu, base, 0);
+    for (int k = lane; k < ne; k += 32) {
+        const unsigned long long q = base + (unsigned)k;
+        if ((long long)q >= E.cap) break;
+        const unsigned ent = sm.ent[w][k];
+        EdgeRec r;
+        r.a = ibase + (int)(ent >> 8);
+        r.b = j0 + (int)(ent & 255u);
+        r.e = -1;
+        r.pad = 0;
+        r.tau = sm.tau[w][k];
+        E.rec[q] = r;
+    }
+}
+
+// Parameters are grid constants: the out-of-line settle takes them by
+// reference without a copy.
+template <int T, int S, int R, bool RAW>
+__global__ void __launch_bounds__(T *S / R, 768 * R / (T * S))
     k_tau_mixed(const __grid_constant__ Level L, const __grid_constant__ FFView F,
                 const __grid_constant__ TauParams P, const __grid_constant__ MixedTauParams Q, DevCounters *ctr,
                 int32_t *near_ij, double *near_tau, long long near_cap, const __grid_constant__ EdgeList E)
 {
-    static_assert(T % 32 == 0 && T % S == 0, "tile shape");
-    __shared__ MixedTauSmem<T, S> sm;
-    const int tid = threadIdx.x, row = tid % T, slice = tid / T;
-    int lo = 0, hi = L.nsets;
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (L.tile_off[mid] <= (int)blockIdx.x) lo = mid; else hi = mid;
-    }
-    const int s = lo;
-    int t = blockIdx.x - L.tile_off[s];
-    const int n = L.set_n[s], start = L.set_start[s];
-    const int nt = (n + T - 1) / T;
-    const int ti = tri_tile_row(t, nt);
-    const int tj = ti + t;
-    const bool diag = ti == tj;
-    const int j0 = start + tj * T;
-    const int jn = min(T, n - tj * T);
-    if (tid == 0) {
-        mbar_init(&sm.bar, 1);
-        fence_mbar_init();
-    }
-    for (int e = tid; e < 2 * T; e += T * S) sm.lp[e] = e;
-    __syncthreads();
-    // fault_test = 1: the copy is announced but never issued, so the wait
-    // below runs out (a test of the bounded wait; no copy is in flight)
-    const bool no_copy = P.fault_test == 1;
-    const long long wait_cycles = no_copy ? FAULT_TEST_WAIT_CYCLES : TMA_WAIT_CYCLES;
-    if (tid == 0) {
-        const unsigned bytes = (unsigned)jn * 32u;
-        mbar_expect_tx(&sm.bar, 2u * bytes);
-        if (!no_copy) {
-            tma_load_1d(sm.pq, F.pq + 2 * (size_t)j0, bytes, &sm.bar);
-            tma_load_1d(sm.vq, F.vq + 2 * (size_t)j0, bytes, &sm.bar);
+    constexpr int THREADS = T * S / R, NW = THREADS / 32, RW = T / (32 * R);
+    constexpr int TC = T / S, GW = TC / TAU_JG;  // a warp's columns and column groups
+    static_assert(T % (32 * R) == 0 && TC % 32 == 0 && T <= 256, "tile shape");
+    __shared__ MixedTauSmem<T, S, R> sm;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, slice = w / RW;
+    const int row0 = (w % RW) * 32 * R + lane;  // the lane's rows: row0 + 32 r
+    int s = 0, t = blockIdx.x, n, start;
+    if constexpr (RAW) {
+        n = L.total;
+        start = 0;
+    } else {
+        int lo = 0, hi = L.nsets;
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (L.tile_off[mid] <= (int)blockIdx.x) lo = mid; else hi = mid;
         }
+        s = lo;
+        t -= L.tile_off[s];
+        n = L.set_n[s];
+        start = L.set_start[s];
     }
-    const int il = ti * T + row;
-    const bool iv = il < n;
-    const int i = start + il;
-    float4 ip0 = make_float4(0, 0, 0, 0), iv0 = ip0;
-    if (iv) {
-        ip0 = F.pq[2 * i];
-        iv0 = F.vq[2 * i];
-    }
-    const bool got = mbar_wait(&sm.bar, 0, wait_cycles);
-    if (__syncthreads_or(!got)) {
-        raise_err(ctr, DERR_TMA_TIMEOUT);
-        // let a copy still in flight land before the CTA exits
-        mbar_wait(&sm.bar, 0, wait_cycles);
-        return;
+    // tile t of the set: by diagonals, the main one first.  In a spatial order
+    // the edges lie near it, and a tile full of edges takes many times an
+    // empty one's time: started last it would be the launch's tail.
+    const int nt = (n + T - 1) / T;
+    const int dt = tri_tile_row(t, nt);
+    const int ti = t, tj = t + dt;
+    const bool diag = dt == 0;
+    const int ibase = start + ti * T, j0 = start + tj * T;
+    const int ni = min(T, n - ti * T), jn = min(T, n - tj * T);
+    for (int e = tid; e < 2 * T; e += THREADS) sm.lp[e] = e;
+    if constexpr (RAW) {
+        for (int p = tid; 2 * p < jn; p += THREADS) {
+            float a[6], b[6], g;
+            tau_load_hi<true>(L, F, Q, j0 + 2 * p, a, g);
+            tau_load_hi<true>(L, F, Q, j0 + min(2 * p + 1, jn - 1), b, g);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) sm.hp[3 * p + c] = make_float4(a[2 * c], b[2 * c], a[2 * c + 1], b[2 * c + 1]);
+        }
+        __syncthreads();
+    } else {
+        if (tid == 0) {
+            mbar_init(&sm.bar, 1);
+            fence_mbar_init();
+        }
+        __syncthreads();
+        // fault_test = 1: the copy is announced but never issued, so the wait
+        // below runs out (a test of the bounded wait; no copy is in flight)
+        const bool no_copy = P.fault_test == 1;
+        const long long wait_cycles = no_copy ? FAULT_TEST_WAIT_CYCLES : TMA_WAIT_CYCLES;
+        if (tid == 0) {
+            // (an odd last body brings its neighbour's slot along: masked below)
+            const unsigned bytes = (unsigned)((jn + 1) / 2) * 48u;
+            mbar_expect_tx(&sm.bar, bytes);
+            if (!no_copy) tma_load_1d(sm.hp, F.hp + 3 * (size_t)(j0 / 2), bytes, &sm.bar);
+        }
+        const bool got = mbar_wait(&sm.bar, 0, wait_cycles);
+        if (__syncthreads_or(!got)) {
+            raise_err(ctr, DERR_TMA_TIMEOUT);
+            // let a copy still in flight land before the CTA exits
+            mbar_wait(&sm.bar, 0, wait_cycles);
+            return;
+        }
     }
     unsigned long long my_edges = 0, my_fp64 = 0;
     const int joff = diag ? 0 : T;  // local index base of the j-tile
-    const int lane = tid & 31, w = tid >> 5;
     const unsigned lt = (1u << lane) - 1u;
-    // column groups per tile, per warp; groups whose boxes a warp computes
-    constexpr int NG = T / TAU_JG, GW = T / S / TAU_JG, GPW = 32 / TAU_JG;
-    // Group certificates: the warp's 32 rows against each TAU_JG-column group
-    // of its columns (tau_groups_apart).  A certified group costs each pair
-    // one velocity difference and a comparison.
-    if (w * GPW < NG) {
-        const int k = TAU_JG * (w * GPW) + lane;  // lane segment s: group w GPW + s
+    // ---- boxes: the column groups' (32 columns a round and warp), the rows'
+    for (int c0 = 32 * w; c0 < T; c0 += 32 * NW) {
+        const int k = c0 + lane;
         GroupBox B;
-        const bool any =
-            warp_group_box<TAU_JG>(k < jn, k < jn ? sm.pq[2 * k] : ip0, k < jn ? sm.vq[2 * k] : iv0, B);
+        box_empty(B);
+        bool wild = false;
+        if (k < jn) {
+            const float *h = reinterpret_cast<const float *>(sm.hp) + (k >> 1) * 12 + (k & 1);
+            const float st[6] = {h[0], h[2], h[4], h[6], h[8], h[10]};
+            float gm;
+            if constexpr (RAW) gm = Q.G * fl32(L.m[j0 + k]);
+            else gm = F.pq[2 * (size_t)(j0 + k)].w;
+            wild = box_add(B, st, gm);
+        }
+        warp_group_box<TAU_JG>(B);
+        const unsigned wb = __ballot_sync(0xffffffffu, wild) >> (lane & ~(TAU_JG - 1));
         if ((lane & (TAU_JG - 1)) == 0) {
-            if (!any) B.gm = -1.f;  // empty group: no pairs
-            sm.jb[w * GPW + lane / TAU_JG] = B;
+            if (k >= jn) B.gm = -1.f;                          // no bodies
+            if (wb & ((1u << TAU_JG) - 1u)) B.gm = CUDART_INF_F;  // a body outside the bounds' range
+            sm.jb[k / TAU_JG] = B;
         }
     }
-    {
-        GroupBox A;
-        const bool any = warp_group_box<32>(iv, ip0, iv0, A);
-        __syncthreads();
-        if (lane < GW) {
-            const GroupBox &B = sm.jb[slice * GW + lane];
-            float thr = -1.f;
-            if (any && B.gm >= 0.f && !diag && !tau_groups_apart(A, B, Q, thr)) thr = -1.f;
-            sm.gthr[w][lane] = thr;
+    uint64_t nx[R][6];  // minus the row's high parts, twice each
+    GroupBox A;
+    box_empty(A);
+    bool awild = false;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int row = row0 + 32 * r;
+        float st[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, gm;
+        if (row < ni) {
+            tau_load_hi<RAW>(L, F, Q, ibase + row, st, gm);
+            awild = box_add(A, st, gm) || awild;
         }
-        __syncwarp();
+#pragma unroll
+        for (int c = 0; c < 6; ++c) nx[r][c] = pack2(-st[c], -st[c]);
     }
-    // the pre-test's error terms for high-part differences: per component
-    // |x_j| <= |x_i| + r, so |dx~ - dx| <= u r + 3.5 u (2 max|x_i| + r): c_x =
-    // 7 u max|x_i| per thread, and the remaining 3.5 u r goes to the
-    // threshold (likewise for the velocities)
-    const float cXh = 7.1f * U32 * fmaxf(fabsf(ip0.x), fmaxf(fabsf(ip0.y), fabsf(ip0.z)));
-    const float cVh = 7.1f * U32 * fmaxf(fabsf(iv0.x), fmaxf(fabsf(iv0.y), fabsf(iv0.z)));
-    // Pairs the certificates leave open are queued per warp and settled 32
-    // at a time, one per lane: taken as they come, a single such pair would
-    // run the certified decision (and possibly FP64) with one lane of 32
-    // active.  Entry = (row in the i-tile << 8) | column in the j-tile.
+    warp_group_box<32>(A);
+    awild = __any_sync(0xffffffffu, awild);
+    __syncthreads();
+    // ---- certificates of the warp's rows against each of its column groups
+    if (lane < GW) {
+        const GroupBox &B = sm.jb[slice * GW + lane];
+        float4 g = make_float4(0.f, 0.f, __int_as_float(TAU_OPEN), A.gm + B.gm);
+        if (!awild && A.gm > 0.f && B.gm > 0.f && B.gm < 1e30f) {
+            float thr;
+            PairBounds b;
+            if (!diag && tau_groups_apart(A, B, Q, thr)) {
+                g.y = -thr;
+                g.z = __int_as_float(TAU_SPEED);
+            } else if (tau_pair_bounds(A.amax, A.vabs, A.gm + B.gm, Q, b)) {
+                g.x = b.p0;
+                g.y = b.w0;
+                g.z = __int_as_float(TAU_BOUNDS);
+            }
+        }
+        sm.gq[w][lane] = g;
+    }
+    __syncwarp();
+    const uint64_t nc2 = pack2(-Q.pb_c2, -Q.pb_c2);
+    int qn = 0, ne = 0;  // pairs queued, edges listed by this warp (warp-uniform)
     auto settle = [&](int cnt) {
-        const uint2 c = tau_settle_batch<T, S>(sm, w, cnt, start + ti * T, j0, joff, L, F, P, Q, ctr, near_ij,
-                                               near_tau, near_cap, E);
-        my_edges += c.x;
+        const uint2 c = tau_settle_batch<T, S, R, RAW>(sm, w, cnt, ne, ibase, j0, joff, L, F, P, Q, ctr, near_ij,
+                                                       near_tau, near_cap, E);
+        const int k = __popc(c.x);
+        my_edges += lane == 0 ? k : 0;
         my_fp64 += c.y;
+        if (!E.rec) return;
+        ne += k;
+        __syncwarp();
+        if (ne > 96) {
+            tau_record<T, S, R>(sm, w, ne, ibase, j0, E);
+            __syncwarp();
+            ne = 0;
+        }
     };
-    int qn = 0;  // entries queued by this warp (warp-uniform)
-    // the warp's columns [kb, k1): one trip count for all its lanes, so each
-    // column ends in a vote (the common case: no lane's pair left open)
-    const int kb = slice * (T / S), k1 = min(jn, kb + T / S);
-    // the full high-part certificate of pair (row, k)
-    auto quick = [&](int k) {
-        const float4 jp0 = sm.pq[2 * k], jv0 = sm.vq[2 * k];
-        return tau_quick_apart(jp0.x - ip0.x, jp0.y - ip0.y, jp0.z - ip0.z, jv0.x - iv0.x, jv0.y - iv0.y,
-                               jv0.z - iv0.z, ip0.w + jp0.w, cXh, cVh, Q);
-    };
-    // Pass 1, the hot loop: certificates only.  A column with open pairs
-    // (rare) leaves its lane word in sm.om and its bit in sm.cm.
-    if (lane < T / S / 32) sm.cm[w][lane] = 0u;
-    __syncwarp();
+    const int kb = slice * TC, k1 = min(jn, kb + TC);
 #pragma unroll 1
-    for (int g = 0; g < GW; ++g) {
-        const int ka = kb + TAU_JG * g, kz = min(k1, ka + TAU_JG);
-        const float thr = sm.gthr[w][g];
-        if (thr >= 0.f) {
-            // certified group: one velocity difference per pair; a pair
-            // below the lower speed root takes the full certificate
-            for (int k = ka; k < kz; ++k) {
-                const bool mine = iv && (!diag || k > row);
-                const float4 jv0 = sm.vq[2 * k];
-                const float a = jv0.x - iv0.x, b = jv0.y - iv0.y, c = jv0.z - iv0.z;
-                const bool slow = mine && fmaf(c, c, fmaf(b, b, a * a)) < thr;
-                if (__ballot_sync(0xffffffffu, slow) == 0u) continue;
-                const unsigned open = __ballot_sync(0xffffffffu, slow && !quick(k));
-                if (open && lane == 0) {
-                    sm.om[w][k - kb] = open;
-                    sm.cm[w][(k - kb) >> 5] |= 1u << ((k - kb) & 31);
+    for (int cb = kb; cb < k1; cb += 32) {
+        // columns cb..cb+31: bit 31 - c of m[r] = pair (row r, column cb + c) is open
+        uint32_t m[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) m[r] = 0u;
+        const int ng = min(4, (k1 - cb + TAU_JG - 1) / TAU_JG);
+#pragma unroll 1
+        for (int g = 0; g < ng; ++g) {
+            const float4 gc = sm.gq[w][(cb - kb) / TAU_JG + g];
+            const int kind = __float_as_int(gc.z);
+            const ulonglong2 *J = reinterpret_cast<const ulonglong2 *>(sm.hp) + 3 * ((cb + TAU_JG * g) >> 1);
+            if (kind == TAU_BOUNDS) {
+                const uint64_t p0 = pack2(gc.x, gc.x), w0 = pack2(gc.y, gc.y);
+#pragma unroll
+                for (int u = 0; u < TAU_JG / 2; ++u) {
+                    const ulonglong2 a = J[3 * u], b = J[3 * u + 1], c = J[3 * u + 2];
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        const uint64_t dx = add2(a.x, nx[r][0]), dy = add2(a.y, nx[r][1]), dz = add2(b.x, nx[r][2]);
+                        const uint64_t du = add2(b.y, nx[r][3]), dv = add2(c.x, nx[r][4]), dw = add2(c.y, nx[r][5]);
+                        const uint64_t pp = fma2(dz, dz, fma2(dy, dy, fma2(dx, dx, p0)));
+                        const uint64_t ww = fma2(dw, dw, fma2(dv, dv, fma2(du, du, w0)));
+                        const uint64_t oo = fma2(ww, nc2, pp) | ww;  // sign bits: open
+                        m[r] = __funnelshift_l((uint32_t)oo, m[r], 1);
+                        m[r] = __funnelshift_l((uint32_t)(oo >> 32), m[r], 1);
+                    }
                 }
+            } else if (kind == TAU_SPEED) {
+                const uint64_t w0 = pack2(gc.y, gc.y);
+#pragma unroll
+                for (int u = 0; u < TAU_JG / 2; ++u) {
+                    const uint64_t b = J[3 * u + 1].y;
+                    const ulonglong2 c = J[3 * u + 2];
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        const uint64_t du = add2(b, nx[r][3]), dv = add2(c.x, nx[r][4]), dw = add2(c.y, nx[r][5]);
+                        const uint64_t ww = fma2(dw, dw, fma2(dv, dv, fma2(du, du, w0)));
+                        m[r] = __funnelshift_l((uint32_t)ww, m[r], 1);
+                        m[r] = __funnelshift_l((uint32_t)(ww >> 32), m[r], 1);
+                    }
+                }
+            } else {
+#pragma unroll
+                for (int r = 0; r < R; ++r) m[r] = (m[r] << TAU_JG) | ((1u << TAU_JG) - 1u);
             }
-        } else {
-            for (int k = ka; k < kz; ++k) {
-                const unsigned open = __ballot_sync(0xffffffffu, iv && (!diag || k > row) && !quick(k));
-                if (open && lane == 0) {
-                    sm.om[w][k - kb] = open;
-                    sm.cm[w][(k - kb) >> 5] |= 1u << ((k - kb) & 31);
+        }
+        // the columns that exist, and (diagonal tiles) lie right of the row
+        int open = 0;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int row = row0 + 32 * r, c0 = diag ? max(0, row + 1 - cb) : 0, c1 = min(32, k1 - cb);
+            m[r] <<= 32 - TAU_JG * ng;
+            m[r] &= row < ni && c0 < c1 ? (0xffffffffu >> c0) & (0xffffffffu << (32 - c1)) : 0u;
+            open += __popc(m[r]);
+        }
+        if (!__any_sync(0xffffffffu, open != 0)) continue;
+        if (__reduce_add_sync(0xffffffffu, (unsigned)open) > 32u * 32u * R / 2u) {
+            // slow bodies everywhere (a cold system: v < v_thr at separations
+            // far above r_min): the full certificate column by column is
+            // cheaper than settling them all
+            for (int c = 0; c < min(32, k1 - cb); ++c) {
+                const int k = cb + c;
+                const float *h = reinterpret_cast<const float *>(sm.hp) + (k >> 1) * 12 + (k & 1);
+                const float mu = sm.gq[w][(k - kb) / TAU_JG].w;
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    float d[6], x[6], e;
+#pragma unroll
+                    for (int q = 0; q < 6; ++q) {
+                        unpack2(nx[r][q], x[q], e);
+                        d[q] = h[2 * q] + x[q];
+                    }
+                    const float cX = 7.1f * U32 * fmaxf(fabsf(x[0]), fmaxf(fabsf(x[1]), fabsf(x[2])));
+                    const float cV = 7.1f * U32 * fmaxf(fabsf(x[3]), fmaxf(fabsf(x[4]), fabsf(x[5])));
+                    if (tau_quick_apart(d[0], d[1], d[2], d[3], d[4], d[5], mu, cX, cV, Q)) m[r] &= ~(0x80000000u >> c);
                 }
             }
         }
-    }
-    __syncwarp();
-    // Pass 2: the open pairs, queued and settled 32 at a time
-    for (int c = 0; c < T / S / 32; ++c) {
-        unsigned cols = sm.cm[w][c];
-        while (cols) {
-            const int k = kb + 32 * c + __ffs(cols) - 1;
-            cols &= cols - 1u;
-            const unsigned open = sm.om[w][k - kb];
-            if ((open >> lane) & 1u) sm.q[w][qn + __popc(open & lt)] = ((unsigned)row << 8) | (unsigned)k;
-            qn += __popc(open);
-            if (qn >= 32) {
-                __syncwarp();
-                settle(32);
-                __syncwarp();
-                if (lane < qn - 32) sm.q[w][lane] = sm.q[w][32 + lane];
-                __syncwarp();
-                qn -= 32;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            for (;;) {
+                const unsigned b = __ballot_sync(0xffffffffu, m[r] != 0u);
+                if (b == 0u) break;
+                if (m[r] != 0u) {
+                    const int c = __clz(m[r]);
+                    m[r] &= ~(0x80000000u >> c);
+                    sm.q[w][qn + __popc(b & lt)] = ((unsigned)(row0 + 32 * r) << 8) | (unsigned)(cb + c);
+                }
+                qn += __popc(b);
+                if (qn >= 32) {
+                    __syncwarp();
+                    settle(32);
+                    __syncwarp();
+                    const uint32_t keep = lane < qn - 32 ? sm.q[w][32 + lane] : 0u;
+                    __syncwarp();
+                    if (lane < qn - 32) sm.q[w][lane] = keep;
+                    qn -= 32;
+                }
             }
         }
     }
@@ -449,14 +671,15 @@ __global__ void __launch_bounds__(T * S, 1024 / (T * S))
         __syncwarp();
         settle(qn);
     }
+    if (ne > 0) tau_record<T, S, R>(sm, w, ne, ibase, j0, E);
     __syncthreads();
     // merge the tile's local components into the global forest: one union
     // per local non-root element instead of one per edge
-    for (int e = tid; e < (diag ? T : 2 * T); e += T * S) {
+    for (int e = tid; e < (diag ? T : 2 * T); e += THREADS) {
         const int r = luf_find(sm.lp, e);
         if (r != e) {
-            const int ge = (e < T) ? start + ti * T + e : j0 + (e - T);
-            const int gr = (r < T) ? start + ti * T + r : j0 + (r - T);
+            const int ge = (e < T) ? ibase + e : j0 + (e - T);
+            const int gr = (r < T) ? ibase + r : j0 + (r - T);
             // (fault_test = 2: every hook gives up at once, a test of the retry cap)
             if (!uf_union(L.parent, ge, gr, P.fault_test == 2 ? 0 : UF_RETRY_MAX)) raise_err(ctr, DERR_UF_RETRY);
         }
@@ -477,20 +700,16 @@ void launch_tau_mixed(const Level &L, const FFView &F, int ntiles, const TauPara
                       cudaStream_t s)
 {
     if (ntiles <= 0) return;
-    MixedTauParams Q;
-    Q.eta = (float)P.eta_in;
-    Q.etah = (float)(P.eta_outside ? P.eta_in * P.eta / P.h : P.eta_in / P.h);
-    Q.eps2 = (float)P.eps2;
-    Q.G = (float)P.G;
-    Q.hq = (float)(P.eta_outside ? P.h / P.eta : P.h);  // h/eta_in in the units of T: eta_in/etah
-    static_assert(TAU_VAR_T[0] == 64 && TAU_VAR_T[1] == 128 && TAU_VAR_T[2] == 64 && TAU_VAR_S[2] == 2,
+    const MixedTauParams Q = mixed_tau_params(P);
+    static_assert(TAU_VAR_T[0] == 128 && TAU_VAR_S[0] == 2 && TAU_VAR_T[1] == 256 && TAU_VAR_T[2] == 64 &&
+                      TAU_VAR_S[2] == 2,
                   "tau variants");
     if (variant == 0)
-        k_tau_mixed<64, 1><<<ntiles, 64, 0, s>>>(L, F, P, Q, ctr, near_ij, near_tau, near_cap, E);
+        k_tau_mixed<128, 2, 2, false><<<ntiles, 128, 0, s>>>(L, F, P, Q, ctr, near_ij, near_tau, near_cap, E);
     else if (variant == 1)
-        k_tau_mixed<128, 1><<<ntiles, 128, 0, s>>>(L, F, P, Q, ctr, near_ij, near_tau, near_cap, E);
+        k_tau_mixed<256, 1, 2, false><<<ntiles, 128, 0, s>>>(L, F, P, Q, ctr, near_ij, near_tau, near_cap, E);
     else
-        k_tau_mixed<64, 2><<<ntiles, 128, 0, s>>>(L, F, P, Q, ctr, near_ij, near_tau, near_cap, E);
+        k_tau_mixed<64, 2, 1, false><<<ntiles, 128, 0, s>>>(L, F, P, Q, ctr, near_ij, near_tau, near_cap, E);
     CC_COUNT_LAUNCH(1);
 }
 

@@ -276,12 +276,9 @@ void launch_edges_reuse(const EdgeList &parent, long long pcount, const Level &P
 {
     if (pcount <= 0) return;
     const double hp = 2.0 * P.h;
-    MixedTauParams Q;
-    Q.eta = (float)P.eta_in;
-    Q.etah = (float)(P.eta_outside ? P.eta_in * P.eta / hp : P.eta_in / hp);
-    Q.eps2 = (float)P.eps2;
-    Q.G = (float)P.G;
-    Q.hq = 0.f;  // (the pre-test is not used here)
+    TauParams PP = P;
+    PP.h = hp;
+    const MixedTauParams Q = mixed_tau_params(PP);
     const unsigned blocks = (unsigned)((pcount + 255) / 256);
     k_edges_filter<<<blocks, 256, 0, s>>>(parent, pcount, PL, PF, Q, mixed ? 1 : 0, inv, C, child, P, ctr, near_ij,
                                           near_tau, near_cap);
@@ -363,7 +360,7 @@ __global__ void __launch_bounds__(TAU_T) k_tau_edges(Level L, TauParams P, DevCo
     }
 }
 
-void launch_tau_hook(const Level &L, int ntiles, const TauParams &P, int variant, DevCounters *ctr,
+void launch_tau_hook(const Level &L, int ntiles, const TauParams &P, DevCounters *ctr,
                      int32_t *edges, long long edge_cap, int32_t *near_ij, double *near_tau, long long near_cap,
                      cudaStream_t s, const EdgeList *rec)
 {
@@ -374,10 +371,7 @@ void launch_tau_hook(const Level &L, int ntiles, const TauParams &P, int variant
         CC_COUNT_LAUNCH(1);
         return;
     }
-    if (variant == 0)
-        k_tau_hook<64><<<ntiles, 64, 0, s>>>(L, P, ctr, near_ij, near_tau, near_cap, E);
-    else
-        k_tau_hook<128><<<ntiles, 128, 0, s>>>(L, P, ctr, near_ij, near_tau, near_cap, E);
+    k_tau_hook<TAU_T><<<ntiles, TAU_T, 0, s>>>(L, P, ctr, near_ij, near_tau, near_cap, E);
     CC_COUNT_LAUNCH(1);
 }
 
