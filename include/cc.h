@@ -175,7 +175,9 @@ int cc_set_stream(cc_ctx *ctx, void *stream);
 /* Time-step graph of Sec. 2.2 on `set` at threshold h: all pairs of the set,
  * tau(i,j) by Eq. (tauij) in FP64 (T_ff = eta sqrt(r^3/mu), T_fb = eta r/|dv|,
  * their time derivatives along the pair's motion, dT/dt clamped at 1), edge iff
- * tau(i,j) < h.  *n_edges = edge count.  edges_out (may be NULL) receives
+ * tau(i,j) < h, decided in FP32 where a rigorous bound settles it and by the
+ * FP64 tau elsewhere (the same edges; near_tol above 1e-6: every tau in
+ * FP64).  *n_edges = edge count.  edges_out (may be NULL) receives
  * min(cap, n_edges) pairs (i<j as particle ids, int32[cap][2]) in
  * lexicographic order.  *n_near = pairs with |tau-h| < near_tol*h (their
  * (i, j, tau) are readable with cc_near_pairs).  Returns CC_E_CAPACITY when
@@ -246,7 +248,8 @@ int cc_timing(cc_ctx *ctx, cc_timing_t *out);
 /* One cell of the launch-shape autotuner: a kernel and a size bin (the
  * launch's pair count in [2^bin, 2^(bin+1))).  Variant v of the kernel is
  * the launch shape (shape[v], slices[v]): for the tau kernels the tile edge
- * (64, 128, 256) and the threads per tile row (its columns split in slices); for
+ * (64, 128) and the threads per tile row (its columns split in slices; the
+ * largest levels run 256-wide tiles by a fixed rule and have no cell); for
  * the FP64 kick the tile edge (32, 64, 128), slices 1; for the mixed kick
  * the j-chunk in tiles of 128 and the column slices of each tile. */
 typedef struct {

@@ -31,7 +31,10 @@ using namespace cc;
 
 namespace {
 
-constexpr int TAU_TILE = 128;   // must match the tau kernel
+// cc_timestep_graph: pairs within this relative distance of the threshold are
+// never decided by the certified FP32 kernel (its error terms and slack leave
+// at least 1.5e-6 open), so it logs every near pair up to this near_tol
+constexpr double GRAPH_NEAR_MAX = 1e-6;
 
 thread_local std::string g_init_err;
 
@@ -119,7 +122,7 @@ struct LevelAlloc {
 // choice except through the rounding order of the mixed kick's j-chunks.
 enum TuneKind { TK_TAU64 = 0, TK_TAUMIX = 1, TK_K64 = 2, TK_MK = 3, TK_N = 4 };
 constexpr int TUNE_BINS = 40, TUNE_MAXV = 3, TUNE_BIG_BIN = 24;
-constexpr int TUNE_NVAR[TK_N] = {N_TAU64_VAR, N_TAU_VAR, N_K64_VAR, N_MK_VAR};
+constexpr int TUNE_NVAR[TK_N] = {N_TAU64_VAR, N_TAU_TUNED, N_K64_VAR, N_MK_VAR};
 
 struct TuneCell {
     double qmin[TUNE_MAXV] = {0, 0, 0};  // fastest trial: ms per unit of work
@@ -378,7 +381,7 @@ static int align_up(int v, int a) { return (v + a - 1) / a * a; }
 // while the plain variant leaves the GPU short of blocks.
 static bool tune_eligible(const cc_ctx *c, int tkind, const long long *blocks, int v)
 {
-    if (tkind == TK_TAUMIX && v == TAU_VAR_SMALL) return blocks[0] < 16ll * c->nsm;
+    if (tkind == TK_TAUMIX && TAU_VAR_S[v] > 1) return blocks[0] < 16ll * c->nsm;
     if (tkind == TK_MK && MK_VAR_SLICE[v] > 1) return blocks[0] < 8ll * c->nsm;
     return true;
 }
@@ -427,6 +430,22 @@ static int tune_pick(cc_ctx *c, int tkind, const long long *blocks, long long wo
     t.picked[pick]++;
     *timed = true;
     return pick;
+}
+
+// The certified tau kernel's shape: 256-wide tiles (two rows a lane: half the
+// prologue and shared-memory reads per pair) where every SM gets at least 24
+// of them, the tuner's choice below.  Measured per 1e6 pairs, 256 against the
+// best tuned shape: 2.1e9 pairs 0.38 / 0.40-0.48 us, 8.0e8 0.79 / 0.92, 2.5e8
+// 0.62 / 0.87; the 16384-body level (1.34e8 pairs in 14 tiles per SM, its
+// edges in the tiles on the diagonal) 1.39 / 0.82.
+static int tau_pick(cc_ctx *c, const LevelAlloc &a, int *bin, bool *timed)
+{
+    if (a.tau_blocks[TAU_VAR_WIDE] >= 24ll * c->nsm) {
+        *bin = 0;
+        *timed = false;
+        return TAU_VAR_WIDE;
+    }
+    return tune_pick(c, TK_TAUMIX, a.tau_blocks, a.pairs, bin, timed);
 }
 
 static void free_level(LevelAlloc &a)
@@ -721,7 +740,7 @@ static int split_launch(cc_ctx *c, LevelAlloc &a, double h, const LevelAlloc *pa
         const int tk = TK_TAUMIX;
         int bin;
         bool timed;
-        const int var = tune_pick(c, tk, a.tau_blocks, a.pairs, &bin, &timed);
+        const int var = tau_pick(c, a, &bin, &timed);
         const long long ntiles = a.tau_blocks[var];
         if (ntiles > 0x7fffffff) return fail(c, CC_E_ARG, "set too large for the tile grid");
         Level L = a.L;
@@ -1811,36 +1830,70 @@ int cc_timestep_graph(cc_ctx *c, const int32_t *set, int64_t n_set, double h, in
     if (!c || !(h > 0.0) || !std::isfinite(h) || cap < 0)
         return c ? fail(c, CC_E_ARG, "cc_timestep_graph: bad argument") : CC_E_ARG;
     CC_TRY(stage_set(c, set, n_set, nullptr));
-    // pass 1: count edges (and split, which also fills the union-find)
-    CC_TRY(reset_call_counters(c));
     LevelAlloc &u = c->unit;
     const TauParams P = tau_params(c, h);
-    const long long nt = (n_set + TAU_TILE - 1) / TAU_TILE;
     Level UL = u.L;
-    UL.tile_off = u.tau_off[TAU_VAR_128];  // 128-wide tiles
-    launch_init_parent(u.L, nullptr, c->stream);
-    launch_tau_hook(UL, (int)(nt * (nt + 1) / 2), P, c->d_ctr, nullptr, 0, c->d_near_ij,
-                    c->d_near_tau, c->near_cap, c->stream);
+    UL.tile_off = u.tau_off[TAU_VAR_128];
+    const int nt128 = (int)u.tau_blocks[TAU_VAR_128];
+    // The certified kernel takes the FP64 predicate's decisions, and sees every
+    // near-threshold pair in FP64 while near_tol is inside what its FP32 bounds
+    // leave open; it records the edges as it finds them.  A wider near_tol
+    // needs the FP64 tau of every pair: one pass to count, one to write.
+    const bool certified = c->p.near_tol <= GRAPH_NEAR_MAX;
     DevCounters h1;
-    CC_CUDA(c, cudaMemcpyAsync(&h1, c->d_ctr, sizeof(h1), cudaMemcpyDeviceToHost, c->stream));
-    CC_CUDA(c, cudaStreamSynchronize(c->stream));
+    auto pass = [&](bool rec) -> int {
+        CC_TRY(reset_call_counters(c));
+        if (certified) {
+            int bin;
+            bool timed;
+            const int var = tau_pick(c, u, &bin, &timed);
+            if (u.tau_blocks[var] > 0x7fffffff) return fail(c, CC_E_ARG, "set too large for the tile grid");
+            Level L = u.L;
+            L.tile_off = u.tau_off[var];
+            launch_prep_ff(u.L, u.F, c->p.G, true, c->stream, true, rec ? u.E.count : nullptr);
+            const int ev = ev_begin(c, 0, nullptr, timed ? TK_TAUMIX : -1, bin, var, (double)u.pairs);
+            launch_tau_mixed(L, u.F, (int)u.tau_blocks[var], P, var, c->d_ctr, c->d_near_ij, c->d_near_tau,
+                             c->near_cap, rec ? u.E : EdgeList{nullptr, nullptr, 0}, c->stream);
+            ev_end(c, ev);
+        } else {
+            launch_init_parent(u.L, nullptr, c->stream);
+            launch_tau_hook(UL, nt128, P, c->d_ctr, nullptr, 0, c->d_near_ij, c->d_near_tau, c->near_cap, c->stream);
+        }
+        CC_CUDA(c, cudaMemcpyAsync(&h1, c->d_ctr, sizeof(h1), cudaMemcpyDeviceToHost, c->stream));
+        CC_CUDA(c, cudaStreamSynchronize(c->stream));
+        ev_resolve(c);
+        return CC_OK;
+    };
+    const bool rec = certified && edges_out;
+    if (rec) CC_TRY(ensure_edges(c, u));
+    CC_TRY(pass(rec));
     const long long ne = (long long)h1.edges;
     if (n_edges) *n_edges = ne;
     if (n_near) *n_near = (long long)h1.near_pairs;
     c->st.edges += h1.edges;
     c->st.near_pairs += h1.near_pairs;
+    c->st.tau_fp64 += h1.tau_fp64;
     c->st.tau_pairs += (unsigned long long)n_set * (n_set - 1) / 2;
+    CC_CUDA(c, cudaMemsetAsync(&c->d_ctr->tau_fp64, 0, sizeof(unsigned long long), c->stream));
     CC_TRY(check_device_error(c));
     if (edges_out && ne > 0) {
-        // pass 2: write the edges, then sort them lexicographically
+        if (rec && ne > u.E.cap) {  // more edges than records: once more, with room for all
+            CC_TRY(ensure_edges(c, u, ne));
+            CC_TRY(pass(true));
+            CC_CUDA(c, cudaMemsetAsync(&c->d_ctr->tau_fp64, 0, sizeof(unsigned long long), c->stream));
+        }
+        // the edges as id pairs, sorted lexicographically
         const size_t need = (size_t)ne * 8 + edge_sort_scratch_bytes(ne) + (size_t)n_set * 16 + 1024;
         CC_TRY(ensure_tmp(c, need));
         int32_t *de = (int32_t *)((char *)c->tmp + (size_t)n_set * 16);
         void *ss = (void *)(de + 2 * ne);
-        CC_TRY(reset_call_counters(c));
-        launch_init_parent(u.L, nullptr, c->stream);
-        launch_tau_hook(UL, (int)(nt * (nt + 1) / 2), P, c->d_ctr, de, ne, c->d_near_ij,
-                        c->d_near_tau, c->near_cap, c->stream);
+        if (rec) {
+            launch_ok_rec_pairs(u.E.rec, ne, u.L.gid, de, c->stream);
+        } else {
+            CC_TRY(reset_call_counters(c));
+            launch_init_parent(u.L, nullptr, c->stream);
+            launch_tau_hook(UL, nt128, P, c->d_ctr, de, ne, c->d_near_ij, c->d_near_tau, c->near_cap, c->stream);
+        }
         int bits = 0;
         while (bits < 31 && (1ll << bits) <= c->n) ++bits;
         launch_sort_edges(de, ne, bits, ss, c->stream);

@@ -289,16 +289,16 @@ extern unsigned long long g_launches;
 
 // cc_pair.cu
 void launch_init_parent(const Level &L, unsigned long long *edge_count, cudaStream_t s);
-// tunable launch shapes (variant index): tau tiles {128, 256, 64, the first
-// and last in two column slices}; FP64 kick tiles {32, 64, 128}; mixed kick (j-chunk in
-// tiles of 128, column slices) {(1, 1), (4, 1), (1, 4)}
-constexpr int N_TAU_VAR = 3, N_K64_VAR = 3, N_MK_VAR = 3;
+// launch shapes (variant index): tau tiles {64, 128, 64 in two column slices}
+// tuned, 256 by rule (tau_pick); FP64 kick tiles {32, 64, 128}; mixed kick
+// (j-chunk in tiles of 128, column slices) {(1, 1), (4, 1), (1, 4)}
+constexpr int N_TAU_VAR = 4, N_K64_VAR = 3, N_MK_VAR = 3;
 // tau variants: tile edge T and column slices S per tile row (the FP64
 // kernels run on the 128-wide tiles)
-constexpr int TAU_VAR_T[N_TAU_VAR] = {128, 256, 64};
-constexpr int TAU_VAR_S[N_TAU_VAR] = {2, 1, 2};
-constexpr int TAU_VAR_SMALL = 2;  // the shape for sets with few tiles
-constexpr int N_TAU64_VAR = 2, TAU_VAR_128 = 0;
+constexpr int TAU_VAR_T[N_TAU_VAR] = {64, 128, 64, 256};
+constexpr int TAU_VAR_S[N_TAU_VAR] = {1, 1, 2, 1};
+constexpr int N_TAU_TUNED = 3, TAU_VAR_WIDE = 3;
+constexpr int N_TAU64_VAR = 2, TAU_VAR_128 = 1;
 static_assert(TAU_VAR_T[TAU_VAR_128] == 128, "128-wide tau tiles");
 constexpr int K64_VAR_T[N_K64_VAR] = {32, 64, 128};
 constexpr int MK_VAR_CHUNK[N_MK_VAR] = {1, 4, 1};
@@ -473,6 +473,11 @@ void launch_prep_ff(const Level &L, const FFView &F, double G, bool with_v, cuda
 void launch_tau_mixed(const Level &L, const FFView &F, int ntiles, const TauParams &P, int variant,
                       DevCounters *ctr, int32_t *near_ij, double *near_tau, long long near_cap, const EdgeList &rec,
                       cudaStream_t s);
+// the certified edges of a caller's FP64 arrays (n bodies, one set) hooked
+// into the forest `parent`; counts and errors on ctr, no pair logged
+// (P.near_tol = 0)
+void launch_tau_raw(const double *m, const double *x3, const double *v3, int n, const TauParams &P, int32_t *parent,
+                    DevCounters *ctr, cudaStream_t s);
 int mixed_kick_blocks(int n, int chunk, int slices);
 int mixed_kick_chunks(int n, int chunk);
 // drift_dt > 0: the level's drift of rest-set members (component size 1 by

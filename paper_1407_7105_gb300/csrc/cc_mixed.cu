@@ -137,7 +137,7 @@ void launch_prep_kick(const Level &L, const FFView &F, const int32_t *order, con
 // in no spatial order (8.0e8 pairs) 1790 -> 630 us, before -> after the
 // comparisons took the place of tau_quick_apart.  In a spatial order the
 // launch ends with the tiles on the diagonal, whose pairs are mostly edges:
-// four warps a 128-wide tile (S = 2) instead of two took the 16384-body level
+// four warps a 128-wide tile (R = 1) instead of two took the 16384-body level
 // from 196 to 126 us.
 // RAW: the set is a caller's FP64 arrays (L.x .. L.m, L.total bodies, no
 // float-float copy): columns and rows are rounded as they are loaded.
@@ -701,15 +701,45 @@ void launch_tau_mixed(const Level &L, const FFView &F, int ntiles, const TauPara
 {
     if (ntiles <= 0) return;
     const MixedTauParams Q = mixed_tau_params(P);
-    static_assert(TAU_VAR_T[0] == 128 && TAU_VAR_S[0] == 2 && TAU_VAR_T[1] == 256 && TAU_VAR_T[2] == 64 &&
-                      TAU_VAR_S[2] == 2,
+    static_assert(TAU_VAR_T[0] == 64 && TAU_VAR_T[1] == 128 && TAU_VAR_T[2] == 64 && TAU_VAR_S[2] == 2 &&
+                      TAU_VAR_T[3] == 256,
                   "tau variants");
     if (variant == 0)
-        k_tau_mixed<128, 2, 2, false><<<ntiles, 128, 0, s>>>(L, F, P, Q, ctr, near_ij, near_tau, near_cap, E);
+        k_tau_mixed<64, 1, 1, false><<<ntiles, 64, 0, s>>>(L, F, P, Q, ctr, near_ij, near_tau, near_cap, E);
     else if (variant == 1)
-        k_tau_mixed<256, 1, 2, false><<<ntiles, 128, 0, s>>>(L, F, P, Q, ctr, near_ij, near_tau, near_cap, E);
-    else
+        k_tau_mixed<128, 1, 1, false><<<ntiles, 128, 0, s>>>(L, F, P, Q, ctr, near_ij, near_tau, near_cap, E);
+    else if (variant == 2)
         k_tau_mixed<64, 2, 1, false><<<ntiles, 128, 0, s>>>(L, F, P, Q, ctr, near_ij, near_tau, near_cap, E);
+    else
+        k_tau_mixed<256, 1, 2, false><<<ntiles, 128, 0, s>>>(L, F, P, Q, ctr, near_ij, near_tau, near_cap, E);
+    CC_COUNT_LAUNCH(1);
+}
+
+// the same over a caller's FP64 arrays as one set, hooked into `parent`: 256-wide
+// tiles while they give every SM two blocks, else 64-wide ones
+constexpr int TAU_RAW_WIDE_N = 6144;
+
+void launch_tau_raw(const double *m, const double *x3, const double *v3, int n, const TauParams &P, int32_t *parent,
+                    DevCounters *ctr, cudaStream_t s)
+{
+    Level L{};
+    double *x = const_cast<double *>(x3), *v = const_cast<double *>(v3);
+    const size_t N = (size_t)n;
+    L.x = x; L.y = x + N; L.z = x + 2 * N;
+    L.vx = v; L.vy = v + N; L.vz = v + 2 * N;
+    L.m = const_cast<double *>(m);
+    L.parent = parent;
+    L.total = n;
+    const MixedTauParams Q = mixed_tau_params(P);
+    const FFView F{};
+    const EdgeList E{nullptr, nullptr, 0};
+    if (n >= TAU_RAW_WIDE_N) {
+        const int nt = (n + 255) / 256;
+        k_tau_mixed<256, 1, 2, true><<<nt * (nt + 1) / 2, 128, 0, s>>>(L, F, P, Q, ctr, nullptr, nullptr, 0, E);
+    } else {
+        const int nt = (n + 63) / 64;
+        k_tau_mixed<64, 2, 1, true><<<nt * (nt + 1) / 2, 128, 0, s>>>(L, F, P, Q, ctr, nullptr, nullptr, 0, E);
+    }
     CC_COUNT_LAUNCH(1);
 }
 
