@@ -20,30 +20,34 @@
 
 namespace cc {
 
-// parent[] and component sizes, then one word for the device error and one
-// for the component count
-static __device__ __align__(256) int32_t g_noalloc_scratch[2 * CC_NOALLOC_MAX_N + 64];
+// parent[] and component sizes, then the component count, the finished
+// blocks of the last kernel and the tau kernel's counters
+constexpr int NA_WORDS = 64, NA_CTR_AT = 8;
+static __device__ __align__(256) int32_t g_noalloc_scratch[2 * CC_NOALLOC_MAX_N + NA_WORDS];
+static_assert(NA_CTR_AT * 4 + sizeof(DevCounters) <= NA_WORDS * 4, "counters in the scratch tail");
 
 namespace {
 
-constexpr int NA_T = 128;
 constexpr int NA_MAX_DEVICES = 64;
 std::mutex g_na_mutex;
 int32_t *g_na_ptr[NA_MAX_DEVICES] = {};
 
 struct NaScratch {
     int32_t *parent, *cnt;
-    unsigned *err;
     int32_t *ncomp;
+    unsigned *done;
+    DevCounters *ctr;
 };
 
 NaScratch na_view(int32_t *base)
 {
     NaScratch s;
+    int32_t *tail = base + 2 * CC_NOALLOC_MAX_N;
     s.parent = base;
     s.cnt = base + CC_NOALLOC_MAX_N;
-    s.err = (unsigned *)(base + 2 * CC_NOALLOC_MAX_N);
-    s.ncomp = base + 2 * CC_NOALLOC_MAX_N + 1;
+    s.ncomp = tail;
+    s.done = (unsigned *)(tail + 1);
+    s.ctr = (DevCounters *)(tail + NA_CTR_AT);
     return s;
 }
 
@@ -59,66 +63,36 @@ __global__ void k_na_init(NaScratch S, int n)
         S.cnt[k] = 0;
     }
     if (k == 0) {
-        *S.err = 0u;
         *S.ncomp = 0;
+        *S.done = 0u;
+        S.ctr->edges = 0ull;
+        S.ctr->tau_fp64 = 0ull;
+        S.ctr->err = 0u;
     }
 }
 
-// tau(i,j) < h over all pairs i < j, hooked into the union-find forest
-// (the same FP64 predicate as the context path, tiles loaded with plain
-// coalesced loads because caller arrays need not be 16-byte aligned)
-__global__ void __launch_bounds__(NA_T) k_na_tau_hook(const double *m, const double *x3, const double *v3, int n,
-                                                      TauParams P, NaScratch S)
+// label = root = smallest index of the component; a component is counted when
+// its second member arrives (one size update per root and warp); the last
+// block writes the count
+__global__ void k_na_compress(int n, NaScratch S, int32_t *labels, int64_t *n_comp_out)
 {
-    __shared__ double col[7][NA_T];
-    const int nt = (n + NA_T - 1) / NA_T;
-    int t = blockIdx.x, ti = 0;
-    while (t >= nt - ti) {
-        t -= nt - ti;
-        ++ti;
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    int r = -1;
+    if (k < n) {
+        r = uf_find(S.parent, k);
+        labels[k] = r;
     }
-    const int tj = ti + t;
-    const int j = tj * NA_T + threadIdx.x;
-    if (j < n) {
-        col[0][threadIdx.x] = x3[j];
-        col[1][threadIdx.x] = x3[(size_t)n + j];
-        col[2][threadIdx.x] = x3[2 * (size_t)n + j];
-        col[3][threadIdx.x] = v3[j];
-        col[4][threadIdx.x] = v3[(size_t)n + j];
-        col[5][threadIdx.x] = v3[2 * (size_t)n + j];
-        col[6][threadIdx.x] = m[j];
+    const unsigned peers = __match_any_sync(0xffffffffu, r);
+    if (r >= 0 && (threadIdx.x & 31) == __ffs(peers) - 1) {
+        const int add = __popc(peers), old = atomicAdd(&S.cnt[r], add);
+        if (old < 2 && old + add >= 2) atomicAdd(S.ncomp, 1);
     }
     __syncthreads();
-    const int i = ti * NA_T + threadIdx.x;
-    if (i >= n) return;
-    const double xi = x3[i], yi = x3[(size_t)n + i], zi = x3[2 * (size_t)n + i];
-    const double vxi = v3[i], vyi = v3[(size_t)n + i], vzi = v3[2 * (size_t)n + i], mi = m[i];
-    const int jn = min(NA_T, n - tj * NA_T);
-    for (int k = (ti == tj) ? threadIdx.x + 1 : 0; k < jn; ++k) {
-        const double tau = tau_fp64(__dsub_rn(xi, col[0][k]), __dsub_rn(yi, col[1][k]), __dsub_rn(zi, col[2][k]),
-                                    __dsub_rn(vxi, col[3][k]), __dsub_rn(vyi, col[4][k]),
-                                    __dsub_rn(vzi, col[5][k]), mi, col[6][k], P);
-        if (tau < P.h && !uf_union(S.parent, i, tj * NA_T + k)) atomicCAS(S.err, 0u, (unsigned)DERR_UF_RETRY);
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(S.done, 1u) == gridDim.x - 1) *n_comp_out = atomicAdd(S.ncomp, 0);
     }
 }
-
-// label = root = smallest index of the component; sizes by root
-__global__ void k_na_compress(int n, NaScratch S, int32_t *labels)
-{
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n) return;
-    const int r = uf_find(S.parent, k);
-    labels[k] = r;
-    atomicAdd(&S.cnt[r], 1);
-}
-
-__global__ void k_na_count(int n, NaScratch S, int64_t *n_comp_out)
-{
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < n && S.cnt[k] >= 2) atomicAdd(S.ncomp, 1);
-}
-
-__global__ void k_na_store(NaScratch S, int64_t *n_comp_out) { *n_comp_out = *S.ncomp; }
 
 }  // namespace cc
 
@@ -193,19 +167,16 @@ extern "C" int cc_components_noalloc(const double *m, const double *x3, const do
     P.near_tol = 0.0;
     P.fault_test = 0;
     const int ni = (int)n, g = (ni + 255) / 256;
-    const long long nt = (n + NA_T - 1) / NA_T;
     k_na_init<<<g, 256, 0, s>>>(S, ni);
-    k_na_tau_hook<<<(int)(nt * (nt + 1) / 2), NA_T, 0, s>>>(m, x3, v3, ni, P, S);
-    k_na_compress<<<g, 256, 0, s>>>(ni, S, labels_out);
-    k_na_count<<<g, 256, 0, s>>>(ni, S, n_comp_out);
-    k_na_store<<<1, 1, 0, s>>>(S, n_comp_out);
-    CC_COUNT_LAUNCH(5);
+    launch_tau_raw(m, x3, v3, ni, P, S.parent, S.ctr, s);
+    k_na_compress<<<g, 256, 0, s>>>(ni, S, labels_out, n_comp_out);
+    CC_COUNT_LAUNCH(2);
     if (cudaPeekAtLastError() != cudaSuccess) {  // a launch was refused: nothing was written
         cudaGetLastError();
         return CC_E_CUDA;
     }
     unsigned err = 0;
-    if (cudaMemcpyAsync(&err, S.err, sizeof(unsigned), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+    if (cudaMemcpyAsync(&err, &S.ctr->err, sizeof(unsigned), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess) {
         cudaGetLastError();
         return CC_E_CUDA;
