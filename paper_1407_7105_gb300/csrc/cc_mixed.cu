@@ -716,8 +716,9 @@ void launch_tau_mixed(const Level &L, const FFView &F, int ntiles, const TauPara
 }
 
 // the same over a caller's FP64 arrays as one set, hooked into `parent`: 256-wide
-// tiles while they give every SM two blocks, else 64-wide ones
-constexpr int TAU_RAW_WIDE_N = 6144;
+// tiles from where they are the faster ones (whole call, 256 / 64-wide: 2048
+// bodies 109 / 79 us, 3072 109 / 112, 4096 113 / 129, 8192 136 / 193)
+constexpr int TAU_RAW_WIDE_N = 3072;
 
 void launch_tau_raw(const double *m, const double *x3, const double *v3, int n, const TauParams &P, int32_t *parent,
                     DevCounters *ctr, cudaStream_t s)

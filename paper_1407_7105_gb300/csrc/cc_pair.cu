@@ -7,6 +7,7 @@
 // j-tiles are staged in shared memory by TMA bulk copies (cp.async.bulk)
 // completing on an mbarrier; every wait is bounded.
 #include "cc_device.cuh"
+#include "cc_fp64.cuh"
 
 namespace cc {
 
@@ -429,14 +430,11 @@ struct __align__(16) KickBSmem {
 // are left out; their kick is the centre-of-mass one that launch_com_apply
 // adds afterwards.  MODE 2 (OK split): the fast pairs (OkView: each row's
 // partners, sorted) are left out, every other pair of the set kicks.
-// MODE 3: as MODE 0 with each pair's force G m_j r_ij^-3 (x_j - x_i) read
-// from the matrices k_pair_forces filled (PairFactors) instead of computed;
-// MODE 4: as MODE 2 with the forces read.
 template <int MODE>
 __global__ void __launch_bounds__(KB_THREADS) k_kick64(Level L, const int32_t *label, double G, double eps2, double h,
-                                                       DevCounters *ctr, ComView cv, OkView okv, PairFactors pf)
+                                                       DevCounters *ctr, ComView cv, OkView okv)
 {
-    constexpr bool COM = MODE == 1, OKM = MODE == 2 || MODE == 4, PRE = MODE >= 3;
+    constexpr bool COM = MODE == 1, OKM = MODE == 2;
     __shared__ KickBSmem sm;
     const int tid = threadIdx.x;
     const int s = find_set(L.itile_off, L.nsets, blockIdx.x);
@@ -473,24 +471,6 @@ __global__ void __launch_bounds__(KB_THREADS) k_kick64(Level L, const int32_t *l
     const int r = tid & 31, c = tid >> 5;  // summing threads: row r, component c (tid < 96)
     double acc = 0.0;
     bool ok = true;
-    // MODE 3/4: this thread's pairs (row (tid >> 5) + 8 q, column tid & 31)
-    // of a j-tile, all three components, loaded a tile ahead
-    double fr[3][KB_Q];
-    const long long nn = (long long)n * n;
-    const double *F = PRE ? pf.S + pf.moff[s] : nullptr;
-    auto load_f = [&](int tj) {
-        const int jl0 = tj * KB_T, jn = min(KB_T, n - jl0);
-#pragma unroll
-        for (int q = 0; q < KB_Q; ++q) {
-            const int ii = (tid >> 5) + q * (KB_THREADS / KB_T), jj = tid & 31;
-            const bool v = ii < ni && jj < jn;
-            const long long e = (long long)(il0 + ii) * n + (jl0 + jj);
-            fr[0][q] = v ? F[e] : 0.0;
-            fr[1][q] = v ? F[nn + e] : 0.0;
-            fr[2][q] = v ? F[2 * nn + e] : 0.0;
-        }
-    };
-    if (PRE) load_f(0);
     for (int tj = 0; tj < nt; ++tj) {
         const int st = tj & 1;
         if (tid == 0 && tj + 1 < nt)
@@ -530,12 +510,6 @@ __global__ void __launch_bounds__(KB_THREADS) k_kick64(Level L, const int32_t *l
             if (COM && use && sm.ci[ii] >= 0 && sm.cj[jj] >= 0)
                 use = cv.far[fo + (long long)sm.ci[ii] * Ks + sm.cj[jj]] == 0;
             if (OKM && use) use = ((sm.okm[ii] >> jj) & 1u) == 0u;
-            if (PRE) {
-                sm.f[0][ii][jj] = use ? fr[0][q] : 0.0;
-                sm.f[1][ii][jj] = use ? fr[1][q] : 0.0;
-                sm.f[2][ii][jj] = use ? fr[2][q] : 0.0;
-                continue;
-            }
             const double dx0 = __dsub_rn(sm.j.col[st][0][jj], sm.xi[0][ii]);
             const double dx1 = __dsub_rn(sm.j.col[st][1][jj], sm.xi[1][ii]);
             const double dx2 = __dsub_rn(sm.j.col[st][2][jj], sm.xi[2][ii]);
@@ -547,8 +521,6 @@ __global__ void __launch_bounds__(KB_THREADS) k_kick64(Level L, const int32_t *l
             sm.f[1][ii][jj] = use ? __dmul_rn(w, dx1) : 0.0;
             sm.f[2][ii][jj] = use ? __dmul_rn(w, dx2) : 0.0;
         }
-        // the next j-tile's forces into registers while this one is summed
-        if (PRE && tj + 1 < nt) load_f(tj + 1);
         __syncthreads();
         if (tid < 3 * KB_T)
             for (int jj = 0; jj < jn; ++jj) acc = __dadd_rn(acc, sm.f[c][r][jj]);
@@ -568,18 +540,39 @@ __global__ void __launch_bounds__(KB_THREADS) k_kick64(Level L, const int32_t *l
     }
 }
 
-// The force G m_j r_ij^-3 (x_j - x_i) of every ordered pair (i, j) of each
-// set into its three n x n matrices (components x, y, z) at pf.moff[s] (row
-// i, column j; the diagonal unused).  One block per 128-wide triangular tile
-// (TI <= TJ; the grid and prefix L.tile_off of the 128-wide tau tiles), in
-// 32 x 32 sub-tiles: every unordered pair is evaluated once with the kick's
-// own operations (dx = x_j - x_i; the squares make r^2, and so r^-3, the same
-// bits for (j, i), and x_i - x_j = -dx exactly); (G m_j) r^-3 dx goes to row
-// i directly, -(G m_i) r^-3 dx to row j through shared memory.
+// rn(1 / rn(r2 rn(sqrt r2))) by the IEEE instructions: what rinv3_rn is, and
+// the way out where it does not apply
+__device__ __noinline__ double rinv3_ieee(double r2) { return __drcp_rn(__dmul_rn(r2, __dsqrt_rn(r2))); }
+
+// a + b as a fused multiply-add by a one the compiler cannot see: the same bits
+// (a times one is exact, zeros keep their signs), and a DFMA holds the pipe 64
+// cycles a warp where a DADD holds it 77 (both measured alone on it)
+__device__ __forceinline__ double add_fma(double a, double b, double one) { return __fma_rn(a, one, b); }
+
+// Three n x n matrices per set (components x, y, z) at pf.moff[s]: row j,
+// column i = the force G m_j r_ij^-3 (x_j - x_i) of j on i (the diagonal
+// unused), so that k_kick_rows, a lane per i, reads them straight.  One block
+// per 128-wide triangular tile (TI <= TJ; the grid and prefix L.tile_off of
+// the 128-wide tau tiles), in 32 x 32 sub-tiles: every unordered pair is
+// evaluated once with the kick's own operations (dx = x_j - x_i; the squares
+// make r^2, and so r^-3, the same bits for (j, i), and x_i - x_j = -dx
+// exactly); the force on j goes out directly, the force on i through shared
+// memory.
+//
+// What bounds it: the FP64 pipe, one warp instruction in 64 cycles.  Of a
+// pair's 18 IEEE operations (more with unequal masses or softening), two of
+// them a square root and a reciprocal, the five additions, two residuals and
+// two products stay there; the other products and r^-3 run on the integer and
+// FP32 pipes meanwhile (cc_fp64.cuh: 66 cycles a product, 300 r^-3).  Equal masses (a sub-tile's warp sees only one): the force on j is
+// the negated force on i, bit for bit.  16384 bodies (1.34e8 pairs): 8.6 ms
+// with every operation on the FP64 pipe, 2.4 ms so (two of the products left
+// on it; none 2.66, one 2.46, three 2.55, four 2.81 ms).
 constexpr int KR_T = 32, KR_W = 128;
 static_assert(KR_T == KB_T, "the force sub-tiles are the kick's i-tiles");
 static_assert(KR_W == TAU_VAR_T[TAU_VAR_128], "the force tiles are the 128-wide tau tiles");
-__global__ void __launch_bounds__(KB_THREADS) k_pair_forces(Level L, double G, double eps2, PairFactors pf)
+template <bool SOFT>
+__global__ void __launch_bounds__(KB_THREADS, 6) k_pair_forces(Level L, double G, double eps2, double one, double nzero,
+                                                            PairFactors pf)
 {
     __shared__ double xi[4][KR_W];  // x, y, z, G m
     __shared__ double xj[4][KR_W];
@@ -594,42 +587,86 @@ __global__ void __launch_bounds__(KB_THREADS) k_pair_forces(Level L, double G, d
     const int i0 = TI * KR_W, j0 = TJ * KR_W;
     const int ni = min(KR_W, n - i0), nj = min(KR_W, n - j0);
     double *S = pf.S + pf.moff[s];
+    bool in = true;  // every G m in the range of the integer products
     for (int e = tid; e < KR_W; e += KB_THREADS) {
         const bool vi = e < ni, vj = e < nj;
         xi[0][e] = vi ? L.x[start + i0 + e] : 0.0;
         xi[1][e] = vi ? L.y[start + i0 + e] : 0.0;
         xi[2][e] = vi ? L.z[start + i0 + e] : 0.0;
-        xi[3][e] = vi ? __dmul_rn(G, L.m[start + i0 + e]) : 0.0;
+        xi[3][e] = vi ? __dmul_rn(G, L.m[start + i0 + e]) : 1.0;
         xj[0][e] = vj ? L.x[start + j0 + e] : 0.0;
         xj[1][e] = vj ? L.y[start + j0 + e] : 0.0;
         xj[2][e] = vj ? L.z[start + j0 + e] : 0.0;
-        xj[3][e] = vj ? __dmul_rn(G, L.m[start + j0 + e]) : 0.0;
+        xj[3][e] = vj ? __dmul_rn(G, L.m[start + j0 + e]) : 1.0;
+        in = in && exp_fast(d2u(xi[3][e])) && exp_fast(d2u(xj[3][e]));
     }
+    in = __syncthreads_and(in) != 0;
     for (int a = 0; a < KR_W / KR_T; ++a) {
         for (int b = TI == TJ ? a : 0; b < KR_W / KR_T; ++b) {
             const int il = a * KR_T, jl = b * KR_T;
             if (il >= ni || jl >= nj) continue;  // (uniform over the block)
-            __syncthreads();  // (the staged rows, or the previous sub-tile's transposed write)
-#pragma unroll
+            __syncthreads();  // (the previous sub-tile's transposed write)
+#pragma unroll 1
             for (int q = 0; q < KB_Q; ++q) {
                 const int pidx = tid + q * KB_THREADS, ii = pidx >> 5, jj = pidx & 31;
                 const int gi = il + ii, gj = jl + jj;
-                if (gi < ni && gj < nj && j0 + gj > i0 + gi) {
-                    const double dx0 = __dsub_rn(xj[0][gj], xi[0][gi]);
-                    const double dx1 = __dsub_rn(xj[1][gj], xi[1][gi]);
-                    const double dx2 = __dsub_rn(xj[2][gj], xi[2][gi]);
+                const bool on = gi < ni && gj < nj && j0 + gj > i0 + gi;
+                const uint64_t gmj = d2u(xj[3][gj]), gmi = d2u(xi[3][gi]);
+                const bool same = __all_sync(0xffffffffu, !on || gmj == gmi);
+                if (!on) continue;
+                const double dx0 = add_fma(xj[0][gj], -xi[0][gi], one);
+                const double dx1 = add_fma(xj[1][gj], -xi[1][gi], one);
+                const double dx2 = add_fma(xj[2][gj], -xi[2][gi], one);
+                const uint64_t d0 = d2u(dx0), d1 = d2u(dx1), d2 = d2u(dx2);
+                uint64_t w, v, f0, f1, f2, g0, g1, g2;
+                bool fast = in && fast_range(d0) && fast_range(d1) && fast_range(d2);
+                if (fast) {
+                    double r2 = add_fma(add_fma(u2d(sqr_rn(d0)), u2d(sqr_rn(d1)), one), u2d(sqr_rn(d2)), one);
+                    if (SOFT) r2 = add_fma(r2, eps2, one);
+                    bool open = !exp_fast(d2u(r2));
+                    v = rinv3_rn(d2u(r2), open);
+                    if (open) {
+                        v = d2u(rinv3_ieee(r2));
+                        fast = exp_fast(d2u(r2));
+                    }
+                }
+                if (fast) {
+                    // (two of the three products of a force on the FP64 pipe: the
+                    // two pipes then finish about together)
+                    w = mul_rn(gmj, v);
+                    f0 = d2u(__fma_rn(u2d(w), dx0, nzero));
+                    f1 = d2u(__fma_rn(u2d(w), dx1, nzero));
+                    f2 = mul_rn(w, d2);
+                    if (same) {
+                        g0 = f0;
+                        g1 = f1;
+                        g2 = f2;
+                    } else {
+                        w = mul_rn(gmi, v);
+                        g0 = mul_rn(w, d0);
+                        g1 = mul_rn(w, d1);
+                        g2 = mul_rn(w, d2);
+                    }
+                } else {
                     const double r2 = __dadd_rn(
                         __dadd_rn(__dadd_rn(__dmul_rn(dx0, dx0), __dmul_rn(dx1, dx1)), __dmul_rn(dx2, dx2)), eps2);
-                    const double v = __drcp_rn(__dmul_rn(r2, __dsqrt_rn(r2)));
-                    const double wij = __dmul_rn(xj[3][gj], v), wji = __dmul_rn(xi[3][gi], v);
-                    const long long e = (long long)(i0 + gi) * n + (j0 + gj);
-                    S[e] = __dmul_rn(wij, dx0);
-                    S[nn + e] = __dmul_rn(wij, dx1);
-                    S[2 * nn + e] = __dmul_rn(wij, dx2);
-                    t[0][ii][jj] = -__dmul_rn(wji, dx0);
-                    t[1][ii][jj] = -__dmul_rn(wji, dx1);
-                    t[2][ii][jj] = -__dmul_rn(wji, dx2);
+                    const double vd = rinv3_ieee(r2);
+                    const double wij = __dmul_rn(u2d(gmj), vd), wji = __dmul_rn(u2d(gmi), vd);
+                    f0 = d2u(__dmul_rn(wij, dx0));
+                    f1 = d2u(__dmul_rn(wij, dx1));
+                    f2 = d2u(__dmul_rn(wij, dx2));
+                    g0 = d2u(__dmul_rn(wji, dx0));
+                    g1 = d2u(__dmul_rn(wji, dx1));
+                    g2 = d2u(__dmul_rn(wji, dx2));
                 }
+                const uint64_t minus = 1ull << 63;
+                const long long e = (long long)(i0 + gi) * n + (j0 + gj);
+                S[e] = u2d(g0 ^ minus);
+                S[nn + e] = u2d(g1 ^ minus);
+                S[2 * nn + e] = u2d(g2 ^ minus);
+                t[0][ii][jj] = u2d(f0);
+                t[1][ii][jj] = u2d(f1);
+                t[2][ii][jj] = u2d(f2);
             }
             __syncthreads();
 #pragma unroll
@@ -647,6 +684,127 @@ __global__ void __launch_bounds__(KB_THREADS) k_pair_forces(Level L, double G, d
     }
 }
 
+// v_i += h sum_j (force of j on i) from k_pair_forces' matrices, over the j of
+// the set in ascending order whose label differs (and, OKM, that are not
+// among i's fast partners, which are sorted): the terms and the order of
+// k_kick64 (a left-out term is an exact +0), so its bits.
+//
+// What bounds it: the chain of n additions of a row, one in 64 cycles however
+// few rows there are, times the warps on a scheduler (3 for 16384 rows).  A
+// warp issues in order, so whatever else it does between two additions comes
+// on top (158 cycles a column when one warp also copied and masked its
+// columns).  Hence two warps: one takes 32 rows of one component, lane = row,
+// and only reads shared memory and adds; its helper copies the columns
+// (coalesced 256-byte pieces, 48 columns ahead) and overwrites the left-out
+// terms with zero; they meet once per KW columns at a barrier of their own.
+// Four pairs a block, so every scheduler gets the same number.  24 bytes a
+// pair, 4.7 TB/s at the additions' rate.  A 16384-body step: 8.5 ms when the
+// tiles were staged by 256 threads for 96 to add, 7.9 ms so.
+constexpr int KW = 16;                      // columns a stage
+constexpr int KR_PAIRS = 4, KR_STAGES = 4;  // 16 KB a pair
+constexpr int KR_SMEM = KR_PAIRS * KR_STAGES * KW * 32 * 8;
+
+// 8 bytes global -> shared, asynchronous (rows of odd n are 8-byte aligned only)
+__device__ __forceinline__ void cp_async8(unsigned dst, const double *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
+}
+
+template <bool OKM>
+__global__ void __launch_bounds__(64 * KR_PAIRS) k_kick_rows(Level L, const int32_t *label, double h, double one,
+                                                             int nitiles, OkView okv, PairFactors pf)
+{
+    extern __shared__ __align__(16) double ring[];  // [pair][stage][column][lane]
+    const int p = (threadIdx.x >> 5) % KR_PAIRS, lane = threadIdx.x & 31;
+    const bool adds = threadIdx.x < 32 * KR_PAIRS;
+    const int w = blockIdx.x * KR_PAIRS + p, tile = w / 3, c = w % 3;
+    if (tile >= nitiles) return;  // (both warps of the pair)
+    const int s = find_set(L.itile_off, L.nsets, tile);
+    const int n = L.set_n[s], start = L.set_start[s];
+    const int il = (tile - L.itile_off[s]) * KB_T + lane;
+    const bool on = il < n;
+    const int i = start + (on ? il : n - 1);
+    double *mine = ring + p * (KR_STAGES * KW * 32) + lane;
+    const int nk = (n + KW - 1) / KW;
+    // (immediate numbers: a register operand would claim all 16 barriers)
+    auto meet = [&]() {
+        if (p == 0) asm volatile("bar.sync 1, 64;" ::: "memory");
+        else if (p == 1) asm volatile("bar.sync 2, 64;" ::: "memory");
+        else if (p == 2) asm volatile("bar.sync 3, 64;" ::: "memory");
+        else asm volatile("bar.sync 4, 64;" ::: "memory");
+    };
+    static_assert(KR_PAIRS == 4, "one barrier a pair");
+    if (adds) {
+        double acc = 0.0;
+        for (int k = 0; k < nk; ++k) {
+            meet();  // stage k is ready
+            const double *f = mine + (k % KR_STAGES) * (KW * 32);
+#pragma unroll
+            for (int u = 0; u < KW; ++u) acc = add_fma(f[u * 32], acc, one);
+        }
+        if (on) {
+            double *v = c == 0 ? L.vx : (c == 1 ? L.vy : L.vz);
+            v[i] = __dadd_rn(v[i], __dmul_rn(h, acc));
+        }
+        return;
+    }
+    const double *F = pf.S + pf.moff[s] + (long long)c * n * n + (i - start);
+    const int32_t *lab = label + start;  // (sets start at multiples of four elements)
+    const int li = label[i];
+    // OKM: the columns of the row's next two fast partners (the second is read
+    // long before it is needed)
+    int fast = 0x7fffffff, ahead = 0x7fffffff, fq = 0, fe = 0;
+    auto next_fast = [&]() {
+        fast = ahead;
+        ahead = fq < fe ? okv.col[2 * (long long)fq + 1] - start : 0x7fffffff;
+        ++fq;
+    };
+    if (OKM) {
+        fq = okv.row_ptr[i];
+        fe = okv.row_ptr[i + 1];
+        next_fast();
+        next_fast();
+    }
+    const unsigned mine_s = smem_u32(mine);
+    auto issue = [&](int k) {
+        const unsigned d = mine_s + (k % KR_STAGES) * (KW * 32 * 8);
+#pragma unroll
+        for (int u = 0; u < KW; ++u) {
+            if (k * KW + u < n) cp_async8(d + u * 256, F);
+            F += n;
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+#pragma unroll
+    for (int k = 0; k < KR_STAGES - 1; ++k) issue(k);
+    for (int k = 0; k < nk; ++k) {
+        const int j = k * KW;
+        uint32_t out = 0u;  // the stage's left-out columns
+        if (OKM) {
+            while (fast < j + KW) {
+                out |= 1u << (fast - j);
+                next_fast();
+            }
+        }
+        // (past a set's end the labels are its padding's or the next set's, in
+        // the same buffer: those columns are left out whatever they hold)
+#pragma unroll
+        for (int u = 0; u < KW; u += 4) {
+            const int4 l = *reinterpret_cast<const int4 *>(lab + j + u);
+            out |= (l.x == li ? 1u << u : 0u) | (l.y == li ? 2u << u : 0u) | (l.z == li ? 4u << u : 0u) |
+                   (l.w == li ? 8u << u : 0u);
+        }
+        if (j + KW > n) out |= 0xffffffffu << (n - j);
+        asm volatile("cp.async.wait_group %0;" ::"n"(KR_STAGES - 2) : "memory");
+        double *f = mine + (k % KR_STAGES) * (KW * 32);
+#pragma unroll
+        for (int u = 0; u < KW; ++u)
+            if (out >> u & 1u) f[u * 32] = 0.0;
+        meet();                    // stage k to the adding warp, which is done with stage k - 1
+        issue(k + KR_STAGES - 1);  // into that one's place
+    }
+}
+
 void launch_kick(const Level &L, const int32_t *label, int nitiles, double G, double eps2, double h,
                  int variant, DevCounters *ctr, cudaStream_t s, const ComView *com, const OkView *okv,
                  const PairFactors *pf)
@@ -655,21 +813,25 @@ void launch_kick(const Level &L, const int32_t *label, int nitiles, double G, do
     if (nitiles <= 0) return;
     const ComView nc{nullptr, nullptr, nullptr, nullptr};
     const OkView no{nullptr, nullptr};
-    const PairFactors np{nullptr, nullptr, 0};
-    if (okv && okv->row_ptr && pf && pf->S) {
-        k_pair_forces<<<pf->nblocks, KB_THREADS, 0, s>>>(L, G, eps2, *pf);
-        k_kick64<4><<<nitiles, KB_THREADS, 0, s>>>(L, label, G, eps2, h, ctr, nc, *okv, *pf);
+    const bool pre = pf && pf->S && !(com && com->cl);
+    if (pre) {
+        if (eps2 != 0.0) k_pair_forces<true><<<pf->nblocks, KB_THREADS, 0, s>>>(L, G, eps2, 1.0, -0.0, *pf);
+        else k_pair_forces<false><<<pf->nblocks, KB_THREADS, 0, s>>>(L, G, eps2, 1.0, -0.0, *pf);
+        const int nb = (3 * nitiles + KR_PAIRS - 1) / KR_PAIRS;
+        if (okv && okv->row_ptr) {
+            cudaFuncSetAttribute(k_kick_rows<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, KR_SMEM);
+            k_kick_rows<true><<<nb, 64 * KR_PAIRS, KR_SMEM, s>>>(L, label, h, 1.0, nitiles, *okv, *pf);
+        } else {
+            cudaFuncSetAttribute(k_kick_rows<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, KR_SMEM);
+            k_kick_rows<false><<<nb, 64 * KR_PAIRS, KR_SMEM, s>>>(L, label, h, 1.0, nitiles, no, *pf);
+        }
         CC_COUNT_LAUNCH(1);
     } else if (okv && okv->row_ptr) {
-        k_kick64<2><<<nitiles, KB_THREADS, 0, s>>>(L, label, G, eps2, h, ctr, nc, *okv, np);
+        k_kick64<2><<<nitiles, KB_THREADS, 0, s>>>(L, label, G, eps2, h, ctr, nc, *okv);
     } else if (com && com->cl) {
-        k_kick64<1><<<nitiles, KB_THREADS, 0, s>>>(L, label, G, eps2, h, ctr, *com, no, np);
-    } else if (pf && pf->S) {
-        k_pair_forces<<<pf->nblocks, KB_THREADS, 0, s>>>(L, G, eps2, *pf);
-        k_kick64<3><<<nitiles, KB_THREADS, 0, s>>>(L, label, G, eps2, h, ctr, nc, no, *pf);
-        CC_COUNT_LAUNCH(1);
+        k_kick64<1><<<nitiles, KB_THREADS, 0, s>>>(L, label, G, eps2, h, ctr, *com, no);
     } else {
-        k_kick64<0><<<nitiles, KB_THREADS, 0, s>>>(L, label, G, eps2, h, ctr, nc, no, np);
+        k_kick64<0><<<nitiles, KB_THREADS, 0, s>>>(L, label, G, eps2, h, ctr, nc, no);
     }
     CC_COUNT_LAUNCH(1);
 }

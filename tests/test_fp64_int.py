@@ -1,0 +1,78 @@
+"""The FP64 products and r^-3 that csrc/cc_fp64.cuh computes on the integer and
+FP32 pipes, compiled for the host and compared bit for bit with the machine's
+own IEEE operations (the FP32 estimates moved by up to their hardware error
+bounds): random significands, ones next to powers of two and to ties, exponents
+over the whole accepted range, zeros."""
+import os
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+SRC = r'''
+#include <cstdio>
+#include <cstdlib>
+#include <random>
+#include "cc_fp64.cuh"
+namespace cc { float est_shift = 0.0f; }
+using namespace cc;
+static std::mt19937_64 g(7);
+static double draw(int emin, int emax)
+{
+    uint64_t m = g() & 0xfffffffffffffull;
+    switch (g() % 6) {
+    case 0: m &= ~0ull << (g() % 53); break;          // few leading bits
+    case 1: m |= ~(~0ull << (g() % 53)); break;       // trailing ones
+    case 2: m = (g() & 7); break;                     // just above a power of two
+    case 3: m = 0xfffffffffffffull - (g() & 7); break;
+    default: break;
+    }
+    m &= 0xfffffffffffffull;
+    const uint64_t e = 1023 + emin + (int)(g() % (uint64_t)(emax - emin + 1));
+    return u2d((e << 52) | m | ((g() & 1) << 63));
+}
+int main(int argc, char **argv)
+{
+    const long n = atol(argv[1]);
+    const float shifts[5] = {0.0f, 1.2e-7f, -1.2e-7f, 6e-8f, -6e-8f};
+    long opened = 0, bad = 0, plain = 0;
+    for (long i = 0; i < n; ++i) {
+        const double a = i % 97 == 0 ? 0.0 * draw(0, 0) : draw(-200, 200), b = draw(-200, 200);
+        volatile double ab = a * b, aa = a * a;
+        if (mul_rn(d2u(a), d2u(b)) != d2u(ab)) { if (++bad < 9) printf("mul %a %a\n", a, b); }
+        if (sqr_rn(d2u(a)) != d2u(aa)) { if (++bad < 9) printf("sqr %a\n", a); }
+        const double x = std::fabs(draw(-200, 200));
+        est_shift = shifts[i % 5];
+        bool open = false;
+        const uint64_t v = rinv3_rn(d2u(x), open);
+        volatile double s = std::sqrt(x), c = x * s, r = 1.0 / c;
+        // (significands without a pattern: the share left to the IEEE path)
+        bool po = false;
+        const double px = u2d((g() & 0xfffffffffffffull) | ((1023 - 200 + g() % 401) << 52));
+        const uint64_t pv = rinv3_rn(d2u(px), po);
+        volatile double ps = std::sqrt(px), pc = px * ps, pr = 1.0 / pc;
+        ++plain;
+        if (po) ++opened;
+        else if (pv != d2u(pr)) { if (++bad < 9) printf("rinv3 %a\n", px); }
+        if (!open && (v != d2u(r))) { if (++bad < 9) printf("rinv3 %a\n", x); }
+        if (!exp_fast(d2u(x)) || !fast_range(d2u(a))) { if (++bad < 9) printf("range %a %a\n", x, a); }
+    }
+    const double out[6] = {1e-300, 5e-324, 1e300, HUGE_VAL, NAN, 1e-62};
+    for (double o : out) if (fast_range(d2u(o))) { ++bad; printf("accepts %a\n", o); }
+    if (!fast_range(d2u(-0.0)) || exp_fast(d2u(0.0))) ++bad;
+    printf("open %ld of %ld, bad %ld\n", opened, plain, bad);
+    return bad != 0 || opened > plain / 1000;  // 2^-11 expected
+}
+'''
+
+
+@pytest.mark.parametrize("opt", ["-O2"])
+def test_against_the_machine(tmp_path, opt):
+    src = tmp_path / "t.cpp"
+    src.write_text(SRC)
+    exe = tmp_path / "t"
+    subprocess.run(["g++", opt, "-std=c++17", "-ffp-contract=off", "-x", "c++", "-I",
+                    os.path.join(ROOT, "paper_1407_7105_gb300", "csrc"), str(src), "-o", str(exe)], check=True)
+    r = subprocess.run([str(exe), "4000000"], capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout
