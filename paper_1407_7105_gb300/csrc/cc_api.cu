@@ -1972,7 +1972,8 @@ int cc_reset_stats(cc_ctx *c)
 int cc_energy(cc_ctx *c, double *E, double *P3, double *L3)
 {
     if (!c) return CC_E_ARG;
-    const int nb = energy_blocks(c->n);
+    const int nsys = (int)c->sys_off.size() - 1;
+    const int nb = energy_blocks(c->n, nsys, c->nsm);
     if (nb > c->partial_cap) {
         if (c->d_partial) cudaFree(c->d_partial);
         c->d_partial = nullptr;
@@ -1980,7 +1981,7 @@ int cc_energy(cc_ctx *c, double *E, double *P3, double *L3)
         c->partial_cap = nb;
     }
     launch_energy(c->d_x3, c->d_v3, c->d_m, c->n, c->p.G, c->p.eps * c->p.eps, c->d_sys_off,
-                  (int)c->sys_off.size() - 1, c->d_partial, nb, c->stream);
+                  nsys, c->d_partial, nb, c->stream);
     std::vector<double> h((size_t)nb * 8);
     CC_CUDA(c, cudaMemcpyAsync(h.data(), c->d_partial, h.size() * 8, cudaMemcpyDeviceToHost, c->stream));
     CC_CUDA(c, cudaStreamSynchronize(c->stream));

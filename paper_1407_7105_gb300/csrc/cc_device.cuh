@@ -32,8 +32,10 @@ constexpr float SLACK = 2e-6f;
 struct MixedTauParams {
     float eta, etah, eps2, G;
     float hq;  // eta/etah (h, or h/eta when eta multiplies the min): the pre-test's q = hq |dv|/r
-    // tau_pair_bounds' constants (mixed_tau_params): c^2, T, V of the bounds
-    // below; pb_c2 < 0: the bounds are off
+};
+// the tau kernel's: with tau_pair_bounds' constants (c^2, T^2, V of its bounds;
+// pb_c2 < 0: they are off)
+struct MixedTauBounds : MixedTauParams {
     float pb_c2, pb_r3, pb_v;
 };
 
@@ -244,7 +246,7 @@ struct PairBounds {
     float p0, w0;  // eps^2 - r_min^2, -v_thr^2
 };
 
-__device__ __forceinline__ bool tau_pair_bounds(float amax, float vabs, float mu_max, const MixedTauParams &Q,
+__device__ __forceinline__ bool tau_pair_bounds(float amax, float vabs, float mu_max, const MixedTauBounds &Q,
                                                 PairBounds &b)
 {
     const float mu = mu_max * 1.0001f;
@@ -260,9 +262,9 @@ __device__ __forceinline__ bool tau_pair_bounds(float amax, float vabs, float mu
 }
 
 // the FP32 constants of a split at threshold P.h
-inline MixedTauParams mixed_tau_params(const TauParams &P)
+inline MixedTauBounds mixed_tau_params(const TauParams &P)
 {
-    MixedTauParams Q;
+    MixedTauBounds Q;
     const double etah = P.eta_outside ? P.eta_in * P.eta / P.h : P.eta_in / P.h;
     const double hq = P.eta_outside ? P.h / P.eta : P.h;  // h/eta_in in the units of T: eta_in/etah
     Q.eta = (float)P.eta_in;

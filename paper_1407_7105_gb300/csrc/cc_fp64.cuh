@@ -14,7 +14,9 @@
 //                    division and square root by Newton steps), the
 //                    correction in units of the last place, and an integer
 //                    rounding of it; a correction too close to a tie for its
-//                    error is reported, and the caller takes the IEEE path.
+//                    error is reported, and the caller takes the IEEE path;
+//   rsqrt_near     : x^-1/2 to 0.51 units of the last place by the same steps,
+//                    for sums that ask for no particular bits.
 // The callers see to the ranges (fast_range): no operand or result is
 // subnormal, infinite or NaN here; zero operands of mul_rn and sqr_rn are.
 // The header compiles for the host too, where the tests compare every
@@ -194,6 +196,49 @@ CC_HD uint64_t rinv3_rn(uint64_t x, bool &open)
     // x = m 2^(2k): C 2^(3k), so the result is Q 2^-(f + 3k)
     const int32_t k = (E - (int32_t)p) >> 1;
     return Q - ((uint64_t)(int64_t)(f + 3 * k) << 52);
+}
+
+// a b for positive normal operands, cut off after 53 bits; rem = the next 32
+CC_HD uint64_t mul_cut(uint64_t a, uint64_t b, uint32_t &rem)
+{
+    const uint32_t a1 = (uint32_t)(a >> 32), b1 = (uint32_t)(b >> 32);
+    const uint32_t ah = (a1 & 0xfffffu) | 0x100000u, al = (uint32_t)a;
+    const uint32_t bh = (b1 & 0xfffffu) | 0x100000u, bl = (uint32_t)b;
+    const uint64_t p1 = (uint64_t)ah * bl + (((uint64_t)al * bl) >> 32);
+    const uint64_t p2 = (uint64_t)al * bh + (uint32_t)p1;
+    const uint64_t p3 = (uint64_t)ah * bh + (p1 >> 32) + (p2 >> 32);
+    const uint32_t h = (uint32_t)(p3 >> 32), l = (uint32_t)p3, t = (uint32_t)p2, big = h >> 9, s = 12u - big;
+    rem = t << s;
+    const uint32_t ex = (a1 & 0x7ff00000u) + (b1 & 0x7ff00000u) - (1024u << 20) + (big << 20);
+    return ((uint64_t)(shl_f(h, l, s) + ex) << 32) | shl_f(l, t, s);
+}
+
+// x^-1/2 for x > 0 with exp_fast(x), within 0.51 ulp
+CC_HD uint64_t rsqrt_near(uint64_t x)
+{
+    const uint32_t h = (uint32_t)(x >> 32), lo = (uint32_t)x;
+    const int32_t E = (int32_t)(h >> 20) - 1023;
+    const uint32_t p = (uint32_t)E & 1u;
+    const uint64_t m = ((uint64_t)((h & 0xfffffu) | ((1023u + p) << 20)) << 32) | lo;  // [1, 4)
+    const float mh = u2f(((h & 0xfffffu) << 3 | lo >> 29) + ((127u + p) << 23)), ml = low_part(lo, p);
+    // y to 2^-22 in [1/2, 1), its FP32 residual e = 1 - m y^2, Z0 to 2^-44
+    float y = rsqrt_est(mh);
+    y = y < 0.5f ? 0.5f : (y > 0.99999994f ? 0.99999994f : y);
+    const float t = mh * y, tl = fma_f(mh, y, -t) + ml * y;
+    const float e = fma_f(-tl, y, fma_f(-t, y, 1.0f));
+    const float zl = y * e * fma_f(0.375f, e, 0.5f);
+    const uint64_t Z0 = 0x3fe0000000000000ull + ((uint64_t)(f2u(y) - 0x3f000000u) << 29) +
+                        (uint64_t)((int64_t)rint_i(zl * 4503599627370496.0f) * 2);
+    // the residual 1 - m Z0^2 (the product's first 53 bits by an FP64
+    // instruction, the rest of it in FP32), its correction in units of 2^-53
+    const double z0 = u2d(Z0);
+    uint32_t rem;
+    const uint64_t u = mul_cut(m, Z0, rem);
+    // (2^-84 times the product's exponent: rem counts 2^-32 of its last place)
+    const float ul = (float)rem * u2f((uint32_t)((u >> 52) - 1023u + 43u) << 23);
+    const float r = trunc_f(d2u(fma_d(-u2d(u), z0, 1.0))) - ul * y;
+    const uint64_t Z = Z0 + (uint64_t)(int64_t)rint_i(r * (y * 4503599627370496.0f));
+    return Z - ((uint64_t)(int64_t)((E - (int32_t)p) >> 1) << 52);
 }
 
 }  // namespace cc

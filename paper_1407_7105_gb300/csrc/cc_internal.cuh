@@ -380,7 +380,7 @@ void launch_ok_tree(const Level &L, const int32_t *list, const long long *seg, c
 void launch_energy(const double *x3, const double *v3, const double *m, long long n, double G, double eps2,
                    const int32_t *sys_off /* nsys + 1 offsets, or null */, int nsys, double *partial /*[nblk*8]*/,
                    int nblk, cudaStream_t s);
-int energy_blocks(long long n);
+int energy_blocks(long long n, int nsys, int nsm);
 
 // cc_graph.cu
 void launch_compress(const Level &L, int32_t *root, cudaStream_t s);

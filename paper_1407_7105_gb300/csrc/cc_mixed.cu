@@ -418,7 +418,7 @@ __device__ __noinline__ void tau_record(MixedTauSmem<T, S, R> &sm, int w, int ne
 template <int T, int S, int R, bool RAW>
 __global__ void __launch_bounds__(T *S / R, 768 * R / (T * S))
     k_tau_mixed(const __grid_constant__ Level L, const __grid_constant__ FFView F,
-                const __grid_constant__ TauParams P, const __grid_constant__ MixedTauParams Q, DevCounters *ctr,
+                const __grid_constant__ TauParams P, const __grid_constant__ MixedTauBounds Q, DevCounters *ctr,
                 int32_t *near_ij, double *near_tau, long long near_cap, const __grid_constant__ EdgeList E)
 {
     constexpr int THREADS = T * S / R, NW = THREADS / 32, RW = T / (32 * R);
@@ -700,7 +700,7 @@ void launch_tau_mixed(const Level &L, const FFView &F, int ntiles, const TauPara
                       cudaStream_t s)
 {
     if (ntiles <= 0) return;
-    const MixedTauParams Q = mixed_tau_params(P);
+    const MixedTauBounds Q = mixed_tau_params(P);
     static_assert(TAU_VAR_T[0] == 64 && TAU_VAR_T[1] == 128 && TAU_VAR_T[2] == 64 && TAU_VAR_S[2] == 2 &&
                       TAU_VAR_T[3] == 256,
                   "tau variants");
@@ -731,7 +731,7 @@ void launch_tau_raw(const double *m, const double *x3, const double *v3, int n, 
     L.m = const_cast<double *>(m);
     L.parent = parent;
     L.total = n;
-    const MixedTauParams Q = mixed_tau_params(P);
+    const MixedTauBounds Q = mixed_tau_params(P);
     const FFView F{};
     const EdgeList E{nullptr, nullptr, 0};
     if (n >= TAU_RAW_WIDE_N) {

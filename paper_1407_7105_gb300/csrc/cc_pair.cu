@@ -8,10 +8,16 @@
 // completing on an mbarrier; every wait is bounded.
 #include "cc_device.cuh"
 #include "cc_fp64.cuh"
+#include <algorithm>
 
 namespace cc {
 
 // ------------------------------------------------------------ helpers
+// a + b as a fused multiply-add by a one the compiler cannot see: the same bits
+// (a times one is exact, zeros keep their signs), and a DFMA holds the pipe 64
+// cycles a warp where a DADD holds it 77 (both measured alone on it)
+__device__ __forceinline__ double add_fma(double a, double b, double one) { return __fma_rn(a, one, b); }
+
 __device__ __forceinline__ int find_set(const int32_t *off, int nsets, int b)
 {
     int lo = 0, hi = nsets;  // off[lo] <= b < off[hi]
@@ -544,11 +550,6 @@ __global__ void __launch_bounds__(KB_THREADS) k_kick64(Level L, const int32_t *l
 // the way out where it does not apply
 __device__ __noinline__ double rinv3_ieee(double r2) { return __drcp_rn(__dmul_rn(r2, __dsqrt_rn(r2))); }
 
-// a + b as a fused multiply-add by a one the compiler cannot see: the same bits
-// (a times one is exact, zeros keep their signs), and a DFMA holds the pipe 64
-// cycles a warp where a DADD holds it 77 (both measured alone on it)
-__device__ __forceinline__ double add_fma(double a, double b, double one) { return __fma_rn(a, one, b); }
-
 // Three n x n matrices per set (components x, y, z) at pf.moff[s]: row j,
 // column i = the force G m_j r_ij^-3 (x_j - x_i) of j on i (the diagonal
 // unused), so that k_kick_rows, a lane per i, reads them straight.  One block
@@ -837,70 +838,130 @@ void launch_kick(const Level &L, const int32_t *label, int nitiles, double G, do
 }
 
 // ------------------------------------------------------------ energy
-constexpr int EN_T = 128;
+constexpr int EN_T = 128;  // rows of a block's tile, one a thread
+constexpr int EN_C = 32;   // its columns
 
-int energy_blocks(long long n) { return (int)((n + EN_T - 1) / EN_T); }
+// tiles (128 rows x 32 columns) holding a pair i < j; blocks share them in turn
+int energy_blocks(long long n, int nsys, int nsm)
+{
+    const long long nt = (n + EN_T - 1) / EN_T, nc = (n + EN_C - 1) / EN_C;
+    const long long tiles = nsys > 1 ? nt : nt * nc - 2 * nt * (nt - 1);
+    return (int)std::min<long long>(tiles, 8ll * nsm);
+}
 
 // Kinetic and potential energy, momentum and angular momentum.  With
 // independent systems (sys_off, nsys + 1 offsets) the potential sums only
 // pairs inside one system: systems never interact, so a pair of two
 // systems belongs to no system's Hamiltonian.
-__global__ void __launch_bounds__(EN_T) k_energy(const double *x3, const double *v3, const double *m,
-                                                  long long n, double G, double eps2, const int32_t *sys_off,
-                                                  int nsys, double *partial)
+//
+// What bounds it: the FP64 pipe.  A pair's IEEE square root and quotient (~35
+// issue slots of 64 cycles with the rest) became r^-1 by rsqrt_near, 0.51 ulp
+// off the FP64 pipe but for one residual; left on it are the differences,
+// two of r^2's three products, the residual and the sum m_j/r: seven.  One
+// system's triangle is cut into tiles of 128 x 32 that the blocks take in
+// turn (rows of very different length left the chip to the last of them).
+// 65536 bodies (2.1e9 pairs): 141.8 ms before, 27.9 ms now (31.6 with all three
+// products of r^2 on the FP64 pipe).
+template <bool ONE, bool SOFT>
+__global__ void __launch_bounds__(EN_T, 8) k_energy(const double *x3, const double *v3, const double *m,
+                                                  long long n, double G, double eps2, double one,
+                                                  const int32_t *sys_off, int nsys, double *partial)
 {
-    __shared__ double sx[EN_T], sy[EN_T], sz[EN_T], smm[EN_T];
+    __shared__ double2 sxy[EN_C], szm[EN_C];
     __shared__ double red[8][EN_T / 32];
     __shared__ long long blk_hi;
-    const long long i = (long long)blockIdx.x * EN_T + threadIdx.x;
-    const bool iv = i < n;
-    double xi = 0, yi = 0, zi = 0, mi = 0, vx = 0, vy = 0, vz = 0;
-    if (iv) {
-        xi = x3[i]; yi = x3[n + i]; zi = x3[2 * n + i];
-        vx = v3[i]; vy = v3[n + i]; vz = v3[2 * n + i];
-        mi = m[i];
-    }
-    // the end of i's system (binary search over the offsets)
-    long long hi = n;
-    if (iv && sys_off && nsys > 1) {
-        int lo = 0, up = nsys;  // sys_off[lo] <= i < sys_off[up]
-        while (up - lo > 1) {
-            const int mid = (lo + up) >> 1;
-            if ((long long)sys_off[mid] <= i) lo = mid;
-            else up = mid;
-        }
-        hi = sys_off[up];
-    }
-    if (threadIdx.x == 0) blk_hi = 0;
-    __syncthreads();
-    if (iv) atomicMax((unsigned long long *)&blk_hi, (unsigned long long)hi);
-    __syncthreads();
-    const long long jend = blk_hi;
-    double V = 0.0;
-    for (long long j0 = (long long)blockIdx.x * EN_T; j0 < jend; j0 += EN_T) {
-        const long long j = j0 + threadIdx.x;
-        __syncthreads();
-        if (j < n) {
-            sx[threadIdx.x] = x3[j]; sy[threadIdx.x] = x3[n + j]; sz[threadIdx.x] = x3[2 * n + j];
-            smm[threadIdx.x] = m[j];
-        }
-        __syncthreads();
-        if (iv) {
-            const int jn = (int)min((long long)EN_T, n - j0);
-            for (int k = 0; k < jn; ++k) {
-                if (j0 + k <= i || j0 + k >= hi) continue;
-                const double dx = sx[k] - xi, dy = sy[k] - yi, dz = sz[k] - zi;
-                V -= G * mi * smm[k] / sqrt(dx * dx + dy * dy + dz * dz + eps2);
+    const long long nt = (n + EN_T - 1) / EN_T, nc = (n + EN_C - 1) / EN_C;
+    double q[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    double xi = 0, yi = 0, zi = 0, mi = 0;
+    long long i = 0, hi = 0;
+    auto take_row = [&](long long b) {  // this thread's body of row tile b, its system's end
+        i = b * EN_T + threadIdx.x;
+        hi = i < n ? n : 0;
+        if (i < n) {
+            xi = x3[i]; yi = x3[n + i]; zi = x3[2 * n + i];
+            mi = m[i];
+            if (!ONE) {
+                int lo = 0, up = nsys;  // sys_off[lo] <= i < sys_off[up]
+                while (up - lo > 1) {
+                    const int mid = (lo + up) >> 1;
+                    if ((long long)sys_off[mid] <= i) lo = mid;
+                    else up = mid;
+                }
+                hi = sys_off[up];
             }
         }
+    };
+    auto single = [&]() {  // the body's own terms, once a row tile
+        if (i >= n) return;
+        const double vx = v3[i], vy = v3[n + i], vz = v3[2 * n + i];
+        q[0] += 0.5 * mi * (vx * vx + vy * vy + vz * vz);
+        q[2] += mi * vx; q[3] += mi * vy; q[4] += mi * vz;
+        q[5] += mi * (yi * vz - zi * vy);
+        q[6] += mi * (zi * vx - xi * vz);
+        q[7] += mi * (xi * vy - yi * vx);
+    };
+    auto columns = [&](long long c) {  // sum of m_j/r over column tile c
+        const long long j0 = c * EN_C;
+        __syncthreads();
+        if (threadIdx.x < EN_C && j0 + threadIdx.x < n) {
+            const long long j = j0 + threadIdx.x;
+            sxy[threadIdx.x] = make_double2(x3[j], x3[n + j]);
+            szm[threadIdx.x] = make_double2(x3[2 * n + j], m[j]);
+        }
+        __syncthreads();
+        const int k0 = (int)max(0ll, i + 1 - j0), k1 = (int)min((long long)EN_C, hi - j0);
+        double acc = 0.0;
+#pragma unroll 2
+        for (int k = 0; k < EN_C; ++k) {
+            const double2 a = sxy[k], b = szm[k];
+            const double dx = add_fma(a.x, -xi, one), dy = add_fma(a.y, -yi, one), dz = add_fma(b.x, -zi, one);
+            const uint64_t dzb = d2u(dz);
+            const bool in = k >= k0 && k < k1;
+            double r2;
+            bool fast = fast_range(dzb);
+            if (fast) {
+                r2 = fma(dx, dx, fma(dy, dy, u2d(sqr_rn(dzb))));
+                if (SOFT) r2 = add_fma(r2, eps2, one);
+                fast = exp_fast(d2u(r2));
+            }
+            double y;
+            if (fast) {
+                y = u2d(rsqrt_near(d2u(r2)));
+            } else {
+                y = in ? 1.0 / sqrt(dx * dx + dy * dy + dz * dz + eps2) : 0.0;
+            }
+            acc = fma(in ? b.y : 0.0, y, acc);
+        }
+        q[1] -= G * mi * acc;
+    };
+    if (ONE) {
+        long long b = 0, c = blockIdx.x, at = -1;
+        for (;; c += gridDim.x) {
+            while (b < nt && c >= nc) {
+                c += 4 * (b + 1) - nc;
+                ++b;
+            }
+            if (b >= nt) break;
+            if (b != at) {
+                at = b;
+                take_row(b);
+            }
+            if (c == 4 * b) single();
+            columns(c);
+        }
+    } else {
+        for (long long b = blockIdx.x; b < nt; b += gridDim.x) {
+            take_row(b);
+            single();
+            if (threadIdx.x == 0) blk_hi = 0;
+            __syncthreads();
+            atomicMax((unsigned long long *)&blk_hi, (unsigned long long)hi);
+            __syncthreads();
+            const long long jend = blk_hi;
+            for (long long c = 4 * b; c * EN_C < jend; ++c) columns(c);
+            __syncthreads();
+        }
     }
-    double q[8];
-    q[0] = iv ? 0.5 * mi * (vx * vx + vy * vy + vz * vz) : 0.0;
-    q[1] = V;
-    q[2] = mi * vx; q[3] = mi * vy; q[4] = mi * vz;
-    q[5] = mi * (yi * vz - zi * vy);
-    q[6] = mi * (zi * vx - xi * vz);
-    q[7] = mi * (xi * vy - yi * vx);
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
         double val = q[c];
@@ -919,7 +980,10 @@ void launch_energy(const double *x3, const double *v3, const double *m, long lon
                    const int32_t *sys_off, int nsys, double *partial, int nblk, cudaStream_t s)
 {
     if (n <= 0) return;
-    k_energy<<<nblk, EN_T, 0, s>>>(x3, v3, m, n, G, eps2, sys_off, nsys, partial);
+    const bool one = !(sys_off && nsys > 1), soft = eps2 != 0.0;
+    const auto k = one ? (soft ? k_energy<true, true> : k_energy<true, false>)
+                       : (soft ? k_energy<false, true> : k_energy<false, false>);
+    k<<<nblk, EN_T, 0, s>>>(x3, v3, m, n, G, eps2, 1.0, sys_off, nsys, partial);
     CC_COUNT_LAUNCH(1);
 }
 

@@ -56,6 +56,12 @@ int main(int argc, char **argv)
         if (po) ++opened;
         else if (pv != d2u(pr)) { if (++bad < 9) printf("rinv3 %a\n", px); }
         if (!open && (v != d2u(r))) { if (++bad < 9) printf("rinv3 %a\n", x); }
+        // rsqrt_near: within 0.51 ulp of the 113-bit value where long double has it
+        // (else of the 64-bit one), the last place being the result's
+        const double z = u2d(rsqrt_near(d2u(x)));
+        const long double zl = 1.0L / std::sqrt((long double)x);
+        const long double ulp = std::ldexp(1.0L, std::ilogb(z) - 52);
+        if (!(std::fabs((long double)z - zl) <= 0.51L * ulp)) { if (++bad < 9) printf("rsqrt %a: %Lg ulp\n", x, std::fabs((long double)z - zl) / ulp); }
         if (!exp_fast(d2u(x)) || !fast_range(d2u(a))) { if (++bad < 9) printf("range %a %a\n", x, a); }
     }
     const double out[6] = {1e-300, 5e-324, 1e300, HUGE_VAL, NAN, 1e-62};
