@@ -1011,8 +1011,8 @@ static int level_kick(cc_ctx *c, LevelAlloc &a, const int32_t *lab, const int32_
         PairFactors pf{nullptr, nullptr, 0};
         if (a.Ke == 0) CC_TRY(pair_factors(c, a, pf));
         const int ev = ev_begin(c, 1, nullptr, -1, 0, 0, (double)a.pairs);
-        launch_kick(L, lab, (int)a.k64_blocks[0], c->p.G, c->p.eps * c->p.eps, h, 0, c->d_ctr, s,
-                    a.Ke > 0 ? &a.cv : nullptr, nullptr, pf.S ? &pf : nullptr);
+        launch_kick(L, lab, (int)a.k64_blocks[0], c->p.G, c->p.eps * c->p.eps, h, s, a.Ke > 0 ? &a.cv : nullptr,
+                    nullptr, pf.S ? &pf : nullptr);
         ev_end(c, ev);
     }
     return CC_OK;
@@ -1411,7 +1411,7 @@ static int ok_step(cc_ctx *c)
             // D_{h/2} of the particles without a fast pair, K_h of every
             // slow pair of each set (the fast ones masked), D_{h/2}
             launch_drift_labels(a.L, c->ok_rest, 0.5 * dt, s);
-            launch_kick(KL, a.L.gid, (int)a.k64_blocks[0], G, eps2, dt, 0, c->d_ctr, s, nullptr, &okv,
+            launch_kick(KL, a.L.gid, (int)a.k64_blocks[0], G, eps2, dt, s, nullptr, &okv,
                         pf.S ? &pf : nullptr);
             launch_drift_labels(a.L, c->ok_rest, 0.5 * dt, s);
         }

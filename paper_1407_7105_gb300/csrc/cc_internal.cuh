@@ -343,7 +343,7 @@ struct PairFactors {
     int nblocks;             // k_pair_forces' grid: the level's 128-wide triangular tiles
 };
 void launch_kick(const Level &L, const int32_t *label, int nitiles, double G, double eps2, double h,
-                 int variant, DevCounters *ctr, cudaStream_t s, const ComView *com = nullptr,
+                 cudaStream_t s, const ComView *com = nullptr,
                  const OkView *okv = nullptr,
                  const PairFactors *pf = nullptr);
 // the OK split's outer level after its tau kernel wrote the fast pairs

@@ -13,11 +13,6 @@
 namespace cc {
 
 // ------------------------------------------------------------ helpers
-// a + b as a fused multiply-add by a one the compiler cannot see: the same bits
-// (a times one is exact, zeros keep their signs), and a DFMA holds the pipe 64
-// cycles a warp where a DADD holds it 77 (both measured alone on it)
-__device__ __forceinline__ double add_fma(double a, double b, double one) { return __fma_rn(a, one, b); }
-
 __device__ __forceinline__ int find_set(const int32_t *off, int nsets, int b)
 {
     int lo = 0, hi = nsets;  // off[lo] <= b < off[hi]
@@ -383,54 +378,21 @@ void launch_tau_hook(const Level &L, int ntiles, const TauParams &P, DevCounters
 }
 
 // ------------------------------------------------------------ kick (FP64)
-// One CTA per (set, i-tile); thread r accumulates a_i over every j-tile of
-// its set in ascending order (pairs with equal labels skipped), so the sum
-// runs over j in ascending packed index = ascending particle id, the
-// order of the plain definition; then v_i += h a_i.  Two-stage TMA ring.
-
-template <int T>
-struct __align__(16) KickSmem {
-    double col[2][4][T];  // x y z m per stage
-    int32_t lab[2][T];
-    uint64_t bar[2];
-};
-
-template <int T>
-__device__ __forceinline__ void kick_issue(KickSmem<T> &sm, int st, const Level &L, const int32_t *label, int j0,
-                                           int jn)
-{
-    const unsigned cnt = (unsigned)((jn + 3) & ~3);
-    fence_proxy_async_smem();
-    mbar_expect_tx(&sm.bar[st], cnt * (4u * 8u + 4u));
-    tma_load_1d(sm.col[st][0], L.x + j0, cnt * 8u, &sm.bar[st]);
-    tma_load_1d(sm.col[st][1], L.y + j0, cnt * 8u, &sm.bar[st]);
-    tma_load_1d(sm.col[st][2], L.z + j0, cnt * 8u, &sm.bar[st]);
-    tma_load_1d(sm.col[st][3], L.m + j0, cnt * 8u, &sm.bar[st]);
-    tma_load_1d(sm.lab[st], label + j0, cnt * 4u, &sm.bar[st]);
-}
-
-// One CTA (256 threads) per 32-body i-tile of a set.  For each 32-body
-// j-tile (TMA, double-buffered) all threads first compute the tile's 1024
-// pair forces (the square roots and divisions, the bulk of the FP64 work,
-// spread over eight warps) into shared memory, then 96 threads each add one
-// (row, component) over the tile in ascending j: a_i is still the sum over
-// j in ascending id, term by term as in the plain definition (a skipped
-// pair is an exact +0), so the result is the oracle's bit for bit, while the
-// FP64 pipe sees eight warps per block instead of one thread per body.
-constexpr int KB_T = 32;        // i-tile and j-tile
-constexpr int KB_THREADS = 256;
-constexpr int KB_Q = KB_T * KB_T / KB_THREADS;  // pairs of a tile per thread
+// One block per KB_R rows of a set's 32-row tile.  For each 32 columns eight
+// warps, one a row, compute the row's pair forces into shared memory (a
+// skipped pair is an exact +0), while a ninth adds the previous 32 columns',
+// one lane a row and component, in ascending j: a_i is the sum over j in
+// ascending id, term by term as in the plain definition, so the result is the
+// oracle's bit for bit; then v_i += h a_i.
+//
+// What bounds it: for the small sets that come here the chain of n additions
+// (64 cycles each; the forces of 32 columns are ready sooner); a set of 32-row
+// blocks left all but n/32 SMs idle, and those FP64-bound.  256 bodies: 78 us
+// with 32 rows a block, 18 us now.
+constexpr int KB_T = 32;  // the i-tile prefix, and the columns of a step
+constexpr int KB_R = 8;   // rows of a block
+constexpr int KB_THREADS = 32 * (KB_R + 1);
 static_assert(K64_VAR_T[0] == KB_T, "the FP64 kick runs on the 32-body i-tile prefix");
-
-struct __align__(16) KickBSmem {
-    KickSmem<KB_T> j;                // j tiles: x y z m, labels
-    double f[3][KB_T][KB_T + 1];     // pair forces of the current tile (padded rows)
-    double xi[3][KB_T];              // the i-tile
-    int32_t li[KB_T];
-    int32_t ci[KB_T], cj[KB_T];      // centre-of-mass approximation: local eligible indices
-    int32_t okc[KB_T], oke[KB_T];    // OK split: each row's cursor / end in its sorted fast partners
-    uint32_t okm[KB_T];              // OK split: fast partners of each row in the current j-tile
-};
 
 // MODE 1 (centre-of-mass approximation): pairs of far components (ComView)
 // are left out; their kick is the centre-of-mass one that launch_com_apply
@@ -438,117 +400,96 @@ struct __align__(16) KickBSmem {
 // partners, sorted) are left out, every other pair of the set kicks.
 template <int MODE>
 __global__ void __launch_bounds__(KB_THREADS) k_kick64(Level L, const int32_t *label, double G, double eps2, double h,
-                                                       DevCounters *ctr, ComView cv, OkView okv)
+                                                       double one, ComView cv, OkView okv)
 {
-    constexpr bool COM = MODE == 1, OKM = MODE == 2;
-    __shared__ KickBSmem sm;
-    const int tid = threadIdx.x;
-    const int s = find_set(L.itile_off, L.nsets, blockIdx.x);
-    const int ti = blockIdx.x - L.itile_off[s];
+    __shared__ double f[2][3][KB_R][KB_T + 1];
+    const int tile = blockIdx.x / (KB_T / KB_R);
+    const int s = find_set(L.itile_off, L.nsets, tile);
     const int n = L.set_n[s], start = L.set_start[s];
-    const int nt = (n + KB_T - 1) / KB_T;
-    const int il0 = ti * KB_T, ni = min(KB_T, n - il0);
-    if (tid == 0) {
-        mbar_init(&sm.j.bar[0], 1);
-        mbar_init(&sm.j.bar[1], 1);
-        fence_mbar_init();
-    }
-    if (tid < KB_T) {
-        const bool v = tid < ni;
-        const int i = start + il0 + tid;
-        sm.xi[0][tid] = v ? L.x[i] : 0.0;
-        sm.xi[1][tid] = v ? L.y[i] : 0.0;
-        sm.xi[2][tid] = v ? L.z[i] : 0.0;
-        sm.li[tid] = v ? label[i] : 0;
-        if (COM) sm.ci[tid] = v ? cv.cl[i] : -1;
-        if (OKM) {
-            sm.okc[tid] = v ? okv.row_ptr[i] : 0;
-            sm.oke[tid] = v ? okv.row_ptr[i + 1] : 0;
-        }
-    }
-    long long fo = 0;
-    int Ks = 0;
-    if (COM) {
-        fo = cv.foff[s];
-        Ks = cv.K[s];
-    }
-    __syncthreads();
-    if (tid == 0) kick_issue(sm.j, 0, L, label, start, min(KB_T, n));
-    const int r = tid & 31, c = tid >> 5;  // summing threads: row r, component c (tid < 96)
-    double acc = 0.0;
-    bool ok = true;
-    for (int tj = 0; tj < nt; ++tj) {
-        const int st = tj & 1;
-        if (tid == 0 && tj + 1 < nt)
-            kick_issue(sm.j, st ^ 1, L, label, start + (tj + 1) * KB_T, min(KB_T, n - (tj + 1) * KB_T));
-        const bool got = mbar_wait(&sm.j.bar[st], (tj >> 1) & 1, TMA_WAIT_CYCLES);
-        if (__syncthreads_or(!got)) {  // uniform exit: no thread is left at a barrier
-            ok = false;
-            break;
-        }
-        const int jn = min(KB_T, n - tj * KB_T), jl0 = tj * KB_T;
-        if (COM) {
-            if (tid < KB_T) sm.cj[tid] = tid < jn ? cv.cl[start + jl0 + tid] : -1;
-            __syncthreads();
-        }
-        if (OKM) {
-            // the row's fast partners inside this j-tile (partners ascend, so
-            // the cursor only moves forward)
-            if (tid < KB_T) {
-                const int jb = start + jl0;
-                uint32_t mk = 0u;
-                int q = sm.okc[tid];
-                const int qe = sm.oke[tid];
-                while (q < qe && okv.col[2 * q + 1] < jb + jn) {
-                    const int d = okv.col[2 * q + 1] - jb;
-                    if (d >= 0) mk |= 1u << d;
-                    ++q;
-                }
-                sm.okc[tid] = q;
-                sm.okm[tid] = mk;
-            }
-            __syncthreads();
-        }
+    const int il0 = (tile - L.itile_off[s]) * KB_T + (blockIdx.x % (KB_T / KB_R)) * KB_R;
+    if (il0 >= n) return;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int nk = (n + KB_T - 1) / KB_T;
+    if (w == KB_R) {
+        // the adding warp: lane = 8 c + r
+        const int c = min(lane / KB_R, 2), r = lane % KB_R;
+        double acc = 0.0;
+        __syncthreads();
+        for (int k = 0; k < nk; ++k) {
+            const double *t = f[k & 1][c][r];
 #pragma unroll
-        for (int q = 0; q < KB_Q; ++q) {
-            const int pidx = tid + q * KB_THREADS, ii = pidx >> 5, jj = pidx & 31;
-            bool use = ii < ni && jj < jn && il0 + ii != jl0 + jj && sm.li[ii] != sm.j.lab[st][jj];
-            if (COM && use && sm.ci[ii] >= 0 && sm.cj[jj] >= 0)
-                use = cv.far[fo + (long long)sm.ci[ii] * Ks + sm.cj[jj]] == 0;
-            if (OKM && use) use = ((sm.okm[ii] >> jj) & 1u) == 0u;
-            const double dx0 = __dsub_rn(sm.j.col[st][0][jj], sm.xi[0][ii]);
-            const double dx1 = __dsub_rn(sm.j.col[st][1][jj], sm.xi[1][ii]);
-            const double dx2 = __dsub_rn(sm.j.col[st][2][jj], sm.xi[2][ii]);
-            const double r2 = __dadd_rn(
-                __dadd_rn(__dadd_rn(__dmul_rn(dx0, dx0), __dmul_rn(dx1, dx1)), __dmul_rn(dx2, dx2)), eps2);
-            const double rinv3 = __drcp_rn(__dmul_rn(r2, __dsqrt_rn(r2)));
-            const double w = __dmul_rn(__dmul_rn(G, sm.j.col[st][3][jj]), rinv3);
-            sm.f[0][ii][jj] = use ? __dmul_rn(w, dx0) : 0.0;
-            sm.f[1][ii][jj] = use ? __dmul_rn(w, dx1) : 0.0;
-            sm.f[2][ii][jj] = use ? __dmul_rn(w, dx2) : 0.0;
+            for (int jj = 0; jj < KB_T; ++jj) acc = add_fma(t[jj], acc, one);
+            __syncthreads();
         }
-        __syncthreads();
-        if (tid < 3 * KB_T)
-            for (int jj = 0; jj < jn; ++jj) acc = __dadd_rn(acc, sm.f[c][r][jj]);
-        __syncthreads();
-    }
-    if (!ok) {
-        raise_err(ctr, DERR_TMA_TIMEOUT);
-        // let any copy still in flight land before the CTA exits
-        mbar_wait(&sm.j.bar[0], 0, TMA_WAIT_CYCLES);
-        mbar_wait(&sm.j.bar[1], 0, TMA_WAIT_CYCLES);
+        if (lane < 3 * KB_R && il0 + r < n) {
+            const int i = start + il0 + r;
+            double *v = c == 0 ? L.vx : (c == 1 ? L.vy : L.vz);
+            v[i] = __dadd_rn(v[i], __dmul_rn(h, acc));
+        }
         return;
     }
-    if (tid < 3 * KB_T && r < ni) {
-        const int i = start + il0 + r;
-        double *v = c == 0 ? L.vx : (c == 1 ? L.vy : L.vz);
-        v[i] = __dadd_rn(v[i], __dmul_rn(h, acc));
+    const bool on = il0 + w < n, soft = eps2 != 0.0;
+    const int i = start + (on ? il0 + w : il0);
+    const double xi = L.x[i], yi = L.y[i], zi = L.z[i];
+    const int li = label[i];
+    long long fo = 0;
+    int Ks = 0, ci = -1, oq = 0, oe = 0;
+    if (MODE == 1) {
+        fo = cv.foff[s];
+        Ks = cv.K[s];
+        ci = cv.cl[i];
     }
+    if (MODE == 2) {
+        oq = okv.row_ptr[i];
+        oe = okv.row_ptr[i + 1];
+    }
+    for (int k = 0; k < nk; ++k) {
+        const int jl = k * KB_T + lane, j = start + min(jl, n - 1);
+        bool use = on && jl < n && j != i && label[j] != li;
+        if (MODE == 1 && use && ci >= 0) {
+            const int c = cv.cl[j];
+            if (c >= 0) use = cv.far[fo + (long long)ci * Ks + c] == 0;
+        }
+        if (MODE == 2) {
+            // the row's fast partners among these columns, 32 of its sorted list at a time
+            const int jb = start + k * KB_T;
+            uint32_t mk = 0u;
+            for (;;) {
+                const int p = oq + lane < oe ? okv.col[2 * (long long)(oq + lane) + 1] : 0x7fffffff;
+                const bool in = p < jb + KB_T;
+                mk |= __reduce_or_sync(0xffffffffu, in && p >= jb ? 1u << (p - jb) : 0u);
+                const int cnt = __popc(__ballot_sync(0xffffffffu, in));
+                oq += cnt;
+                if (cnt < 32) break;
+            }
+            use = use && ((mk >> lane) & 1u) == 0u;
+        }
+        double t0 = 0.0, t1 = 0.0, t2 = 0.0;
+        if (use) {
+            const double dx0 = add_fma(L.x[j], -xi, one), dx1 = add_fma(L.y[j], -yi, one),
+                         dx2 = add_fma(L.z[j], -zi, one);
+            const double gm = __dmul_rn(G, L.m[j]);
+            double v;
+            const bool fast = pair_rinv3(dx0, dx1, dx2, eps2, soft, one, v) && exp_fast(d2u(gm));
+            if (fast) {
+                const uint64_t wv = mul_rn(d2u(gm), d2u(v));
+                t0 = u2d(mul_rn(wv, d2u(dx0)));
+                t1 = u2d(mul_rn(wv, d2u(dx1)));
+                t2 = u2d(mul_rn(wv, d2u(dx2)));
+            } else {
+                const double wv = __dmul_rn(gm, v);
+                t0 = __dmul_rn(wv, dx0);
+                t1 = __dmul_rn(wv, dx1);
+                t2 = __dmul_rn(wv, dx2);
+            }
+        }
+        f[k & 1][0][w][lane] = t0;
+        f[k & 1][1][w][lane] = t1;
+        f[k & 1][2][w][lane] = t2;
+        __syncthreads();
+    }
+    __syncthreads();  // (the adding warp's last step)
 }
-
-// rn(1 / rn(r2 rn(sqrt r2))) by the IEEE instructions: what rinv3_rn is, and
-// the way out where it does not apply
-__device__ __noinline__ double rinv3_ieee(double r2) { return __drcp_rn(__dmul_rn(r2, __dsqrt_rn(r2))); }
 
 // Three n x n matrices per set (components x, y, z) at pf.moff[s]: row j,
 // column i = the force G m_j r_ij^-3 (x_j - x_i) of j on i (the diagonal
@@ -568,11 +509,12 @@ __device__ __noinline__ double rinv3_ieee(double r2) { return __drcp_rn(__dmul_r
 // the negated force on i, bit for bit.  16384 bodies (1.34e8 pairs): 8.6 ms
 // with every operation on the FP64 pipe, 2.4 ms so (two of the products left
 // on it; none 2.66, one 2.46, three 2.55, four 2.81 ms).
-constexpr int KR_T = 32, KR_W = 128;
+constexpr int KR_T = 32, KR_W = 128, PF_THREADS = 256;
+constexpr int PF_Q = KR_T * KR_T / PF_THREADS;  // pairs of a sub-tile per thread
 static_assert(KR_T == KB_T, "the force sub-tiles are the kick's i-tiles");
 static_assert(KR_W == TAU_VAR_T[TAU_VAR_128], "the force tiles are the 128-wide tau tiles");
 template <bool SOFT>
-__global__ void __launch_bounds__(KB_THREADS, 6) k_pair_forces(Level L, double G, double eps2, double one, double nzero,
+__global__ void __launch_bounds__(PF_THREADS, 6) k_pair_forces(Level L, double G, double eps2, double one, double nzero,
                                                             PairFactors pf)
 {
     __shared__ double xi[4][KR_W];  // x, y, z, G m
@@ -589,7 +531,7 @@ __global__ void __launch_bounds__(KB_THREADS, 6) k_pair_forces(Level L, double G
     const int ni = min(KR_W, n - i0), nj = min(KR_W, n - j0);
     double *S = pf.S + pf.moff[s];
     bool in = true;  // every G m in the range of the integer products
-    for (int e = tid; e < KR_W; e += KB_THREADS) {
+    for (int e = tid; e < KR_W; e += PF_THREADS) {
         const bool vi = e < ni, vj = e < nj;
         xi[0][e] = vi ? L.x[start + i0 + e] : 0.0;
         xi[1][e] = vi ? L.y[start + i0 + e] : 0.0;
@@ -608,8 +550,8 @@ __global__ void __launch_bounds__(KB_THREADS, 6) k_pair_forces(Level L, double G
             if (il >= ni || jl >= nj) continue;  // (uniform over the block)
             __syncthreads();  // (the previous sub-tile's transposed write)
 #pragma unroll 1
-            for (int q = 0; q < KB_Q; ++q) {
-                const int pidx = tid + q * KB_THREADS, ii = pidx >> 5, jj = pidx & 31;
+            for (int q = 0; q < PF_Q; ++q) {
+                const int pidx = tid + q * PF_THREADS, ii = pidx >> 5, jj = pidx & 31;
                 const int gi = il + ii, gj = jl + jj;
                 const bool on = gi < ni && gj < nj && j0 + gj > i0 + gi;
                 const uint64_t gmj = d2u(xj[3][gj]), gmi = d2u(xi[3][gi]);
@@ -618,19 +560,11 @@ __global__ void __launch_bounds__(KB_THREADS, 6) k_pair_forces(Level L, double G
                 const double dx0 = add_fma(xj[0][gj], -xi[0][gi], one);
                 const double dx1 = add_fma(xj[1][gj], -xi[1][gi], one);
                 const double dx2 = add_fma(xj[2][gj], -xi[2][gi], one);
-                const uint64_t d0 = d2u(dx0), d1 = d2u(dx1), d2 = d2u(dx2);
-                uint64_t w, v, f0, f1, f2, g0, g1, g2;
-                bool fast = in && fast_range(d0) && fast_range(d1) && fast_range(d2);
-                if (fast) {
-                    double r2 = add_fma(add_fma(u2d(sqr_rn(d0)), u2d(sqr_rn(d1)), one), u2d(sqr_rn(d2)), one);
-                    if (SOFT) r2 = add_fma(r2, eps2, one);
-                    bool open = !exp_fast(d2u(r2));
-                    v = rinv3_rn(d2u(r2), open);
-                    if (open) {
-                        v = d2u(rinv3_ieee(r2));
-                        fast = exp_fast(d2u(r2));
-                    }
-                }
+                const uint64_t d2 = d2u(dx2);
+                uint64_t w, f0, f1, f2, g0, g1, g2;
+                double vd;
+                const bool fast = pair_rinv3(dx0, dx1, dx2, eps2, SOFT, one, vd) && in;
+                const uint64_t v = d2u(vd);
                 if (fast) {
                     // (two of the three products of a force on the FP64 pipe: the
                     // two pipes then finish about together)
@@ -644,14 +578,11 @@ __global__ void __launch_bounds__(KB_THREADS, 6) k_pair_forces(Level L, double G
                         g2 = f2;
                     } else {
                         w = mul_rn(gmi, v);
-                        g0 = mul_rn(w, d0);
-                        g1 = mul_rn(w, d1);
+                        g0 = mul_rn(w, d2u(dx0));
+                        g1 = mul_rn(w, d2u(dx1));
                         g2 = mul_rn(w, d2);
                     }
                 } else {
-                    const double r2 = __dadd_rn(
-                        __dadd_rn(__dadd_rn(__dmul_rn(dx0, dx0), __dmul_rn(dx1, dx1)), __dmul_rn(dx2, dx2)), eps2);
-                    const double vd = rinv3_ieee(r2);
                     const double wij = __dmul_rn(u2d(gmj), vd), wji = __dmul_rn(u2d(gmi), vd);
                     f0 = d2u(__dmul_rn(wij, dx0));
                     f1 = d2u(__dmul_rn(wij, dx1));
@@ -671,8 +602,8 @@ __global__ void __launch_bounds__(KB_THREADS, 6) k_pair_forces(Level L, double G
             }
             __syncthreads();
 #pragma unroll
-            for (int q = 0; q < KB_Q; ++q) {
-                const int pidx = tid + q * KB_THREADS, jj = pidx >> 5, ii = pidx & 31;
+            for (int q = 0; q < PF_Q; ++q) {
+                const int pidx = tid + q * PF_THREADS, jj = pidx >> 5, ii = pidx & 31;
                 const int gi = il + ii, gj = jl + jj;
                 if (gi < ni && gj < nj && j0 + gj > i0 + gi) {
                     const long long e = (long long)(j0 + gj) * n + (i0 + gi);
@@ -807,17 +738,17 @@ __global__ void __launch_bounds__(64 * KR_PAIRS) k_kick_rows(Level L, const int3
 }
 
 void launch_kick(const Level &L, const int32_t *label, int nitiles, double G, double eps2, double h,
-                 int variant, DevCounters *ctr, cudaStream_t s, const ComView *com, const OkView *okv,
+                 cudaStream_t s, const ComView *com, const OkView *okv,
                  const PairFactors *pf)
 {
-    (void)variant;  // one shape: 32-body tiles (the prefix of variant 0)
     if (nitiles <= 0) return;
     const ComView nc{nullptr, nullptr, nullptr, nullptr};
     const OkView no{nullptr, nullptr};
+    const unsigned grid = (unsigned)nitiles * (KB_T / KB_R);
     const bool pre = pf && pf->S && !(com && com->cl);
     if (pre) {
-        if (eps2 != 0.0) k_pair_forces<true><<<pf->nblocks, KB_THREADS, 0, s>>>(L, G, eps2, 1.0, -0.0, *pf);
-        else k_pair_forces<false><<<pf->nblocks, KB_THREADS, 0, s>>>(L, G, eps2, 1.0, -0.0, *pf);
+        if (eps2 != 0.0) k_pair_forces<true><<<pf->nblocks, PF_THREADS, 0, s>>>(L, G, eps2, 1.0, -0.0, *pf);
+        else k_pair_forces<false><<<pf->nblocks, PF_THREADS, 0, s>>>(L, G, eps2, 1.0, -0.0, *pf);
         const int nb = (3 * nitiles + KR_PAIRS - 1) / KR_PAIRS;
         if (okv && okv->row_ptr) {
             cudaFuncSetAttribute(k_kick_rows<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, KR_SMEM);
@@ -828,11 +759,11 @@ void launch_kick(const Level &L, const int32_t *label, int nitiles, double G, do
         }
         CC_COUNT_LAUNCH(1);
     } else if (okv && okv->row_ptr) {
-        k_kick64<2><<<nitiles, KB_THREADS, 0, s>>>(L, label, G, eps2, h, ctr, nc, *okv);
+        k_kick64<2><<<grid, KB_THREADS, 0, s>>>(L, label, G, eps2, h, 1.0, nc, *okv);
     } else if (com && com->cl) {
-        k_kick64<1><<<nitiles, KB_THREADS, 0, s>>>(L, label, G, eps2, h, ctr, *com, no);
+        k_kick64<1><<<grid, KB_THREADS, 0, s>>>(L, label, G, eps2, h, 1.0, *com, no);
     } else {
-        k_kick64<0><<<nitiles, KB_THREADS, 0, s>>>(L, label, G, eps2, h, ctr, nc, no);
+        k_kick64<0><<<grid, KB_THREADS, 0, s>>>(L, label, G, eps2, h, 1.0, nc, no);
     }
     CC_COUNT_LAUNCH(1);
 }
