@@ -241,6 +241,27 @@ CC_HD uint64_t rsqrt_near(uint64_t x)
     return Z - ((uint64_t)(int64_t)((E - (int32_t)p) >> 1) << 52);
 }
 
+// x / C for a small whole constant, the division's bits in three operations:
+// quotient by the rounded reciprocal, exact residual, correction (Markstein's
+// theorem for a correctly rounded reciprocal; C's significand is not all ones)
+// Explicit operations: what the compiler contracts around them stays as it is.
+CC_HD double div_const(double x, double c)
+{
+#ifdef __CUDA_ARCH__
+    const double y = 1.0 / c, q = __dmul_rn(x, y);
+#else
+    const double y = 1.0 / c, q = x * y;
+#endif
+    return fma_d(fma_d(-q, c, x), y, q);
+}
+template <int C>
+CC_HD float div_const_f(float x)
+{
+    constexpr float y = 1.0f / C;
+    const float q = x * y;
+    return fma_f(fma_f(-q, (float)C, x), y, q);
+}
+
 #ifdef __CUDACC__
 // a + b and a b as fused multiply-adds with a one and a minus zero that the
 // compiler cannot see: the same bits (a times one is exact, a sum with -0

@@ -18,6 +18,21 @@ SRC = r'''
 namespace cc { float est_shift = 0.0f; }
 using namespace cc;
 static std::mt19937_64 g(7);
+template <int C> static long divs(float x)
+{
+    volatile float c = C, q = x / c;
+    return f2u(div_const_f<C>(x)) != f2u(q);
+}
+static long divs64(double x)
+{
+    long bad = 0;
+    for (int k = 0; k < 10; ++k) {
+        volatile double a = (2.0 * k + 3.0) * (2.0 * k + 4.0), b = (2.0 * k + 4.0) * (2.0 * k + 5.0);
+        volatile double p = x / a, q = x / b;
+        bad += (d2u(div_const(x, a)) != d2u(p)) + (d2u(div_const(x, b)) != d2u(q));
+    }
+    return bad;
+}
 static double draw(int emin, int emax)
 {
     uint64_t m = g() & 0xfffffffffffffull;
@@ -56,6 +71,11 @@ int main(int argc, char **argv)
         if (po) ++opened;
         else if (pv != d2u(pr)) { if (++bad < 9) printf("rinv3 %a\n", px); }
         if (!open && (v != d2u(r))) { if (++bad < 9) printf("rinv3 %a\n", x); }
+        // the Stumpff series' divisions
+        const float y = (float)draw(-60, 6);
+        const long dv = divs<12>(y) + divs<20>(y) + divs<30>(y) + divs<42>(y) + divs<56>(y) + divs<72>(y) + divs<90>(y) +
+                        divs<110>(y) + divs<132>(y) + divs<156>(y) + divs64(draw(-200, 6));
+        if (dv) { bad += dv; if (bad < 9) printf("div %a\n", y); }
         // rsqrt_near: within 0.51 ulp of the 113-bit value where long double has it
         // (else of the 64-bit one), the last place being the result's
         const double z = u2d(rsqrt_near(d2u(x)));
