@@ -998,8 +998,8 @@ static int level_kick(cc_ctx *c, LevelAlloc &a, const int32_t *lab, const int32_
         CC_TRY(ensure_kpart(c, a.mk_chunks_max[var], a.F.cap));
         const int ev = ev_begin(c, 1, nullptr, timed ? TK_MK : -1, bin, var, (double)a.pairs);
         launch_kick_mixed(L, a.F, order, a.mk_off[var], (int)a.mk_blocks[var], MK_VAR_CHUNK[var], MK_VAR_SLICE[var],
-                          a.mk_chunks_max[var] > 1, c->p.eps * c->p.eps, h, c->d_ctr, c->d_kpart, lab, drift_dt, s,
-                          a.Ke > 0 ? &a.cv : nullptr);
+                          a.mk_chunks_max[var] > 1, c->p.eps * c->p.eps, h, c->d_ctr, c->d_kpart, lab, drift_dt,
+                          a.pairs >= MK_PACKED_MIN, s, a.Ke > 0 ? &a.cv : nullptr);
         ev_end(c, ev);
     } else {
         // FP64: one shape (32-body i-tiles; the row order fixes the rounding).
@@ -1028,7 +1028,7 @@ static int dkd(cc_ctx *c, LevelAlloc &a, double h)
         // positions in the root-sorted order of the split (members of one
         // component adjacent: tiles inside one component are skipped); both
         // drifts ride on the copy and on the partial reduce
-        launch_prep_kick(a.L, a.F, a.members, a.root, c->p.G, 0.5 * h, s);
+        launch_prep_kick(a.L, a.F, a.members, a.root, c->p.G, 0.5 * h, a.pairs >= MK_PACKED_MIN, s);
         CC_TRY(level_kick(c, a, a.root, a.members, h, 0.5 * h));
         // the FP32 kick left the far pairs out: the monopole kick instead
         if (a.Ke > 0)
@@ -1917,7 +1917,7 @@ int cc_kick(cc_ctx *c, const int32_t *set, int64_t n_set, const int32_t *labels,
     if (c->p.precision == CC_PREC_MIXED && !(h < c->p.h_fp64)) {
         // the mixed kick works in label-sorted order (members of a group adjacent)
         launch_label_order(dl, (int)n_set, u.L.total, order, c->seg_scratch, c->stream);
-        launch_prep_kick(u.L, u.F, order, dl, c->p.G, 0.0, c->stream);
+        launch_prep_kick(u.L, u.F, order, dl, c->p.G, 0.0, u.pairs >= MK_PACKED_MIN, c->stream);
     }
     CC_TRY(level_kick(c, u, dl, order, h));
     CC_CUDA(c, cudaStreamSynchronize(c->stream));

@@ -303,6 +303,8 @@ static_assert(TAU_VAR_T[TAU_VAR_128] == 128, "128-wide tau tiles");
 constexpr int K64_VAR_T[N_K64_VAR] = {32, 64, 128};
 constexpr int MK_VAR_CHUNK[N_MK_VAR] = {1, 4, 1};
 constexpr int MK_VAR_SLICE[N_MK_VAR] = {1, 1, 4};
+// pairs of a level from which its mixed kick is the packed one (cc_mixed.cu)
+constexpr long long MK_PACKED_MIN = 1ll << 29;
 constexpr int MK_TILE = 128;
 void launch_tau_hook(const Level &L, int ntiles, const TauParams &P, DevCounters *ctr,
                      int32_t *edges, long long edge_cap, int32_t *near_ij, double *near_tau, long long near_cap,
@@ -484,10 +486,10 @@ int mixed_kick_chunks(int n, int chunk);
 // root) fused in: before the positions are copied (prep), after the kick
 // (the partial reduce, launched for it even without multi-chunk sets)
 void launch_prep_kick(const Level &L, const FFView &F, const int32_t *order, const int32_t *root, double G,
-                      double drift_dt, cudaStream_t s);
+                      double drift_dt, bool packed, cudaStream_t s);
 void launch_kick_mixed(const Level &L, const FFView &F, const int32_t *order, const int32_t *koff, int nblocks,
                        int chunk, int slices, bool multi_chunk, double eps2, double h, DevCounters *ctr,
-                       double *partial, const int32_t *root, double drift_dt, cudaStream_t s,
+                       double *partial, const int32_t *root, double drift_dt, bool packed, cudaStream_t s,
                        const ComView *com = nullptr);
 
 // cc_small.cu

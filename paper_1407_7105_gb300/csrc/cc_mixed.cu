@@ -114,7 +114,7 @@ void launch_prep_ff(const Level &L, const FFView &F, double G, bool with_v, cuda
     CC_COUNT_LAUNCH(1);
 }
 
-// The kick's copy, in F.pq's place: two bodies together, four float4 a pair
+// The packed kick's copy, in F.pq's place: two bodies together, four float4 a pair
 //   (x x' y y') (z z' Gm Gm') (xlo xlo' ylo ylo') (zlo zlo' - -)
 // so that the pair loop's packed operands come straight from a 16-byte load.
 __device__ __forceinline__ float *kick_slot(const FFView &F, int t)
@@ -126,7 +126,8 @@ __device__ __forceinline__ float *kick_slot(const FFView &F, int t)
 // split: position t holds packed element order[t].  dt > 0: the level's
 // first drift D_{h/2,T_R} of rest-set members (component size 1, Eq. drift,
 // exact IEEE operations) is applied first, in the same pass.
-__global__ void k_prep_kick(Level L, FFView F, const int32_t *order, const int32_t *root, float G, double dt)
+__global__ void k_prep_kick(Level L, FFView F, const int32_t *order, const int32_t *root, float G, double dt,
+                            int packed)
 {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= L.total) return;
@@ -144,21 +145,27 @@ __global__ void k_prep_kick(Level L, FFView F, const int32_t *order, const int32
     float hi[3], lo[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) ff_split(xs[c], hi[c], lo[c]);
-    float *q = kick_slot(F, t);
+    const float gm = G * fl32(L.m[k]);
+    if (!packed) {
+        F.pq[2 * t] = make_float4(hi[0], hi[1], hi[2], gm);
+        F.pq[2 * t + 1] = make_float4(lo[0], lo[1], lo[2], 0.f);
+    } else {
+        float *q = kick_slot(F, t);
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        q[2 * c] = hi[c];
-        q[8 + 2 * c] = lo[c];
+        for (int c = 0; c < 3; ++c) {
+            q[2 * c] = hi[c];
+            q[8 + 2 * c] = lo[c];
+        }
+        q[6] = gm;
     }
-    q[6] = G * fl32(L.m[k]);
     L.klab[t] = root[k];
 }
 
 void launch_prep_kick(const Level &L, const FFView &F, const int32_t *order, const int32_t *root, double G,
-                      double drift_dt, cudaStream_t s)
+                      double drift_dt, bool packed, cudaStream_t s)
 {
     if (L.total <= 0) return;
-    k_prep_kick<<<(L.total + 255) / 256, 256, 0, s>>>(L, F, order, root, (float)G, drift_dt);
+    k_prep_kick<<<(L.total + 255) / 256, 256, 0, s>>>(L, F, order, root, (float)G, drift_dt, packed ? 1 : 0);
     CC_COUNT_LAUNCH(1);
 }
 
@@ -772,8 +779,17 @@ void launch_tau_raw(const double *m, const double *x3, const double *v3, int n, 
 // columns at a time in packed FP32 (one issue slot for both) take ~17 issue
 // slots a pair where one column at a time took ~27.  Each term and the order
 // of the sums are as they were, so are the bits.  65536-body fractal, top
-// level (4.3e9 directed pairs): 3.77 -> 3.05 ms; 16384-body Plummer, top level:
-// 125 -> 103 us.
+// level (4.3e9 directed pairs): 3.77 -> 3.05 ms.
+// PACKED = false is the same operations a column at a time, for levels below
+// MK_PACKED_MIN pairs.  A column rounds alike in both, but the launch shapes do
+// not sum alike (a chunk is a partial sum), the tuner chooses between them by
+// their times, and packed arithmetic favours the long chunk by 5 to 10 %.  From
+// 2^29 pairs on chunk 4 wins by 6 to 17 % either way (chunk 4 against 1, a
+// column at a time 0.83-0.94, packed 0.79-0.93).  Below, the two lie within a few
+// per cent (32768 bodies, 2^24-pair levels: 1.03-1.06, packed 0.94-1.01), and a
+// different choice would move the last bits of a kick, which a hard binary
+// magnifies by 1e4 and more before the step is over (1.5e-8 of the velocities).
+// There the packed form would save ~20 us of a 2.8 ms step (16384 bodies).
 constexpr int MK_T = 128;
 constexpr int MK_CHUNK_MAX = 4;  // j-tiles per chunk (tuned per size bin)
 static_assert(MK_VAR_CHUNK[0] <= MK_CHUNK_MAX && MK_VAR_CHUNK[1] <= MK_CHUNK_MAX && MK_VAR_CHUNK[2] <= MK_CHUNK_MAX,
@@ -790,13 +806,14 @@ struct __align__(16) MixedKickSmem {
     uint64_t bar[2];
 };
 
+template <bool PACKED>
 __device__ __forceinline__ void mk_issue(MixedKickSmem &sm, int st, const FFView &F, const int32_t *label,
                                          int j0, int jn)
 {
     const unsigned cnt = (unsigned)((jn + 3) & ~3);
     fence_proxy_async_smem();
-    // (an odd last body brings its neighbour's slot along: not added)
-    const unsigned bytes = (unsigned)((jn + 1) / 2) * 64u;
+    // (packed, an odd last body brings its neighbour's slot along: not added)
+    const unsigned bytes = PACKED ? (unsigned)((jn + 1) / 2) * 64u : (unsigned)jn * 32u;
     mbar_expect_tx(&sm.bar[st], bytes + cnt * 4u);
     tma_load_1d(sm.pq[st], F.pq + 2 * (size_t)j0, bytes, &sm.bar[st]);
     tma_load_1d(sm.lab[st], label + j0, cnt * 4u, &sm.bar[st]);
@@ -806,7 +823,7 @@ __device__ __forceinline__ void mk_issue(MixedKickSmem &sm, int st, const FFView
 // each j-tile); the S partial sums of a row are combined in slice order.
 // COM: pairs of two far components (ComView, the centre-of-mass
 // approximation) are left out, as in the FP64 kick.
-template <int S, bool COM>
+template <int S, bool COM, bool PACKED>
 __global__ void __launch_bounds__(MK_T) k_kick_mixed(Level L, FFView F, const int32_t *order, const int32_t *koff,
                                                       int chunk, float eps2, double h, DevCounters *ctr,
                                                       double *partial, ComView cv)
@@ -851,15 +868,21 @@ __global__ void __launch_bounds__(MK_T) k_kick_mixed(Level L, FFView F, const in
     }
     __syncthreads();
     const int nt = sm.ntiles;
-    if (tid == 0 && nt > 0) mk_issue(sm, 0, F, label, start + sm.tiles[0] * MK_T, min(MK_T, n - sm.tiles[0] * MK_T));
+    if (tid == 0 && nt > 0) mk_issue<PACKED>(sm, 0, F, label, start + sm.tiles[0] * MK_T, min(MK_T, n - sm.tiles[0] * MK_T));
     uint64_t nh[3] = {0, 0, 0}, nl[3] = {0, 0, 0};  // minus the row's position, twice each
+    float4 ip0 = make_float4(0, 0, 0, 0), ip1 = ip0;  // the row's position, a column at a time
     int li = 0, ci = -1;
     if (iv) {
-        const float *q = kick_slot(F, t);
+        if constexpr (PACKED) {
+            const float *q = kick_slot(F, t);
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            nh[c] = pack2(-q[2 * c], -q[2 * c]);
-            nl[c] = pack2(-q[8 + 2 * c], -q[8 + 2 * c]);
+            for (int c = 0; c < 3; ++c) {
+                nh[c] = pack2(-q[2 * c], -q[2 * c]);
+                nl[c] = pack2(-q[8 + 2 * c], -q[8 + 2 * c]);
+            }
+        } else {
+            ip0 = F.pq[2 * t];
+            ip1 = F.pq[2 * t + 1];
         }
         li = label[t];
         if constexpr (COM) ci = cv.cl[order[t]];
@@ -878,7 +901,7 @@ __global__ void __launch_bounds__(MK_T) k_kick_mixed(Level L, FFView F, const in
         const int tj = sm.tiles[q], st = q & 1;
         if (tid == 0 && q + 1 < nt) {
             const int tn = sm.tiles[q + 1];
-            mk_issue(sm, st ^ 1, F, label, start + tn * MK_T, min(MK_T, n - tn * MK_T));
+            mk_issue<PACKED>(sm, st ^ 1, F, label, start + tn * MK_T, min(MK_T, n - tn * MK_T));
         }
         const bool got = mbar_wait(&sm.bar[st], (q >> 1) & 1, TMA_WAIT_CYCLES);
         if (__syncthreads_or(!got)) {
@@ -903,7 +926,7 @@ __global__ void __launch_bounds__(MK_T) k_kick_mixed(Level L, FFView F, const in
             // after the other (two: whether the second exists)
             const ulonglong2 *J = reinterpret_cast<const ulonglong2 *>(sm.pq[st]);
             const uint64_t e2 = pack2(eps2, eps2), mh = pack2(-0.5f, -0.5f), c15 = pack2(1.5f, 1.5f);
-            auto term = [&](int k, bool check, bool two) {
+            auto pair = [&](int k, bool check, bool two) {
                 const ulonglong2 a = J[2 * k], b = J[2 * k + 1], c = J[2 * k + 2];
                 const uint64_t lz = J[2 * k + 3].x;
                 const uint64_t dx = add2(add2(a.x, nh[0]), add2(c.x, nl[0]));
@@ -938,6 +961,25 @@ __global__ void __launch_bounds__(MK_T) k_kick_mixed(Level L, FFView F, const in
                     gz = fmaf(wb, zb, gz);
                 }
             };
+            // one column
+            auto term = [&](int k, bool check) {
+                const float4 jp0 = sm.pq[st][2 * k], jp1 = sm.pq[st][2 * k + 1];
+                const float dx = (jp0.x - ip0.x) + (jp1.x - ip1.x);
+                const float dy = (jp0.y - ip0.y) + (jp1.y - ip1.y);
+                const float dz = (jp0.z - ip0.z) + (jp1.z - ip1.z);
+                const float r2 = fmaf(dz, dz, fmaf(dy, dy, fmaf(dx, dx, eps2)));
+                float ri = rsqrtf(r2);
+                ri = ri * fmaf(-0.5f * r2, ri * ri, 1.5f);  // one Newton step
+                float w = jp0.w * (ri * ri * ri);            // G m_j / r^3
+                if (check && sm.lab[st][k] == li) w = 0.f;  // same component (and self)
+                if constexpr (COM) {
+                    const int c = sm.cj[k];
+                    if (fchk && ci >= 0 && c >= 0 && cv.far[fo + (long long)ci * Ks + c]) w = 0.f;
+                }
+                gx = fmaf(w, dx, gx);
+                gy = fmaf(w, dy, gy);
+                gz = fmaf(w, dz, gz);
+            };
             auto flush = [&]() {
                 kahan_add(sx, cx, gx);
                 kahan_add(sy, cy, gy);
@@ -949,12 +991,18 @@ __global__ void __launch_bounds__(MK_T) k_kick_mixed(Level L, FFView F, const in
                 for (; k + MK_GROUP <= k1; k += MK_GROUP) {
                     gx = gy = gz = 0.f;
 #pragma unroll
-                    for (int u = 0; u < MK_GROUP; u += 2) term(k + u, check, true);
+                    for (int u = 0; u < MK_GROUP; u += PACKED ? 2 : 1) {
+                        if constexpr (PACKED) pair(k + u, check, true);
+                        else term(k + u, check);
+                    }
                     flush();
                 }
                 if (k < k1) {
                     gx = gy = gz = 0.f;
-                    for (; k < k1; k += 2) term(k, check, k + 1 < k1);
+                    for (; k < k1; k += PACKED ? 2 : 1) {
+                        if constexpr (PACKED) pair(k, check, k + 1 < k1);
+                        else term(k, check);
+                    }
                     flush();
                 }
             };
@@ -1061,22 +1109,17 @@ int mixed_kick_chunks(int n, int chunk)
 
 void launch_kick_mixed(const Level &L, const FFView &F, const int32_t *order, const int32_t *koff, int nblocks,
                        int chunk, int slices, bool multi_chunk, double eps2, double h, DevCounters *ctr,
-                       double *partial, const int32_t *root, double drift_dt, cudaStream_t s, const ComView *com)
+                       double *partial, const int32_t *root, double drift_dt, bool packed, cudaStream_t s, const ComView *com)
 {
     if (nblocks > 0) {
         const ComView cv = com ? *com : ComView{nullptr, nullptr, nullptr, nullptr};
         const float e2 = (float)eps2;
-        if (com) {
-            if (slices == 4)
-                k_kick_mixed<4, true><<<nblocks, MK_T, 0, s>>>(L, F, order, koff, chunk, e2, h, ctr, partial, cv);
-            else
-                k_kick_mixed<1, true><<<nblocks, MK_T, 0, s>>>(L, F, order, koff, chunk, e2, h, ctr, partial, cv);
-        } else {
-            if (slices == 4)
-                k_kick_mixed<4, false><<<nblocks, MK_T, 0, s>>>(L, F, order, koff, chunk, e2, h, ctr, partial, cv);
-            else
-                k_kick_mixed<1, false><<<nblocks, MK_T, 0, s>>>(L, F, order, koff, chunk, e2, h, ctr, partial, cv);
-        }
+        auto k = com ? (slices == 4 ? k_kick_mixed<4, true, true> : k_kick_mixed<1, true, true>)
+                     : (slices == 4 ? k_kick_mixed<4, false, true> : k_kick_mixed<1, false, true>);
+        if (!packed)
+            k = com ? (slices == 4 ? k_kick_mixed<4, true, false> : k_kick_mixed<1, true, false>)
+                    : (slices == 4 ? k_kick_mixed<4, false, false> : k_kick_mixed<1, false, false>);
+        k<<<nblocks, MK_T, 0, s>>>(L, F, order, koff, chunk, e2, h, ctr, partial, cv);
         CC_COUNT_LAUNCH(1);
     }
     if ((multi_chunk && nblocks > 0) || (drift_dt > 0.0 && L.total > 0)) {
