@@ -53,6 +53,7 @@ struct LevelAlloc {
     Level L{};
     FFView F{};
     bool classified = false;  // the last split's segmenting CTA also wrote the integrator lists
+    bool gathered = false;    // the level was just gathered: its forest, edge count and maxima are started
     // launch-shape variants: block prefixes over the sets (device) and the
     // total blocks (host) of every tunable shape, for the current layout
     int32_t *tau_off[N_TAU_VAR] = {}, *k64_off[N_K64_VAR] = {}, *mk_off[N_MK_VAR] = {};
@@ -584,9 +585,12 @@ static int ensure_level(cc_ctx *c, LevelAlloc &a, int need, int nsets)
 // incomplete list only means the next first-half split evaluates tau itself.
 constexpr long long EDGE_CAP_MAX = 1ll << 22;
 
+// the edge-record count of a level, in its split summary block
+static unsigned long long *edge_count_of(const LevelAlloc &a) { return (unsigned long long *)(a.d_ncomp + 2); }
+
 static int ensure_edges(cc_ctx *c, LevelAlloc &a, long long at_least = 0)
 {
-    a.E.count = (unsigned long long *)(a.d_ncomp + 2);  // in the split summary block
+    a.E.count = edge_count_of(a);
     const long long cap_max = c->p.edge_rec_max > 0 ? (long long)c->p.edge_rec_max : EDGE_CAP_MAX;
     long long want = std::max<long long>(std::max<long long>(4096, 4ll * a.cap), at_least);
     if (a.ecount > a.E.cap) want = std::max(want, 2 * a.ecount);
@@ -603,7 +607,7 @@ static int ensure_edges(cc_ctx *c, LevelAlloc &a, long long at_least = 0)
     }
     a.E.rec = (EdgeRec *)((char *)a.eblock + 256);
     a.E.cap = want;
-    a.E.count = (unsigned long long *)(a.d_ncomp + 2);
+    a.E.count = edge_count_of(a);
     return CC_OK;
 }
 
@@ -727,8 +731,11 @@ static int split_launch(cc_ctx *c, LevelAlloc &a, double h, const LevelAlloc *pa
     // FP32 kernel, the FP64 tau where the FP32 bounds leave it open: the
     // decisions are the FP64 predicate's, so the FP64 form's components,
     // and with them its state, stay the oracle's bit for bit.
-    // (a fresh split initialises its forest in the float-float copy's pass)
-    if (parent) launch_init_parent(a.L, a.E.count, s);
+    // (the forest, the edge count and the maxima start in the gather of this
+    // level, else in the float-float copy's pass)
+    const bool gathered = a.gathered;
+    a.gathered = false;
+    if (parent && !gathered) launch_init_parent(a.L, a.E.count, s);
     bool hook_in_seg = false;  // a first half's child edges hooked by the one-CTA segmentation
     const bool hold = c->p.split == CC_SPLIT_HOLD;
     if (parent) {
@@ -745,7 +752,7 @@ static int split_launch(cc_ctx *c, LevelAlloc &a, double h, const LevelAlloc *pa
         if (ntiles > 0x7fffffff) return fail(c, CC_E_ARG, "set too large for the tile grid");
         Level L = a.L;
         L.tile_off = a.tau_off[var];
-        launch_prep_ff(a.L, a.F, c->p.G, true, s, true, a.E.count);
+        launch_prep_ff(a.L, a.F, c->p.G, true, s, !gathered, a.E.count);
         const int ev = ev_begin(c, 0, nullptr, timed ? tk : -1, bin, var, (double)a.pairs);
         launch_tau_mixed(L, a.F, (int)ntiles, P, var, c->d_ctr, c->d_near_ij, c->d_near_tau, c->near_cap, a.E, s);
         ev_end(c, ev);
@@ -1178,7 +1185,8 @@ static int process(cc_ctx *c, int d, double h, const LevelAlloc *parent)
         }
         if (nl) {
             LevelAlloc &ch = c->lv[d + 1];
-            launch_gather(a.L, ch.L, a.members, a.lcomp_start, a.inv, s);
+            launch_gather(a.L, ch.L, a.members, a.lcomp_start, a.inv, edge_count_of(ch), ch.F.maxes, s);
+            ch.gathered = true;
             // first half: the state this split saw, so its edge records
             // (when complete) give the child's split; second half: fresh
             const bool reuse = half == 0 && a.ecount <= a.E.cap;

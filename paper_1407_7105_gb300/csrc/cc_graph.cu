@@ -48,6 +48,7 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int *tmp, int &total)
 // out[k] = sum of in[0..k); block sums to bsum
 __global__ void __launch_bounds__(SCAN_T) k_scan_tiles(const int *in, int *out, int n, int *bsum)
 {
+    pdl_begin();
     __shared__ int tmp[SCAN_T / 32];
     const int base = blockIdx.x * SCAN_TILE + threadIdx.x * SCAN_ITEMS;
     int v[SCAN_ITEMS], s = 0;
@@ -69,6 +70,7 @@ __global__ void __launch_bounds__(SCAN_T) k_scan_tiles(const int *in, int *out, 
 // single block: exclusive scan of bsum[0..nb) in place, chunked
 __global__ void __launch_bounds__(SCAN_T) k_scan_sums(int *bsum, int nb, int *grand)
 {
+    pdl_begin();
     __shared__ int tmp[SCAN_T / 32];
     __shared__ int carry;
     if (threadIdx.x == 0) carry = 0;
@@ -87,6 +89,7 @@ __global__ void __launch_bounds__(SCAN_T) k_scan_sums(int *bsum, int nb, int *gr
 
 __global__ void k_scan_add(int *out, int n, const int *bsum)
 {
+    pdl_begin();
     const int k = blockIdx.x * SCAN_TILE + threadIdx.x;
     const int add = bsum[blockIdx.x];
     for (int q = 0; q < SCAN_ITEMS; ++q) {
@@ -102,12 +105,12 @@ static void device_scan(const int *in, int *out, int n, int *bsum, int *grand, c
 {
     if (n <= 0) return;
     const int nb = scan_blocks(n);
-    k_scan_tiles<<<nb, SCAN_T, 0, s>>>(in, out, n, bsum);
+    launch_next(k_scan_tiles, nb, SCAN_T, 0, s, in, out, n, bsum);
     CC_COUNT_LAUNCH(1);
-    k_scan_sums<<<1, SCAN_T, 0, s>>>(bsum, nb, grand);
+    launch_next(k_scan_sums, 1, SCAN_T, 0, s, bsum, nb, grand);
     CC_COUNT_LAUNCH(1);
     if (nb > 1) {
-        k_scan_add<<<nb, SCAN_T, 0, s>>>(out, n, bsum);
+        launch_next(k_scan_add, nb, SCAN_T, 0, s, out, n, bsum);
         CC_COUNT_LAUNCH(1);
     }
 }
@@ -130,6 +133,7 @@ constexpr int RS_TILE = RS_T * RS_ROUNDS;
 
 __global__ void __launch_bounds__(RS_T) k_rs_hist(const uint32_t *keys, int n, int shift, int *hist, int ntiles)
 {
+    pdl_begin();
     __shared__ int h[256];
     h[threadIdx.x] = 0;
     __syncthreads();
@@ -146,6 +150,7 @@ __global__ void __launch_bounds__(RS_T) k_rs_scatter(const uint32_t *kin, const 
                                                       int32_t *vout, int n, int shift, const int *offs,
                                                       int ntiles)
 {
+    pdl_begin();
     __shared__ int base[256];
     __shared__ int wc[RS_T / 32][257];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -209,10 +214,10 @@ static void radix_sort(uint32_t *k, int32_t *v, int n, int bits, void *scratch, 
     int passes = (bits + 7) / 8;
     for (int p = 0; p < passes; ++p) {
         const int shift = 8 * p;
-        k_rs_hist<<<nt, RS_T, 0, s>>>(ka, n, shift, hist, nt);
+        launch_next(k_rs_hist, nt, RS_T, 0, s, ka, n, shift, hist, nt);
         CC_COUNT_LAUNCH(1);
         device_scan(hist, hist, 256 * nt, bsum, nullptr, s);
-        k_rs_scatter<<<nt, RS_T, 0, s>>>(ka, va, kb, vb, n, shift, hist, nt);
+        launch_next(k_rs_scatter, nt, RS_T, 0, s, ka, va, kb, vb, n, shift, hist, nt);
         CC_COUNT_LAUNCH(1);
         uint32_t *tk = ka; ka = kb; kb = tk;
         int32_t *tv = va; va = vb; vb = tv;
@@ -237,6 +242,7 @@ static int bits_for(long long maxval)
 // otherwise queue on one counter)
 __global__ void k_compress(Level L, int32_t *root)
 {
+    pdl_begin();
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     const bool in = k < L.total;
     const bool valid = in && L.gid[k] >= 0;
@@ -249,7 +255,7 @@ __global__ void k_compress(Level L, int32_t *root)
 void launch_compress(const Level &L, int32_t *root, cudaStream_t s)
 {
     if (L.total <= 0) return;
-    k_compress<<<(L.total + 255) / 256, 256, 0, s>>>(L, root);
+    launch_next(k_compress, (L.total + 255) / 256, 256, 0, s, L, root);
     CC_COUNT_LAUNCH(1);
 }
 
@@ -260,6 +266,7 @@ void launch_compress(const Level &L, int32_t *root, cudaStream_t s)
 // sit between runs in ascending order.  comp_start indexes this order.
 __global__ void k_seg_keys(Level L, const int32_t *root, uint32_t *key, int32_t *val)
 {
+    pdl_begin();
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= L.total) return;
     key[k] = L.gid[k] >= 0 ? (uint32_t)root[k] : (uint32_t)k;
@@ -268,6 +275,7 @@ __global__ void k_seg_keys(Level L, const int32_t *root, uint32_t *key, int32_t 
 
 __global__ void k_seg_heads(Level L, const uint32_t *key, int n, int *flag)
 {
+    pdl_begin();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= n) return;
     flag[t] = L.cnt[key[t]] >= 2 && (t == 0 || key[t] != key[t - 1]) ? 1 : 0;
@@ -276,6 +284,7 @@ __global__ void k_seg_heads(Level L, const uint32_t *key, int n, int *flag)
 __global__ void k_seg_bounds(Level L, const uint32_t *key, const int32_t *val, const int *flag, const int *cidx,
                              int n, int32_t *members, int32_t *comp_start, int32_t *comp_size, int32_t *ncomp)
 {
+    pdl_begin();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= n) return;
     members[t] = val[t];
@@ -306,13 +315,13 @@ void launch_segment(const Level &L, const int32_t *root, int32_t *members, int32
     int *bsum = cidx + n;
     void *sort_scratch = (void *)(bsum + scan_blocks(n) + 16);
     const int g = (n + 255) / 256;
-    k_seg_keys<<<g, 256, 0, s>>>(L, root, key, val);
+    launch_next(k_seg_keys, g, 256, 0, s, L, root, key, val);
     CC_COUNT_LAUNCH(1);
     radix_sort(key, val, n, bits_for(n), sort_scratch, s);
-    k_seg_heads<<<g, 256, 0, s>>>(L, key, n, flag);
+    launch_next(k_seg_heads, g, 256, 0, s, L, key, n, flag);
     CC_COUNT_LAUNCH(1);
     device_scan(flag, cidx, n, bsum, nullptr, s);
-    k_seg_bounds<<<g, 256, 0, s>>>(L, key, val, flag, cidx, n, members, comp_start, comp_size, d_ncomp);
+    launch_next(k_seg_bounds, g, 256, 0, s, L, key, val, flag, cidx, n, members, comp_start, comp_size, d_ncomp);
     CC_COUNT_LAUNCH(1);
 }
 
@@ -457,6 +466,7 @@ __global__ void __launch_bounds__(SEG1_T) k_segment_small(Level L, int32_t *root
                                                           int32_t *comp_start, int32_t *comp_size, int32_t *ncomp,
                                                           EdgeList hook, DevCounters *ctr, ClassifyArgs cls)
 {
+    pdl_begin();
     extern __shared__ int seg1_smem[];
     const int n = L.total, tid = threadIdx.x;
     int *s_root = seg1_smem;      // roots (-1: padding), then the member list being built
@@ -668,7 +678,7 @@ bool launch_compress_segment(const Level &L, int32_t *root, int32_t *members, in
         const EdgeList none{nullptr, nullptr, 0};
         ClassifyArgs nc{};
         if (cls) nc = *cls;
-        k_segment_small<<<1, SEG1_T, (size_t)L.total * 8, s>>>(L, root, members, comp_start, comp_size, d_ncomp,
+        launch_next(k_segment_small, 1, SEG1_T, (size_t)L.total * 8, s, L, root, members, comp_start, comp_size, d_ncomp,
                                                                hook ? *hook : none, ctr, nc);
         CC_COUNT_LAUNCH(1);
         return cls != nullptr;
@@ -778,10 +788,18 @@ __device__ __forceinline__ int upper_find(const int32_t *off, int nsets, int t)
 // c (child set c) copies its state from the parent, a padding slot is
 // marked (gid = -1); inv[k] = the child index of parent element k (written
 // for the gathered elements only; a reader checks C.src[inv[k]] == k)
-__global__ void k_gather(Level P, Level C, const int32_t *members, const int32_t *lcomp_start, int32_t *inv)
+__global__ void k_gather(Level P, Level C, const int32_t *members, const int32_t *lcomp_start, int32_t *inv,
+                         unsigned long long *edge_count, float *maxes)
 {
+    pdl_begin();
     const int d = blockIdx.x * blockDim.x + threadIdx.x;
     if (d >= C.total) return;
+    C.parent[d] = d;
+    C.cnt[d] = 0;
+    if (d == 0) {
+        *edge_count = 0ull;
+        maxes[0] = maxes[1] = 0.f;
+    }
     const int c = upper_find(C.set_start, C.nsets, d);
     const int w = d - C.set_start[c];
     if (w >= C.set_n[c]) {
@@ -800,16 +818,18 @@ __global__ void k_gather(Level P, Level C, const int32_t *members, const int32_t
 }
 
 void launch_gather(const Level &P, const Level &C, const int32_t *members, const int32_t *lcomp_start, int32_t *inv,
-                   cudaStream_t s)
+                   unsigned long long *edge_count, float *maxes, cudaStream_t s)
 {
     if (C.total > 0) {
-        k_gather<<<(C.total + 255) / 256, 256, 0, s>>>(P, C, members, lcomp_start, inv);
+        launch_next(k_gather, (C.total + 255) / 256, 256, 0, s, P, C, members, lcomp_start, inv, edge_count,
+                    maxes);
         CC_COUNT_LAUNCH(1);
     }
 }
 
 __global__ void k_scatter(Level P, Level C)
 {
+    pdl_begin();
     const int d = blockIdx.x * blockDim.x + threadIdx.x;
     if (d >= C.total || C.gid[d] < 0) return;
     const int k = C.src[d];
@@ -820,7 +840,7 @@ __global__ void k_scatter(Level P, Level C)
 void launch_scatter(const Level &P, const Level &C, cudaStream_t s)
 {
     if (C.total > 0) {
-        k_scatter<<<(C.total + 255) / 256, 256, 0, s>>>(P, C);
+        launch_next(k_scatter, (C.total + 255) / 256, 256, 0, s, P, C);
         CC_COUNT_LAUNCH(1);
     }
 }
@@ -940,6 +960,7 @@ void launch_label_canon(const Level &L, const int32_t *root, int32_t *labels_out
 // x_i += dt * v_i (Eq. drift) for rest-set members: component size 1
 __global__ void k_drift_root(Level L, const int32_t *root, double dt)
 {
+    pdl_begin();
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= L.total || L.gid[k] < 0 || L.cnt[root[k]] != 1) return;
     L.x[k] = __dadd_rn(L.x[k], __dmul_rn(dt, L.vx[k]));
@@ -950,7 +971,7 @@ __global__ void k_drift_root(Level L, const int32_t *root, double dt)
 void launch_drift(const Level &L, const int32_t *root, double dt, cudaStream_t s)
 {
     if (L.total > 0) {
-        k_drift_root<<<(L.total + 255) / 256, 256, 0, s>>>(L, root, dt);
+        launch_next(k_drift_root, (L.total + 255) / 256, 256, 0, s, L, root, dt);
         CC_COUNT_LAUNCH(1);
     }
 }
@@ -1103,6 +1124,7 @@ __device__ __forceinline__ uint32_t spread3(uint32_t v)
 
 __global__ void k_morton_keys(const double *x3, long long n, const unsigned *box, uint32_t *key, int32_t *val)
 {
+    pdl_begin();
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= n) return;
     uint32_t code = 0;
@@ -1120,6 +1142,7 @@ __global__ void k_morton_keys(const double *x3, long long n, const unsigned *box
 
 __global__ void k_perm_from_sorted(const int32_t *val, long long n, int32_t *perm)
 {
+    pdl_begin();
     const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (p < n) perm[val[p]] = (int32_t)p;
 }
@@ -1134,9 +1157,9 @@ void launch_spatial_order(const double *x3, long long n, int32_t *perm, unsigned
     k_pos_box<<<g, 256, 0, s>>>(x3, n, box);
     uint32_t *key = (uint32_t *)scratch;
     int32_t *val = (int32_t *)(key + n);
-    k_morton_keys<<<g, 256, 0, s>>>(x3, n, box, key, val);
+    launch_next(k_morton_keys, g, 256, 0, s, x3, n, box, key, val);
     radix_sort(key, val, (int)n, 30, (void *)(val + n), s);
-    k_perm_from_sorted<<<g, 256, 0, s>>>(val, n, perm);
+    launch_next(k_perm_from_sorted, g, 256, 0, s, val, n, perm);
     CC_COUNT_LAUNCH(3);
 }
 

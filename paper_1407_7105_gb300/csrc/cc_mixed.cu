@@ -54,6 +54,7 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
 // float-float copy of the packed state; per-level maxima of |x| and |v|
 __global__ void k_prep_ff(Level L, FFView F, float G, int with_v, int init_forest, unsigned long long *edge_count)
 {
+    pdl_begin();
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     float ax = 0.f, av = 0.f;
     if (init_forest) {
@@ -104,12 +105,12 @@ __global__ void k_prep_ff(Level L, FFView F, float G, int with_v, int init_fores
     }
 }
 
-void launch_prep_ff(const Level &L, const FFView &F, double G, bool with_v, cudaStream_t s, bool init_forest,
+void launch_prep_ff(const Level &L, const FFView &F, double G, bool with_v, cudaStream_t s, bool init,
                     unsigned long long *edge_count)
 {
     if (L.total <= 0) return;
-    cudaMemsetAsync(F.maxes, 0, 2 * sizeof(float), s);
-    k_prep_ff<<<(L.total + 255) / 256, 256, 0, s>>>(L, F, (float)G, with_v ? 1 : 0, init_forest ? 1 : 0,
+    if (init) cudaMemsetAsync(F.maxes, 0, 2 * sizeof(float), s);
+    launch_next(k_prep_ff, (L.total + 255) / 256, 256, 0, s, L, F, (float)G, with_v ? 1 : 0, init ? 1 : 0,
                                                     edge_count);
     CC_COUNT_LAUNCH(1);
 }
@@ -129,6 +130,7 @@ __device__ __forceinline__ float *kick_slot(const FFView &F, int t)
 __global__ void k_prep_kick(Level L, FFView F, const int32_t *order, const int32_t *root, float G, double dt,
                             int packed)
 {
+    pdl_begin();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= L.total) return;
     const int k = order[t];
@@ -165,7 +167,7 @@ void launch_prep_kick(const Level &L, const FFView &F, const int32_t *order, con
                       double drift_dt, bool packed, cudaStream_t s)
 {
     if (L.total <= 0) return;
-    k_prep_kick<<<(L.total + 255) / 256, 256, 0, s>>>(L, F, order, root, (float)G, drift_dt, packed ? 1 : 0);
+    launch_next(k_prep_kick, (L.total + 255) / 256, 256, 0, s, L, F, order, root, (float)G, drift_dt, packed ? 1 : 0);
     CC_COUNT_LAUNCH(1);
 }
 
@@ -441,6 +443,7 @@ __global__ void __launch_bounds__(T *S / R, 768 * R / (T * S))
                 const __grid_constant__ TauParams P, const __grid_constant__ MixedTauBounds Q, DevCounters *ctr,
                 int32_t *near_ij, double *near_tau, long long near_cap, const __grid_constant__ EdgeList E)
 {
+    pdl_begin();
     constexpr int THREADS = T * S / R, NW = THREADS / 32, RW = T / (32 * R);
     constexpr int TC = T / S, GW = TC / TAU_JG;  // a warp's columns and column groups
     static_assert(T % (32 * R) == 0 && TC % 32 == 0 && T <= 256, "tile shape");
@@ -725,13 +728,13 @@ void launch_tau_mixed(const Level &L, const FFView &F, int ntiles, const TauPara
                       TAU_VAR_T[3] == 256,
                   "tau variants");
     if (variant == 0)
-        k_tau_mixed<64, 1, 1, false><<<ntiles, 64, 0, s>>>(L, F, P, Q, ctr, near_ij, near_tau, near_cap, E);
+        launch_next(k_tau_mixed<64, 1, 1, false>, ntiles, 64, 0, s, L, F, P, Q, ctr, near_ij, near_tau, near_cap, E);
     else if (variant == 1)
-        k_tau_mixed<128, 1, 1, false><<<ntiles, 128, 0, s>>>(L, F, P, Q, ctr, near_ij, near_tau, near_cap, E);
+        launch_next(k_tau_mixed<128, 1, 1, false>, ntiles, 128, 0, s, L, F, P, Q, ctr, near_ij, near_tau, near_cap, E);
     else if (variant == 2)
-        k_tau_mixed<64, 2, 1, false><<<ntiles, 128, 0, s>>>(L, F, P, Q, ctr, near_ij, near_tau, near_cap, E);
+        launch_next(k_tau_mixed<64, 2, 1, false>, ntiles, 128, 0, s, L, F, P, Q, ctr, near_ij, near_tau, near_cap, E);
     else
-        k_tau_mixed<256, 1, 2, false><<<ntiles, 128, 0, s>>>(L, F, P, Q, ctr, near_ij, near_tau, near_cap, E);
+        launch_next(k_tau_mixed<256, 1, 2, false>, ntiles, 128, 0, s, L, F, P, Q, ctr, near_ij, near_tau, near_cap, E);
     CC_COUNT_LAUNCH(1);
 }
 
@@ -828,6 +831,7 @@ __global__ void __launch_bounds__(MK_T) k_kick_mixed(Level L, FFView F, const in
                                                       int chunk, float eps2, double h, DevCounters *ctr,
                                                       double *partial, ComView cv)
 {
+    pdl_begin();
     constexpr int R = MK_T / S;  // i rows per block
     static_assert(R % 32 == 0, "one slice per warp");
     __shared__ MixedKickSmem sm;
@@ -1055,6 +1059,7 @@ constexpr int KR_LANES = 8;
 __global__ void k_kick_reduce(Level L, FFView F, const int32_t *order, int chunk, double h, const double *partial,
                               const int32_t *root, double drift_dt)
 {
+    pdl_begin();
     const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const int t = (int)(g / KR_LANES), sub = (int)(g % KR_LANES);
     int k = -1, nchunk = 1;
@@ -1119,12 +1124,12 @@ void launch_kick_mixed(const Level &L, const FFView &F, const int32_t *order, co
         if (!packed)
             k = com ? (slices == 4 ? k_kick_mixed<4, true, false> : k_kick_mixed<1, true, false>)
                     : (slices == 4 ? k_kick_mixed<4, false, false> : k_kick_mixed<1, false, false>);
-        k<<<nblocks, MK_T, 0, s>>>(L, F, order, koff, chunk, e2, h, ctr, partial, cv);
+        launch_next(k, nblocks, MK_T, 0, s, L, F, order, koff, chunk, e2, h, ctr, partial, cv);
         CC_COUNT_LAUNCH(1);
     }
     if ((multi_chunk && nblocks > 0) || (drift_dt > 0.0 && L.total > 0)) {
         const long long threads = (long long)L.total * KR_LANES;
-        k_kick_reduce<<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(L, F, order, multi_chunk ? chunk : 1 << 30, h,
+        launch_next(k_kick_reduce, (unsigned)((threads + 255) / 256), 256, 0, s, L, F, order, multi_chunk ? chunk : 1 << 30, h,
                                                                         partial, root, drift_dt);
         CC_COUNT_LAUNCH(1);
     }
