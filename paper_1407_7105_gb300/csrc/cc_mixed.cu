@@ -1119,11 +1119,10 @@ void launch_kick_mixed(const Level &L, const FFView &F, const int32_t *order, co
     if (nblocks > 0) {
         const ComView cv = com ? *com : ComView{nullptr, nullptr, nullptr, nullptr};
         const float e2 = (float)eps2;
-        auto k = com ? (slices == 4 ? k_kick_mixed<4, true, true> : k_kick_mixed<1, true, true>)
-                     : (slices == 4 ? k_kick_mixed<4, false, true> : k_kick_mixed<1, false, true>);
-        if (!packed)
-            k = com ? (slices == 4 ? k_kick_mixed<4, true, false> : k_kick_mixed<1, true, false>)
-                    : (slices == 4 ? k_kick_mixed<4, false, false> : k_kick_mixed<1, false, false>);
+        // (levels of packed size have far more blocks than the sliced shape is for)
+        auto k = packed ? (com ? k_kick_mixed<1, true, true> : k_kick_mixed<1, false, true>)
+                 : slices == 4 ? (com ? k_kick_mixed<4, true, false> : k_kick_mixed<4, false, false>)
+                               : (com ? k_kick_mixed<1, true, false> : k_kick_mixed<1, false, false>);
         launch_next(k, nblocks, MK_T, 0, s, L, F, order, koff, chunk, e2, h, ctr, partial, cv);
         CC_COUNT_LAUNCH(1);
     }
