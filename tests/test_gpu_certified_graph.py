@@ -8,6 +8,7 @@ import numpy as np
 import pytest
 
 from oracle import oracle as O
+from paper_1407_7105_gb300 import ics
 
 pytestmark = pytest.mark.gpu
 
@@ -88,3 +89,18 @@ def test_noalloc_on_values_no_context_takes(cclib, plummer_ic, what, bad):
         want = new
     assert np.array_equal(lab, want)
     assert k == int((np.bincount(want) >= 2).sum())
+
+
+@pytest.mark.parametrize("n", [2, 46, 64, 511, 512, 513, 600])
+def test_graph_of_every_pair_is_sorted(cclib, n):
+    """Every pair an edge: the edge list in order, at sizes around the sort's
+    tiles (1024 keys: 46 bodies have 1035 pairs) and around the 128 tiles up to
+    which the scatter scans the histograms itself (512: 130816 pairs, 513:
+    131328)."""
+    m, x, v = ics.plummer(n, seed=n, exact_scale=False)
+    c = cclib.Context(m, x, v)
+    edges, count, _ = c.timestep_graph(1e4, cap=n * n)
+    c.close()
+    i, j = np.triu_indices(n, 1)
+    assert count == i.size
+    assert np.array_equal(edges, np.stack([i, j], axis=1))
