@@ -45,13 +45,13 @@ TAU_FLOPS = 47   # Eq. tauij as evaluated: 3 sqrt, 6 div, 38 add/sub/mul
 KICK_FLOPS = 25  # one pair force applied to both bodies (Eqs. kickij/kickji): the difference (3), r^2 (6),
                  # r^-3 (sqrt, mul, div: 3), the weights (2 x 2) and the two 3-vector updates (2 x 3); the
                  # mixed form's row kick evaluates each pair from both sides, which is not credited (the
-                 # FP64 kick evaluates each unordered pair once, k_pair_forces, and sums rows, k_kick64)
+                 # FP64 kick evaluates each unordered pair once, k_pair_forces, and sums rows, k_kick_rows)
 # DRAM bytes (read + write) per launch of the pair kernels, averaged over the
 # launches of one step in an ncu capture (dram__bytes_read.sum +
 # dram__bytes_write.sum): profiles/launches_plummer16384_mixed.md (mixed form)
 # and profiles/k_tau_hook_k_kick64_plummer16384_fp64.md (FP64 form; the FP64
 # kick's two kernels per kick call: profiles/launches_plummer16384_fp64.md)
-KERNEL_TRAFFIC = {"k_kick_mixed": 391e3, "k_tau_mixed": 850e3, "k_pair_forces+k_kick64": 3.07e9, "k_tau_hook": 616e3}
+KERNEL_TRAFFIC = {"k_kick_mixed": 391e3, "k_tau_mixed": 850e3, "k_pair_forces+k_kick_rows": 3.07e9, "k_tau_hook": 616e3}
 
 
 WORKLOADS = {
@@ -477,7 +477,7 @@ def run_gpu(args, rank, world):
     # both forms' splits run the certified FP32 tau kernel; the kicks are the
     # form's own (FP32 in the mixed form, FP64 in the FP64 form)
     fp32 = fp32 or kname == "tau"
-    kname = "k_tau_mixed" if kname == "tau" else ("k_kick_mixed" if fp32 else "k_pair_forces+k_kick64")
+    kname = "k_tau_mixed" if kname == "tau" else ("k_kick_mixed" if fp32 else "k_pair_forces+k_kick_rows")
     achieved = flops / (kms * 1e-3) / 1e12 if kms > 0 else None
     peak = (f32_peak if fp32 else f64_peak) / 1e12
     small_flops = TAU_FLOPS * tm["small_tau_evaluated"] + KICK_FLOPS * tm["small_kick_pairs"]

@@ -79,8 +79,9 @@ typedef struct {
                           list, and the first halves of its components then run
                           a fresh split (results are the same, only slower)    */
     int    fault_test; /* 0 in normal use.  Failure-path test hooks of the tau
-                          kernels (the certified one of every split, the FP64
-                          one of cc_timestep_graph), so that a test can see a
+                          kernels (the certified one of every split and of
+                          cc_timestep_graph, there with near_tol above 1e-6 the
+                          FP64 one), so that a test can see a
                           bounded wait or retry run out and the call return
                           CC_E_TIMEOUT without any GPU fault: 1 = the tile copy
                           is announced but never issued, so the mbarrier wait

@@ -343,7 +343,7 @@ constexpr long long MK_PACKED_MIN = 1ll << 29;
 constexpr int MK_TILE = 128;
 void launch_tau_hook(const Level &L, int ntiles, const TauParams &P, DevCounters *ctr,
                      int32_t *edges, long long edge_cap, int32_t *near_ij, double *near_tau, long long near_cap,
-                     cudaStream_t s, const EdgeList *rec = nullptr);
+                     cudaStream_t s);
 // first-half split from the parent split's edge records: the records that
 // are edges at P.h and whose endpoints the gather moved to this level (inv =
 // parent index -> child index) are hooked and recorded for this split

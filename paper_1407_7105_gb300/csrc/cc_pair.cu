@@ -1,8 +1,12 @@
 // cc_pair.cu -- pairwise kernels of the CC split (arXiv:1407.7105):
-//   * tau(i,j) over all pairs of each set fused with the edge test
-//     tau < h (Sec. 2.2) and union-find hooking of every edge;
+//   * tau(i,j) in FP64 over all pairs of a set fused with the edge test
+//     tau < h (Sec. 2.2), for a time-step graph whose near_tol is wider than
+//     the certified kernel's bounds, and the edge list itself;
+//   * a first half's edges from its parent's records;
 //   * the kick K_{h,V_ij} between members of different components
-//     (Eqs. kickij, kickji; Sec. 2.2 K_{h, V_R + V_CC + V_CR});
+//     (Eqs. kickij, kickji; Sec. 2.2 K_{h, V_R + V_CC + V_CR}) in FP64: rows
+//     in place (k_kick64), or from 2^18 pairs each pair's force once
+//     (k_pair_forces) and the rows summed after it (k_kick_rows);
 //   * the energy diagnostic H (Eq. Hamiltonian).
 // j-tiles are staged in shared memory by TMA bulk copies (cp.async.bulk)
 // completing on an mbarrier; every wait is bounded.
@@ -68,7 +72,7 @@ __device__ __forceinline__ void log_pair(const TauParams &P, double tau, int gi,
 
 template <int T>
 __global__ void __launch_bounds__(T) k_tau_hook(Level L, TauParams P, DevCounters *ctr, int32_t *near_ij,
-                                                     double *near_tau, long long near_cap, EdgeList E)
+                                                     double *near_tau, long long near_cap)
 {
     __shared__ TauSmem<T> sm;
     const int tid = threadIdx.x;
@@ -146,10 +150,6 @@ __global__ void __launch_bounds__(T) k_tau_hook(Level L, TauParams P, DevCounter
             if (tau < P.h) {
                 ++my_edges;
                 if (!uf_union(L.parent, i, j, uf_retry)) raise_err(ctr, DERR_UF_RETRY);
-                // a record serves the first half at h/2: kept when the pair
-                // is an edge there or near h/2
-                if (E.rec && (tau < 0.5 * P.h || fabs(tau - 0.5 * P.h) < P.near_tol * 0.5 * P.h))
-                    record_edge(E, i, j, -1, tau);
             }
         }
     }
@@ -367,16 +367,15 @@ __global__ void __launch_bounds__(TAU_T) k_tau_edges(Level L, TauParams P, DevCo
 
 void launch_tau_hook(const Level &L, int ntiles, const TauParams &P, DevCounters *ctr,
                      int32_t *edges, long long edge_cap, int32_t *near_ij, double *near_tau, long long near_cap,
-                     cudaStream_t s, const EdgeList *rec)
+                     cudaStream_t s)
 {
     if (ntiles <= 0) return;
-    const EdgeList E = rec ? *rec : EdgeList{nullptr, nullptr, 0};
     if (edges) {
         k_tau_edges<<<ntiles, TAU_T, 0, s>>>(L, P, ctr, edges, edge_cap, near_ij, near_tau, near_cap);
         CC_COUNT_LAUNCH(1);
         return;
     }
-    k_tau_hook<TAU_T><<<ntiles, TAU_T, 0, s>>>(L, P, ctr, near_ij, near_tau, near_cap, E);
+    k_tau_hook<TAU_T><<<ntiles, TAU_T, 0, s>>>(L, P, ctr, near_ij, near_tau, near_cap);
     CC_COUNT_LAUNCH(1);
 }
 
