@@ -1,295 +1,13 @@
 // cc_device.cuh -- device functions shared by several kernels of libcc.so:
-// the certified FP32 decision of the edge predicate tau(i,j) < h
-// (arXiv:1407.7105 Eq. tauij), compensated summation, and the universal-
-// variable two-body flow of the CC_KEPLER variant (Sec. 3.2).
+// float-float splits, edge depths, compensated summation, and the universal-
+// variable two-body flow of the CC_KEPLER variant (arXiv:1407.7105 Sec. 3.2).
+// (The certified FP32 decision of the edge predicate is in cc_tau32.cuh.)
 #pragma once
 #include "cc_fp64.cuh"
 #include "cc_internal.cuh"
+#include "cc_tau32.cuh"
 
 namespace cc {
-
-// ------------------------------------------------------------ tau, FP32 certified
-// Error model (u = 2^-24; +,-,*,fma round to nearest: u each; rsqrtf within
-// 2 ulp, budgeted 8u; every bound below is budgeted generously):
-//   |dx~ - dx| <= er r,  er = 2.05u + 11u^2 X / r      (float-float difference)
-//   |dv~ - dv| <= ev |dv|, ev = 2.05u + 11u^2 V / |dv|
-//   rinv = rsqrt(r2), s1 = rsqrt(r mu), s2 = rsqrt(v2)
-//   T_ff = eta r2 s1          (= eta sqrt(r^3/mu)),      rel. error <= 40u + 3er
-//   T_fb = eta r s2           (= eta r/|dv|),            rel. error <= 40u + 3er + 3ev
-//   dT_ff = 1.5 eta rv s1,  dT_fb = eta rv s2 rinv (1 + mu s2^2 rinv)
-//   rv = dx.dv has no relative bound (cancellation): |drv| <= (er+ev+4u) r |dv|,
-//   so |d dT| <= 32u|dT_ff| + 1.5 eta s1 |drv|   (ff)
-//              80u|dT_fb| + eta s2 rinv (1 + mu s2^2 rinv) |drv|   (fb)
-//   D = 1 - min(dT,1)/2 >= 1/2,  |dD| <= |d dT|/2 + 2u D
-// tau_x = T_x / D_x < h is certain when T~(1+eT)(1+s) < h (D~ - dD), and
-// certainly false when T~(1-eT)(1-s) >= h (D~ + dD); the slack s = 2e-6
-// covers the FP32 evaluation of the bounds and the FP64 predicate's own
-// rounding.  Any NaN/Inf fails both tests: the pair is undecided.
-constexpr float U32 = 5.9604645e-8f;  // 2^-24
-constexpr float SLACK = 2e-6f;
-
-// eta and eta/h in float (the decision compares T/h with D); c_x = 11 u^2 X
-// and c_v = 11 u^2 V carry the float-float rounding of the differences
-struct MixedTauParams {
-    float eta, etah, eps2, G;
-    float hq;  // eta/etah (h, or h/eta when eta multiplies the min): the pre-test's q = hq |dv|/r
-};
-// the tau kernel's: with tau_pair_bounds' constants (c^2, T^2, V of its bounds;
-// pb_c2 < 0: they are off)
-struct MixedTauBounds : MixedTauParams {
-    float pb_c2, pb_r3, pb_v;
-};
-
-// The h-independent part of the decision: everything except T/h.  The
-// decision at a threshold h then costs two products and four comparisons,
-// and since eta/h doubles exactly when h halves, T/h at h 2^-m is T/h at h
-// times 2^m bit for bit: decide(prep, etah * 2^m) is the decision the full
-// evaluation would take at h 2^-m for the same state.
-struct TauPrep32 {
-    float r2, s1, r, s2;         // Tff/h = (etah r2) s1, Tfb/h = (etah r) s2
-    float ffA, ffB, ffLo, ffHi;  // ff edge certain: Tff ffA < ffLo; no edge certain: Tff ffB >= ffHi
-    float fbA, fbB, fbLo, fbHi;  // the same for the flyby term
-    bool fb;                     // flyby term usable (else only a certain ff edge decides)
-};
-
-__device__ __forceinline__ TauPrep32 tau_prep_fp32(float dx0, float dx1, float dx2, float dv0, float dv1, float dv2,
-                                                   float mu, float c_x, float c_v, const MixedTauParams &Q)
-{
-    TauPrep32 t;
-    const float A = 1.f + SLACK, B = 1.f - SLACK;
-    const float r2 = fmaf(dx2, dx2, fmaf(dx1, dx1, fmaf(dx0, dx0, Q.eps2)));
-    const float v2 = fmaf(dv2, dv2, fmaf(dv1, dv1, dv0 * dv0));
-    const float rv = fmaf(dx2, dv2, fmaf(dx1, dv1, dx0 * dv0));
-    const float rinv = rsqrtf(r2);
-    const float r = r2 * rinv;
-    const float s1 = rsqrtf(r * mu);
-    const float er = fmaf(c_x, rinv, 2.05f * U32);
-    const float s2 = v2 > 0.f ? rsqrtf(v2) : 0.f;
-    const float vn = v2 * s2;  // |dv|
-    const float ev = fmaf(c_v, s2, 2.05f * U32);
-    const float drv = (er + ev + 4.f * U32) * (r * vn);
-    // free fall: T/h = (eta/h) r2 s1, dT/dt = 1.5 eta rv s1
-    const float dTff = 1.5f * Q.eta * rv * s1;
-    const float Dff = fmaf(-0.5f, fminf(dTff, 1.f), 1.f);
-    const float dDff = fmaf(0.5f, fmaf(32.f * U32, fabsf(dTff), 1.5f * Q.eta * s1 * drv), 2.f * U32 * Dff);
-    const float eff = fmaf(3.f, er, 40.f * U32);
-    t.r2 = r2;
-    t.s1 = s1;
-    t.r = r;
-    t.s2 = s2;
-    t.ffA = fmaf(eff, A, A);
-    t.ffB = fmaf(-eff, B, B);
-    t.ffLo = Dff - dDff;
-    t.ffHi = Dff + dDff;
-    // an exactly zero (or unresolved) FP32 velocity difference may hide a
-    // tiny nonzero FP64 one, whose flyby term can be small: only a certain
-    // free-fall edge decides such a pair
-    t.fb = (v2 > 0.f) && !(vn < 6.f * c_v);
-    // flyby: T/h = (eta/h) r s2, dT/dt = eta rv s2 rinv (1 + mu s2^2 rinv)
-    const float g = fmaf(mu * s2 * s2, rinv, 1.f);
-    const float k = s2 * rinv * g;
-    const float dTfb = Q.eta * rv * k;
-    const float Dfb = fmaf(-0.5f, fminf(dTfb, 1.f), 1.f);
-    const float dDfb = fmaf(0.5f, fmaf(80.f * U32, fabsf(dTfb), Q.eta * k * drv), 2.f * U32 * Dfb);
-    const float efb = fmaf(3.f, er + ev, 40.f * U32);
-    t.fbA = fmaf(efb, A, A);
-    t.fbB = fmaf(-efb, B, B);
-    t.fbLo = Dfb - dDfb;
-    t.fbHi = Dfb + dDfb;
-    return t;
-}
-
-// returns 1 = edge certain, 0 = no edge certain, -1 = undecided; etah =
-// eta/h in float
-__device__ __forceinline__ int tau_decide_at(const TauPrep32 &t, float etah)
-{
-    const float Tff = etah * t.r2 * t.s1;
-    const bool ff_yes = Tff * t.ffA < t.ffLo;
-    if (!t.fb) return ff_yes ? 1 : -1;
-    const bool ff_no = Tff * t.ffB >= t.ffHi;
-    const float Tfb = etah * t.r * t.s2;
-    const bool fb_yes = Tfb * t.fbA < t.fbLo;
-    const bool fb_no = Tfb * t.fbB >= t.fbHi;
-    if (ff_yes || fb_yes) return 1;
-    if (ff_no && fb_no) return 0;
-    return -1;
-}
-
-// A sufficient test for "no edge" that skips the certified evaluation for
-// the great majority of pairs (those whose tau is well above h).  With T =
-// T_ff or T_fb and D = 1 - min(dT/dt, 1)/2, tau_x = T/D and D <= 1 + |dT/dt|/2:
-//   free fall: |dT_ff/dt| = 1.5 T_ff |rv|/r^2 <= 1.5 T_ff |dv|/r, so
-//     tau_ff >= h  if  (T_ff/h) (1 - 0.75 q) >= 1,  q = h|dv|/r (q < 4/3);
-//   flyby:     |dT_fb/dt| <= eta (1 + mu/(r v^2))  (T_fb = eta r/|dv|), so
-//     tau_fb >= h  if  T_fb/h >= 1 + eta (1 + mu/(r v^2))/2.
-// (eta is the factor inside T: Q.eta; hq = h/eta_in, the same as
-// eta/etah in both readings of the eta placement.)  The differences may be
-// formed from the rounded high parts alone: then |dx~ - dx| <= u r + c_x
-// + 3.5 u r with c_x = 7 u max|x_i| (per component |x_j| <= |x_i| + r),
-// likewise c_v for the velocities.  Once (c_x + 3.5 u r)/r and the velocity
-// analogue are below 1e-4, every FP32 quantity used has relative
-// error below 1e-3 (the error model above: 40u + 3(er + ev) plus the rsqrt
-// budget), so a 2 % margin on each inequality makes the test rigorous; a
-// pair it does not settle goes to the certified decision.
-// reciprocal square root, PTX rsqrt.approx.ftz.f32 (relative error below
-// 2^-22.9 for normal inputs; a denormal input is flushed to zero and gives
-// +inf, which the pre-test's comparisons reject)
-__device__ __forceinline__ float rsqrt_ftz(float x)
-{
-    float y;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
-__device__ __forceinline__ bool tau_quick_apart(float dx0, float dx1, float dx2, float dv0, float dv1, float dv2,
-                                                float mu, float c_x, float c_v, const MixedTauParams &Q)
-{
-    const float r2 = fmaf(dx2, dx2, fmaf(dx1, dx1, fmaf(dx0, dx0, Q.eps2)));
-    const float v2 = fmaf(dv2, dv2, fmaf(dv1, dv1, dv0 * dv0));
-    const float rinv = rsqrt_ftz(r2);
-    const float r = r2 * rinv;
-    const float s1 = rsqrt_ftz(r * mu);
-    const float s2 = rsqrt_ftz(v2);   // inf for v2 = 0: rejected below
-    const float vn = v2 * s2;         // |dv|
-    const float Tff = Q.etah * r2 * s1;                  // T_ff / h
-    const float q = Q.hq * vn * rinv;                    // h |dv| / r
-    const float Tfb = Q.etah * r * s2;                   // T_fb / h
-    const float g = mu * rinv * s2 * s2;                 // mu / (r v^2)
-    const float M = 1.02f;
-    // (the bounds below leave 3.5u for a relative part of c_x/r, c_v/|dv|;
-    // all conditions are evaluated: no short-circuit branches)
-    const bool ok = (c_x * rinv <= 0.99e-4f) & (v2 > 0.f) & (c_v * s2 <= 0.99e-4f) & (0.75f * M * q < 1.f) &
-                    (Tff * fmaf(-0.75f * M, q, 1.f) >= M) & (Tfb >= M * fmaf(0.5f * Q.eta, 1.f + g, 1.f));
-    return ok;
-}
-
-// The same bounds over every pair of two groups of bodies at once.  A group
-// is summarised by the boxes of its high parts (positions, velocities) and
-// its largest G m.  Over pairs (i in A, j in B): r >= d = the boxes'
-// distance (softened), |dv| <= vmax (the velocity boxes' widest relative
-// speed), mu <= muA + muB.  Free fall: T_ff/h = etah sqrt(r^3/mu) grows with
-// r and falls with mu, q = hq |dv|/r grows with |dv| and falls with r, so
-// (T_ff/h)(1 - 0.75 q) >= 1 for every pair once it holds at (d, vmax,
-// mu_max).  Flyby: with T_fb/h = etah r/v and |dT/dt| <= eta (1 + mu/(r
-// v^2)), tau_fb/h >= f(r, v) = 2 etah r^2 v / ((2 + eta) r v^2 + eta mu),
-// which grows with r and falls with mu; f >= 1 holds for v between the two
-// roots v- < v+ of (2 + eta) d v^2 - 2 etah d^2 v + eta mu_max = 0.  Slow
-// pairs fall below v- (approaching bodies with |dv| -> 0 have tau -> 0 in
-// this form), so the groups are certified apart only for pairs with
-// |dv| >= v-: the function returns true when every pair has tau_ff >= h
-// and vmax <= v+, and sets vthr2 so that a pair whose high-part velocity
-// difference has |dv~|^2 >= vthr2 is certified apart (vthr adds 16 u max|v|
-// for the high parts' rounding and that of their difference: at most
-// sqrt(3) (2 u max|v| + u |dv~|) <= 9.5 u max|v|).  pad_x, pad_v bound |x - x_hi| + |x' - x'_hi|
-// over the two groups (likewise v); the 2 % margin M absorbs the FP32
-// rounding of these few operations.
-struct GroupBox {
-    float xlo[3], xhi[3], vlo[3], vhi[3];
-    float gm;    // max G m of the group (high part)
-    float amax;  // max |x_hi| component
-    float vabs;  // max |v_hi| component
-};
-
-__device__ __forceinline__ bool tau_groups_apart(const GroupBox &A, const GroupBox &B, const MixedTauParams &Q,
-                                                 float &vthr2)
-{
-    const float M = 1.02f;
-    const float pad_x = 4.f * U32 * fmaxf(A.amax, B.amax);
-    const float pad_v = 4.f * U32 * fmaxf(A.vabs, B.vabs);
-    float d2 = Q.eps2, w2 = 0.f;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        const float g = fmaxf(0.f, fmaxf(B.xlo[k] - A.xhi[k], A.xlo[k] - B.xhi[k]) - pad_x);
-        const float w = fmaxf(0.f, fmaxf(B.vhi[k] - A.vlo[k], A.vhi[k] - B.vlo[k])) + pad_v;
-        d2 = fmaf(g, g, d2);
-        w2 = fmaf(w, w, w2);
-    }
-    const float d = sqrtf(d2), vmax = sqrtf(w2);
-    const float mu = (A.gm + B.gm) * 1.0001f;
-    if (!(d > 0.f) || !(mu > 0.f)) return false;
-    // free fall at (d, vmax, mu_max)
-    const float X = Q.etah * d * sqrtf(d / mu);
-    const float q = Q.hq * vmax / d;
-    if (!(X * (1.f - 0.75f * M * q) >= M)) return false;
-    // flyby: roots of a v^2 - b v + c with the margin M on f >= 1
-    const float a = M * (2.f + Q.eta) * d, b = 2.f * Q.etah * d2, c = M * Q.eta * mu;
-    const float disc = b * b - 4.f * a * c;
-    if (!(disc > 0.f)) return false;
-    const float vp = (b + sqrtf(disc)) / (2.f * a);
-    const float vm = c / (a * vp);  // the product of the roots is c/a
-    if (!(vmax <= vp * 0.9999f)) return false;
-    const float vt = vm * 1.0001f + 4.f * pad_v;
-    vthr2 = vt * vt;
-    return true;
-}
-
-// The same two bounds for single pairs of the groups, as three comparisons on
-// r~^2 and |dv~|^2 (no square root, no division): with T_ff/h = etah
-// sqrt(r^3/mu), f(r, v) as above and mu <= mu_max,
-//   (3) r >= c v,  c = M (2 + eta) / (2 etah (1 - D)):  the first term of the
-//       flyby's denominator takes the share 1 - D of its numerator, and q =
-//       hq v/r <= hq/c;
-//   (1) r >= r_min, r_min^3 = mu_max T^2, T = M/(etah (1 - 0.75 M hq/c)):
-//       free fall at that q;
-//   (2) v >= v_thr = V mu_max/r_min^2, V = M eta/(2 etah D): the flyby's second
-//       term takes the share D.
-// M = 1.02 covers the FP32 rounding and the high parts': r_min >= 1.02e3 c_x
-// and v_thr >= 1.02e3 c_v (c_x = 7.1 u max|x_i|, c_v likewise) put the
-// relative error of r~ and v~ below 1e-3 + 4.5u, of r^2 v below 4e-3.
-// The kernel forms p = r~^2 - r_min^2 and w = v~^2 - v_thr^2 by starting
-// their sums at -r_min^2 (+ eps^2) and -v_thr^2, and asks for w >= 0 and p -
-// c^2 w >= 0: that is (3) with r_min^2 - c^2 v_thr^2 to spare (r_min is
-// raised until it is not negative), and it implies (1).  Returns false when
-// the bounds cannot be used (the caller then leaves every pair open); the
-// caller has seen that all |x|, |v| are below TAU_WILD, so no sum overflows.
-constexpr float TAU_WILD = 1e15f;
-struct PairBounds {
-    float p0, w0;  // eps^2 - r_min^2, -v_thr^2
-};
-
-__device__ __forceinline__ bool tau_pair_bounds(float amax, float vabs, float mu_max, const MixedTauBounds &Q,
-                                                PairBounds &b)
-{
-    const float mu = mu_max * 1.0001f;
-    const float r3 = mu * Q.pb_r3;
-    // r_min by exp2(log2/3): the approximations' error is far inside 5e-4
-    float rmin = 1.0005f * exp2f(__log2f(r3) * (1.f / 3.f));
-    rmin = fmaxf(rmin, fmaxf(1.02e3f * 7.1f * U32 * amax, 1e-15f));
-    float vt = fmaxf(1.0001f * Q.pb_v * mu / (rmin * rmin), fmaxf(1.02e3f * 7.1f * U32 * vabs, 1e-15f));
-    const float w2 = vt * vt, p2 = fmaxf(rmin * rmin, 1.0001f * Q.pb_c2 * w2);
-    b.p0 = Q.eps2 - p2;
-    b.w0 = -w2;
-    return Q.pb_c2 >= 0.f && r3 > 1e-36f && r3 < 1e36f && w2 < 1e30f && p2 < 1e30f;
-}
-
-// the FP32 constants of a split at threshold P.h
-inline MixedTauBounds mixed_tau_params(const TauParams &P)
-{
-    MixedTauBounds Q;
-    const double etah = P.eta_outside ? P.eta_in * P.eta / P.h : P.eta_in / P.h;
-    const double hq = P.eta_outside ? P.h / P.eta : P.h;  // h/eta_in in the units of T: eta_in/etah
-    Q.eta = (float)P.eta_in;
-    Q.etah = (float)etah;
-    Q.eps2 = (float)P.eps2;
-    Q.G = (float)P.G;
-    Q.hq = (float)hq;
-    // D: a 3 % tighter (3) at the usual eta; more where eta is not small
-    const double M = 1.02, D = fmax(1.0 / 32, 0.75 * P.eta_in / (2.0 + P.eta_in));
-    const double c = M * (2.0 + P.eta_in) / (2.0 * etah * (1.0 - D));
-    const double q = hq / c, T = M / (etah * (1.0 - 0.75 * M * q));
-    Q.pb_c2 = (float)(c * c * 1.0001);
-    Q.pb_r3 = (float)(T * T * 1.0001);
-    Q.pb_v = (float)(M * P.eta_in / (2.0 * etah * D) * 1.0001);
-    // (q >= 4/(3M) has no free-fall bound; constants outside the float range)
-    if (!(0.75 * M * q < 0.95) || !(Q.pb_c2 < 1e30f) || !(Q.pb_r3 < 1e36f) || !(Q.pb_v < 1e36f)) Q.pb_c2 = -1.f;
-    return Q;
-}
-
-__device__ __forceinline__ int tau_decide_fp32(float dx0, float dx1, float dx2, float dv0, float dv1, float dv2,
-                                               float mu, float c_x, float c_v, const MixedTauParams &Q)
-{
-    return tau_decide_at(tau_prep_fp32(dx0, dx1, dx2, dv0, dv1, dv2, mu, c_x, c_v, Q), Q.etah);
-}
 
 // 2^k as a float (0 <= k <= 127); 2^-k as a double (0 <= k <= 1022)
 __device__ __forceinline__ float pow2f(int k) { return __int_as_float((127 + k) << 23); }

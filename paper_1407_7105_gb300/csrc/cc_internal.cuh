@@ -7,6 +7,7 @@
 #include <utility>
 
 #include "../../include/cc.h"
+#include "cc_tau32.cuh"
 
 namespace cc {
 
@@ -105,12 +106,6 @@ struct SmallParams {
     double G, eps2, eta, eta_in, h0, near_tol, h_fp64;
     int eta_outside, kepler, precision, depth0, max_depth;
     int hold;  // HOLD split: a set's members with an edge form one fast set
-};
-
-struct TauParams {
-    double G, eps2, eta_in, eta, h, near_tol;
-    int eta_outside;
-    int fault_test;  // failure-path test hooks of the tau kernels (cc_params.fault_test)
 };
 
 // --------------------------------------------------------------- helpers

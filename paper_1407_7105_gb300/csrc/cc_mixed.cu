@@ -20,36 +20,6 @@
 
 namespace cc {
 
-// two packed FP32 values; the operations round each half as the scalar ones do
-__device__ __forceinline__ uint64_t pack2(float a, float b)
-{
-    uint64_t v;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(a), "f"(b));
-    return v;
-}
-__device__ __forceinline__ void unpack2(uint64_t v, float &a, float &b)
-{
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
-}
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
-{
-    uint64_t d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b)
-{
-    uint64_t d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
-{
-    uint64_t d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-
 // ------------------------------------------------------------ prep
 // float-float copy of the packed state; per-level maxima of |x| and |v|
 __global__ void k_prep_ff(Level L, FFView F, float G, int with_v, int init_forest, unsigned long long *edge_count)
@@ -268,20 +238,18 @@ __device__ __forceinline__ void box_empty(GroupBox &B)
 }
 
 // adds one body to box B; returns whether it is outside what the bounds
-// allow for (TAU_WILD, a mass that is not positive and finite, NaN)
+// allow for (tau_in_box)
 __device__ __forceinline__ bool box_add(GroupBox &B, const float s[6], float gm)
 {
-    bool in = gm > 0.f && gm < 1e30f;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         B.xlo[k] = fminf(B.xlo[k], s[k]);
         B.xhi[k] = fmaxf(B.xhi[k], s[k]);
         B.vlo[k] = fminf(B.vlo[k], s[3 + k]);
         B.vhi[k] = fmaxf(B.vhi[k], s[3 + k]);
-        in = in && fabsf(s[k]) < TAU_WILD && fabsf(s[3 + k]) < TAU_WILD;
     }
     B.gm = fmaxf(B.gm, gm);
-    return !in;
+    return !tau_in_box(s, gm);
 }
 
 // local union-find in shared memory (indices 0..2T-1, links to the smaller)
@@ -609,9 +577,7 @@ __global__ void __launch_bounds__(T *S / R, 768 * R / (T * S))
                     for (int r = 0; r < R; ++r) {
                         const uint64_t dx = add2(a.x, nx[r][0]), dy = add2(a.y, nx[r][1]), dz = add2(b.x, nx[r][2]);
                         const uint64_t du = add2(b.y, nx[r][3]), dv = add2(c.x, nx[r][4]), dw = add2(c.y, nx[r][5]);
-                        const uint64_t pp = fma2(dz, dz, fma2(dy, dy, fma2(dx, dx, p0)));
-                        const uint64_t ww = fma2(dw, dw, fma2(dv, dv, fma2(du, du, w0)));
-                        const uint64_t oo = fma2(ww, nc2, pp) | ww;  // sign bits: open
+                        const uint64_t oo = tau_pair_open(dx, dy, dz, du, dv, dw, p0, w0, nc2);
                         m[r] = __funnelshift_l((uint32_t)oo, m[r], 1);
                         m[r] = __funnelshift_l((uint32_t)(oo >> 32), m[r], 1);
                     }
@@ -625,7 +591,7 @@ __global__ void __launch_bounds__(T *S / R, 768 * R / (T * S))
 #pragma unroll
                     for (int r = 0; r < R; ++r) {
                         const uint64_t du = add2(b, nx[r][3]), dv = add2(c.x, nx[r][4]), dw = add2(c.y, nx[r][5]);
-                        const uint64_t ww = fma2(dw, dw, fma2(dv, dv, fma2(du, du, w0)));
+                        const uint64_t ww = tau_speed_open(du, dv, dw, w0);
                         m[r] = __funnelshift_l((uint32_t)ww, m[r], 1);
                         m[r] = __funnelshift_l((uint32_t)(ww >> 32), m[r], 1);
                     }

@@ -1,0 +1,234 @@
+"""The certified FP32 decision of the edge predicate and the tests that certify
+pairs and groups apart (csrc/cc_tau32.cuh), compiled for the host and compared
+with the predicate in 64 bits: what they settle is what the predicate says, on
+pairs over many scales of separation and speed (a third head on, a third slowly
+approaching), at thresholds far from a pair's tau and next to it, and at the
+thresholds h 2^-m that follow from one preparation."""
+import os
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+SRC = r'''
+#include <cstdio>
+#include <cstdlib>
+#include <random>
+#include "cc_tau32.cuh"
+namespace cc { float est_shift = 0.0f; }
+using namespace cc;
+static std::mt19937_64 g(11);
+static double uni(double a, double b) { return a + (b - a) * ((g() >> 11) * 0x1p-53); }
+static double gauss()
+{
+    static std::normal_distribution<double> d;
+    return d(g);
+}
+struct Body { double s[6], m; };
+
+// tau(i,j), the 64-bit predicate's operations
+static double tau64(const Body &a, const Body &b, const TauParams &P)
+{
+    double r2 = 0, v2 = 0, rv = 0;
+    for (int k = 0; k < 3; ++k) {
+        const double x = a.s[k] - b.s[k], v = a.s[3 + k] - b.s[3 + k];
+        r2 += x * x; v2 += v * v; rv += x * v;
+    }
+    r2 += P.eps2;
+    const double r = std::sqrt(r2), mu = P.G * (a.m + b.m);
+    const double T = P.eta_in * std::sqrt(r2 * r / mu), d = 1.5 * T * rv / r2;
+    double t = T / (1.0 - 0.5 * (d < 1.0 ? d : 1.0));
+    if (v2 > 0.0) {
+        const double F = P.eta_in * (r / std::sqrt(v2)), e = F * (rv / r2) * (1.0 + mu / (r * v2));
+        const double f = F / (1.0 - 0.5 * (e < 1.0 ? e : 1.0));
+        t = t < f ? t : f;
+    }
+    return P.eta_outside ? P.eta * t : t;
+}
+static float hi_of(double x) { return (float)x; }
+static float diff(double a, double b)  // b - a from the float pairs
+{
+    const float ah = (float)a, al = (float)(a - (double)ah), bh = (float)b, bl = (float)(b - (double)bh);
+    return (bh - ah) + (bl - al);
+}
+static float big(const Body &a, int q)
+{
+    return std::fmax(std::fabs(hi_of(a.s[q])), std::fmax(std::fabs(hi_of(a.s[q + 1])), std::fabs(hi_of(a.s[q + 2]))));
+}
+static float gm_of(const Body &a, const MixedTauParams &Q) { return Q.G * (float)a.m; }
+static int decide(const Body &a, const Body &b, const MixedTauParams &Q, int m)
+{
+    const float c11 = 11.f * U32 * U32;
+    const TauPrep32 t = tau_prep_fp32(diff(a.s[0], b.s[0]), diff(a.s[1], b.s[1]), diff(a.s[2], b.s[2]),
+                                      diff(a.s[3], b.s[3]), diff(a.s[4], b.s[4]), diff(a.s[5], b.s[5]),
+                                      gm_of(a, Q) + gm_of(b, Q), c11 * fmaxf(big(a, 0), big(b, 0)),
+                                      c11 * fmaxf(big(a, 3), big(b, 3)), Q);
+    return tau_decide_at(t, Q.etah * (float)std::ldexp(1.0, m));
+}
+static bool quick(const Body &a, const Body &b, const MixedTauParams &Q)
+{
+    float d[6];
+    for (int k = 0; k < 6; ++k) d[k] = hi_of(b.s[k]) - hi_of(a.s[k]);
+    return tau_quick_apart(d[0], d[1], d[2], d[3], d[4], d[5], gm_of(a, Q) + gm_of(b, Q), 7.1f * U32 * big(a, 0),
+                           7.1f * U32 * big(a, 3), Q);
+}
+static GroupBox box_of(const Body *b, int n, const MixedTauParams &Q, bool &in)
+{
+    GroupBox B;
+    in = true;
+    for (int k = 0; k < 3; ++k) { B.xlo[k] = B.vlo[k] = HUGE_VALF; B.xhi[k] = B.vhi[k] = -HUGE_VALF; }
+    B.gm = B.amax = B.vabs = 0.f;
+    for (int i = 0; i < n; ++i) {
+        float s[6];
+        for (int k = 0; k < 6; ++k) s[k] = hi_of(b[i].s[k]);
+        for (int k = 0; k < 3; ++k) {
+            B.xlo[k] = fminf(B.xlo[k], s[k]); B.xhi[k] = fmaxf(B.xhi[k], s[k]);
+            B.vlo[k] = fminf(B.vlo[k], s[3 + k]); B.vhi[k] = fmaxf(B.vhi[k], s[3 + k]);
+        }
+        B.gm = fmaxf(B.gm, gm_of(b[i], Q));
+        B.amax = fmaxf(B.amax, big(b[i], 0));
+        B.vabs = fmaxf(B.vabs, big(b[i], 3));
+        in = in && tau_in_box(s, gm_of(b[i], Q));
+    }
+    return B;
+}
+static long bad = 0, settled = 0, asked = 0, apart = 0, pairs_apart = 0, speeds = 0;
+static void wrong(const char *what, const Body &a, const Body &b, double tau, double h, const TauParams &P)
+{
+    if (++bad > 8) return;
+    double r2 = 0, v2 = 0;
+    for (int k = 0; k < 3; ++k) {
+        r2 += (a.s[k] - b.s[k]) * (a.s[k] - b.s[k]);
+        v2 += (a.s[3 + k] - b.s[3 + k]) * (a.s[3 + k] - b.s[3 + k]);
+    }
+    printf("%s: tau/h %g r %g v %g mu %g h %g eps2 %g\n", what, tau / h, std::sqrt(r2), std::sqrt(v2), P.G * (a.m + b.m),
+           h, P.eps2);
+}
+
+// argv: trials, outside, eta, G, L, M, V, eps, scatter (decades by which each
+// trial moves its own length, mass, speed and G)
+int main(int, char **argv)
+{
+    const long n = atol(argv[1]);
+    const int outside = atoi(argv[2]);
+    const double eta = atof(argv[3]), G0 = atof(argv[4]), L0 = atof(argv[5]), M0 = atof(argv[6]), V0 = atof(argv[7]);
+    const double eps = atof(argv[8]), sc = atof(argv[9]);
+    for (long it = 0; it < n; ++it) {
+        auto dec = [&]() { return std::pow(10.0, uni(-sc, sc)); };
+        TauParams P{};
+        P.G = G0 * dec();
+        const double L = L0 * dec(), M = M0 * dec(), V = V0 * dec();
+        P.eps2 = eps * L * eps * L;
+        P.eta = eta;
+        P.eta_in = outside ? 1.0 : eta;
+        P.eta_outside = outside;
+        // a group of 4 and one of 8 bodies: each around a point, 0.01..10 apart
+        Body a[4], b[8];
+        const double X = std::exp(uni(-6, 6)), U = std::exp(uni(-6, 3)), sep = std::exp(uni(-7, 2)), sp = std::exp(uni(-10, 1));
+        const double in = sep * std::exp(uni(-6, 0)), iv = sp * std::exp(uni(-6, 0));
+        double c[6], d[6], nd = 0;
+        for (int k = 0; k < 6; ++k) { c[k] = (k < 3 ? X : U) * uni(-1, 1); d[k] = gauss(); }
+        for (int k = 0; k < 3; ++k) nd += d[k] * d[k];
+        if (it % 3 == 0) for (int k = 0; k < 3; ++k) d[3 + k] = -d[k] / std::sqrt(nd);  // head on
+        if (it % 3 == 1) for (int k = 0; k < 3; ++k) d[3 + k] = -1e-3 * d[k];           // slowly
+        for (int i = 0; i < 12; ++i) {
+            Body &q = i < 4 ? a[i] : b[i - 4];
+            for (int k = 0; k < 6; ++k) {
+                const double off = (i < 4 ? 0.0 : (k < 3 ? sep : sp) * d[k]) + (k < 3 ? in : iv) * 0.3 * gauss();
+                q.s[k] = (k < 3 ? L : V) * (c[k] + off);
+            }
+            q.m = M * std::exp(uni(-3, 3));
+            if (it % 5 == 0) for (int k = 3; k < 6; ++k) q.s[k] = V * U;  // at rest together
+        }
+        // thresholds: next to one pair's tau, and far from it
+        const double t0 = tau64(a[0], b[0], P);
+        const double f[8] = {1.0 + 1e-5, 1.0 - 1e-5, 1.01, 0.97, 0.5, 2.0, std::exp(uni(-14, 14)), std::exp(uni(-40, 40))};
+        for (double q : f) {
+            P.h = t0 * q;
+            if (!(P.h > 1e-290) || !(P.h < 1e290)) continue;
+            const MixedTauBounds Q = mixed_tau_params(P);
+            for (int i = 0; i < 4; ++i)
+                for (int j = 0; j < 8; ++j) {
+                    if (i && j) continue;  // one row, one column
+                    const double t = tau64(a[i], b[j], P);
+                    for (int m = 0; m < 60; m = 2 * m + 1) {
+                        const int e = decide(a[i], b[j], Q, m);
+                        ++asked;
+                        settled += e >= 0;
+                        if (e >= 0 && e != (int)(t < std::ldexp(P.h, -m))) wrong("decision", a[i], b[j], t, std::ldexp(P.h, -m), P);
+                    }
+                    if (quick(a[i], b[j], Q)) {
+                        ++apart;
+                        if (t < P.h) wrong("quick", a[i], b[j], t, P.h, P);
+                    }
+                }
+            bool ia, ib;
+            const GroupBox A = box_of(a, 4, Q, ia), B = box_of(b, 8, Q, ib);
+            if (!ia || !ib) continue;
+            float thr;
+            if (tau_groups_apart(A, B, Q, thr)) {
+                const uint64_t w0 = pack2(-thr, -thr);
+                for (auto &p : a)
+                    for (auto &r : b) {
+                        uint64_t e[3];
+                        for (int k = 0; k < 3; ++k) {
+                            const float x = hi_of(r.s[3 + k]) - hi_of(p.s[3 + k]);
+                            e[k] = pack2(x, x);
+                        }
+                        if (tau_speed_open(e[0], e[1], e[2], w0) >> 63) continue;
+                        ++speeds;
+                        if (tau64(p, r, P) < P.h) wrong("group", p, r, tau64(p, r, P), P.h, P);
+                    }
+            }
+            PairBounds bd;
+            if (tau_pair_bounds(A.amax, A.vabs, A.gm + B.gm, Q, bd)) {
+                for (auto &p : a)
+                    for (auto &r : b) {
+                        uint64_t e[6];
+                        for (int k = 0; k < 6; ++k) {
+                            const float x = hi_of(r.s[k]) - hi_of(p.s[k]);
+                            e[k] = pack2(x, x);
+                        }
+                        if (tau_pair_open(e[0], e[1], e[2], e[3], e[4], e[5], pack2(bd.p0, bd.p0), pack2(bd.w0, bd.w0),
+                                          pack2(-Q.pb_c2, -Q.pb_c2)) >> 63)
+                            continue;
+                        ++pairs_apart;
+                        if (tau64(p, r, P) < P.h) wrong("pair", p, r, tau64(p, r, P), P.h, P);
+                    }
+            }
+        }
+    }
+    printf("settled %ld of %ld, apart: quick %ld, pair %ld, speed %ld; wrong %ld\n", settled, asked, apart, pairs_apart,
+           speeds, bad);
+    return bad != 0;
+}
+'''
+
+
+@pytest.fixture(scope="module")
+def harness(tmp_path_factory):
+    d = tmp_path_factory.mktemp("tau32")
+    (d / "t.cpp").write_text(SRC)
+    subprocess.run(["g++", "-O2", "-std=c++17", "-ffp-contract=off", "-x", "c++", "-I",
+                    os.path.join(ROOT, "paper_1407_7105_gb300", "csrc"), str(d / "t.cpp"), "-o", str(d / "t")],
+                   check=True)
+
+    def run(n, outside=0, eta=0.03, G=1.0, L=1.0, M=1e-4, V=1.0, eps=0.0, scatter=0.0):
+        r = subprocess.run([str(d / "t"), *map(repr, (n, outside, eta, G, L, M, V, eps, scatter))], capture_output=True,
+                           text=True)
+        assert r.returncode == 0, r.stdout
+        w = r.stdout.split()
+        return {"settled": int(w[1]) / int(w[3].rstrip(",")), "quick": int(w[6].rstrip(",")),
+                "pair": int(w[8].rstrip(",")), "speed": int(w[10].rstrip(";"))}
+
+    return run
+
+
+@pytest.mark.parametrize("outside", [0, 1])
+@pytest.mark.parametrize("eta", [0.0025, 0.03, 0.4])
+@pytest.mark.parametrize("eps", [0.0, 1 / 256])
+def test_nbody_units(harness, outside, eta, eps):
+    got = harness(3000, outside=outside, eta=eta, eps=eps)
+    # (and they do settle: most decisions, and some of each certificate)
+    assert got["settled"] > 0.7 and got["quick"] and got["pair"] and got["speed"], got
