@@ -35,6 +35,38 @@ __device__ __forceinline__ int first_level_at_or_below(double tau, double h, int
     return m < levels ? m : levels;
 }
 
+// The first m in [m0, levels) at which the wide decision says no edge at
+// h 2^-m; `levels` if every one is an edge; -1 when it leaves one open (or
+// there are more than a hundred: 2^m is a float).
+__device__ __forceinline__ int tau_wide_level(const TauWide &w, int m0, int levels)
+{
+    for (int m = m0; m < levels; ++m) {
+        if (m > 100) return -1;
+        const int dec = tau_decide_wide(w, w.etah * pow2f(m));
+        if (dec < 0) return -1;
+        if (dec == 0) return m;
+    }
+    return levels;
+}
+
+// What the FP32 decision left open at h 2^-m0: the first of the thresholds up
+// to h 2^-levels that the pair is no edge at (e), from the decision in the pair's
+// own units, else (e = -1) the FP64 tau.
+struct TauOpen {
+    double tau;
+    int e;
+};
+__device__ __forceinline__ TauOpen tau_open(double dx0, double dx1, double dx2, double dv0, double dv1, double dv2,
+                                            double mi, double mj, const TauParams &P, double h, int m0, int levels)
+{
+    const double dx[3] = {dx0, dx1, dx2}, dv[3] = {dv0, dv1, dv2};
+    TauOpen o;
+    o.tau = 0.0;
+    o.e = tau_wide_level(tau_wide(dx, dv, mi, mj, P, h), m0, levels);
+    if (o.e < 0) o.tau = tau_fp64(dx0, dx1, dx2, dv0, dv1, dv2, mi, mj, P);
+    return o;
+}
+
 // Float-float split of a double: hi = fl32(x) (round to nearest even),
 // lo = fl32(x - hi).  For |x| in [2^-74, 2^127) it is computed with integer
 // operations and int->float conversions (the significand rounded to 24

@@ -312,70 +312,82 @@ __device__ __forceinline__ int tau_decide_pair(const Level &L, const FFView &F, 
             d[c] = (jh - ih) + (jl - il);
             big[c / 3] = fmaxf(big[c / 3], fmaxf(fabsf(ih), fabsf(jh)));
         }
-        return tau_decide_fp32(d[0], d[1], d[2], d[3], d[4], d[5], Q.G * fl32(L.m[i]) + Q.G * fl32(L.m[j]),
-                               c11 * big[0], c11 * big[1], Q);
+        return tau_decide_own(d, Q.G * fl32(L.m[i]) + Q.G * fl32(L.m[j]), c11 * big[0], c11 * big[1], Q);
     } else {
         const float4 a0 = F.pq[2 * i], a1 = F.pq[2 * i + 1], b0 = F.vq[2 * i], b1 = F.vq[2 * i + 1];
         const float4 p0 = F.pq[2 * j], p1 = F.pq[2 * j + 1], v0 = F.vq[2 * j], v1 = F.vq[2 * j + 1];
-        return tau_decide_fp32((p0.x - a0.x) + (p1.x - a1.x), (p0.y - a0.y) + (p1.y - a1.y),
-                               (p0.z - a0.z) + (p1.z - a1.z), (v0.x - b0.x) + (v1.x - b1.x),
-                               (v0.y - b0.y) + (v1.y - b1.y), (v0.z - b0.z) + (v1.z - b1.z), a0.w + p0.w,
-                               c11 * F.maxes[0], c11 * F.maxes[1], Q);
+        const float d[6] = {(p0.x - a0.x) + (p1.x - a1.x), (p0.y - a0.y) + (p1.y - a1.y), (p0.z - a0.z) + (p1.z - a1.z),
+                            (v0.x - b0.x) + (v1.x - b1.x), (v0.y - b0.y) + (v1.y - b1.y), (v0.z - b0.z) + (v1.z - b1.z)};
+        return tau_decide_own(d, a0.w + p0.w, c11 * F.maxes[0], c11 * F.maxes[1], Q);
     }
 }
 
-// Settles the warp's queued pairs sm.q[w][0..cnt), one per lane: the
-// certified FP32 decision on the float-float differences, the exact FP64
-// predicate when it is undecided, then the local union; edges join the warp's
-// list of edges to record (ne of them so far).  Out of line: the pair loop
-// keeps only the high parts and its masks in registers.
-template <int T, int S, int R, bool RAW>
-__device__ __noinline__ uint2 tau_settle_batch(MixedTauSmem<T, S, R> &sm, int w, int cnt, int ne, int ibase, int j0,
-                                              int joff,
-                                              const Level &L, const FFView &F, const TauParams &P,
-                                              const MixedTauParams &Q, DevCounters *ctr, int32_t *near_ij,
-                                              double *near_tau, long long near_cap, const EdgeList &E)
+// an edge of each lane with `edge`: the local union, and a place in the warp's list
+// of edges to record (ne of them so far); returns those lanes
+template <int T, int S, int R>
+__device__ __forceinline__ unsigned tau_edges(MixedTauSmem<T, S, R> &sm, int w, bool edge, unsigned ent, double tau,
+                                              int ne, int joff, DevCounters *ctr, const EdgeList &E)
 {
-    // returns (lanes whose pair is an edge, FP64 evaluations of this lane's pair)
-    const int lane = threadIdx.x & 31;
-    const unsigned lt = (1u << lane) - 1u;
-    const bool has = lane < cnt;
-    const unsigned ent = has ? sm.q[w][lane] : 0u;
-    const int ii = (int)(ent >> 8), kk = (int)(ent & 255u);
-    int dec = 0;
-    unsigned nfp64 = 0u;
-    double tau = CUDART_NAN;
-    if (has) {
-        const int gi = ibase + ii, gj = j0 + kk;
-        dec = tau_decide_pair<RAW>(L, F, Q, gi, gj);
-        if (dec < 0) {
-            // undecided: the exact FP64 predicate
-            tau = tau_fp64(__dsub_rn(L.x[gi], L.x[gj]), __dsub_rn(L.y[gi], L.y[gj]), __dsub_rn(L.z[gi], L.z[gj]),
-                           __dsub_rn(L.vx[gi], L.vx[gj]), __dsub_rn(L.vy[gi], L.vy[gj]),
-                           __dsub_rn(L.vz[gi], L.vz[gj]), L.m[gi], L.m[gj], P);
-            nfp64 = 1u;
-            if (fabs(tau - P.h) < P.near_tol * P.h) {
-                const unsigned long long q = atomicAdd(&ctr->near_pairs, 1ull);
-                if ((long long)q < near_cap) {
-                    const int pi = L.gid[gi], pj = L.gid[gj];
-                    near_ij[2 * q] = pi < pj ? pi : pj;
-                    near_ij[2 * q + 1] = pi < pj ? pj : pi;
-                    near_tau[q] = tau;
-                }
-            }
-            dec = tau < P.h ? 1 : 0;
-        }
-    }
-    const bool edge = dec > 0;
+    const unsigned lt = (1u << (threadIdx.x & 31)) - 1u;
     const unsigned eb = __ballot_sync(0xffffffffu, edge);
-    if (eb == 0u) return make_uint2(0u, nfp64);
-    if (edge && !luf_union(sm.lp, ii, joff + kk)) raise_err(ctr, DERR_UF_RETRY);
+    if (edge && !luf_union(sm.lp, (int)(ent >> 8), joff + (int)(ent & 255u))) raise_err(ctr, DERR_UF_RETRY);
     if (edge && E.rec) {
         const int q = ne + __popc(eb & lt);
         sm.ent[w][q] = ent;
         sm.tau[w][q] = tau;
     }
-    return make_uint2(eb, nfp64);
+    return eb;
+}
+
+// Settles the warp's queued pairs sm.q[w][0..cnt), one per lane, by the certified
+// FP32 decision on the float-float differences.  Out of line: the pair loop
+// keeps only the high parts and its masks in registers.  Returns (lanes whose
+// pair is an edge, lanes whose pair is undecided: for tau_settle_open).
+template <int T, int S, int R, bool RAW>
+__device__ __noinline__ uint2 tau_settle_batch(MixedTauSmem<T, S, R> &sm, int w, int cnt, int ne, int ibase, int j0,
+                                               int joff, const Level &L, const FFView &F, const MixedTauParams &Q,
+                                               DevCounters *ctr, const EdgeList &E)
+{
+    const int lane = threadIdx.x & 31;
+    const bool has = lane < cnt;
+    const unsigned ent = has ? sm.q[w][lane] : 0u;
+    int dec = 0;
+    if (has) dec = tau_decide_pair<RAW>(L, F, Q, ibase + (int)(ent >> 8), j0 + (int)(ent & 255u));
+    const unsigned ub = __ballot_sync(0xffffffffu, dec < 0);
+    return make_uint2(tau_edges(sm, w, dec > 0, ent, CUDART_NAN, ne, joff, ctr, E), ub);
+}
+
+// The undecided ones of them (lanes ub) by the exact FP64 predicate (logged when
+// near the threshold).  Returns (lanes whose pair is an edge, FP64 evaluations of
+// this lane's pair).  Apart from the batch above, which is the common one.
+template <int T, int S, int R>
+__device__ __noinline__ uint2 tau_settle_open(MixedTauSmem<T, S, R> &sm, int w, unsigned ub, int ne, int ibase, int j0,
+                                              int joff, const Level &L, const TauParams &P, DevCounters *ctr,
+                                              int32_t *near_ij, double *near_tau, long long near_cap, const EdgeList &E)
+{
+    const int lane = threadIdx.x & 31;
+    const unsigned ent = (ub >> lane) & 1u ? sm.q[w][lane] : 0u;
+    bool edge = false;
+    unsigned nfp64 = 0u;
+    double tau = CUDART_NAN;
+    if ((ub >> lane) & 1u) {
+        const int gi = ibase + (int)(ent >> 8), gj = j0 + (int)(ent & 255u);
+        tau = tau_fp64(__dsub_rn(L.x[gi], L.x[gj]), __dsub_rn(L.y[gi], L.y[gj]), __dsub_rn(L.z[gi], L.z[gj]),
+                       __dsub_rn(L.vx[gi], L.vx[gj]), __dsub_rn(L.vy[gi], L.vy[gj]), __dsub_rn(L.vz[gi], L.vz[gj]),
+                       L.m[gi], L.m[gj], P);
+        nfp64 = 1u;
+        if (fabs(tau - P.h) < P.near_tol * P.h) {
+            const unsigned long long q = atomicAdd(&ctr->near_pairs, 1ull);
+            if ((long long)q < near_cap) {
+                const int pi = L.gid[gi], pj = L.gid[gj];
+                near_ij[2 * q] = pi < pj ? pi : pj;
+                near_ij[2 * q + 1] = pi < pj ? pj : pi;
+                near_tau[q] = tau;
+            }
+        }
+        edge = tau < P.h;
+    }
+    return make_uint2(tau_edges(sm, w, edge, ent, tau, ne, joff, ctr, E), nfp64);
 }
 
 // Records the warp's ne listed edges (the decision at h/2 is left to the first
@@ -523,7 +535,7 @@ __global__ void __launch_bounds__(T *S / R, 768 * R / (T * S))
     if (lane < GW) {
         const GroupBox &B = sm.jb[slice * GW + lane];
         float4 g = make_float4(0.f, 0.f, __int_as_float(TAU_OPEN), A.gm + B.gm);
-        if (!awild && A.gm > 0.f && B.gm > 0.f && B.gm < 1e30f) {
+        if (!awild && B.gm >= 0.f && B.gm < CUDART_INF_F) {
             float thr;
             PairBounds b;
             if (!diag && tau_groups_apart(A, B, Q, thr)) {
@@ -540,12 +552,9 @@ __global__ void __launch_bounds__(T *S / R, 768 * R / (T * S))
     __syncwarp();
     const uint64_t nc2 = pack2(-Q.pb_c2, -Q.pb_c2);
     int qn = 0, ne = 0;  // pairs queued, edges listed by this warp (warp-uniform)
-    auto settle = [&](int cnt) {
-        const uint2 c = tau_settle_batch<T, S, R, RAW>(sm, w, cnt, ne, ibase, j0, joff, L, F, P, Q, ctr, near_ij,
-                                                       near_tau, near_cap, E);
-        const int k = __popc(c.x);
+    auto listed = [&](unsigned eb) {  // edges just listed: counted, recorded when there are many
+        const int k = __popc(eb);
         my_edges += lane == 0 ? k : 0;
-        my_fp64 += c.y;
         if (!E.rec) return;
         ne += k;
         __syncwarp();
@@ -553,6 +562,16 @@ __global__ void __launch_bounds__(T *S / R, 768 * R / (T * S))
             tau_record<T, S, R>(sm, w, ne, ibase, j0, E);
             __syncwarp();
             ne = 0;
+        }
+    };
+    auto settle = [&](int cnt) {
+        const uint2 c = tau_settle_batch<T, S, R, RAW>(sm, w, cnt, ne, ibase, j0, joff, L, F, Q, ctr, E);
+        listed(c.x);
+        if (c.y != 0u) {
+            const uint2 d = tau_settle_open<T, S, R>(sm, w, c.y, ne, ibase, j0, joff, L, P, ctr, near_ij, near_tau,
+                                                     near_cap, E);
+            my_fp64 += d.y;
+            listed(d.x);
         }
     };
     const int kb = slice * TC, k1 = min(jn, kb + TC);

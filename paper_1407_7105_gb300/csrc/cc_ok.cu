@@ -27,15 +27,15 @@ __host__ __device__ inline MixedTauParams ok_q(const TauParams &P)
 {
     MixedTauParams Q;
     Q.eta = (float)P.eta_in;
-    Q.etah = (float)(P.eta_outside ? P.eta_in * P.eta / P.h : P.eta_in / P.h);
+    Q.etah = mixed_etah(P.eta_in, P.eta, P.eta_outside, P.h, P.G, P.eps2);
     Q.eps2 = (float)P.eps2;
     Q.G = (float)P.G;
     Q.hq = 0.f;
     return Q;
 }
 
-// tau(a,b) < P.h from the rounded FP64 differences (a < b): certified FP32,
-// else the FP64 tau (logged when within near_tol of the pivot; ++nfp64)
+// tau(a,b) < P.h from the rounded FP64 differences (a < b): certified FP32, also
+// in the pair's own units, else the FP64 tau (logged when within near_tol of the pivot; ++nfp64)
 __device__ __forceinline__ bool ok_fast(const double *x, const double *y, const double *z, const double *vx,
                                         const double *vy, const double *vz, const double *m, const int32_t *gid,
                                         int a, int b, const TauParams &P, const MixedTauParams &Q, DevCounters *ctr,
@@ -48,8 +48,10 @@ __device__ __forceinline__ bool ok_fast(const double *x, const double *y, const 
                                       Q.G * (fl32(m[a]) + fl32(m[b])), 0.f, 0.f, Q);
     const int dec = tau_decide_at(t, Q.etah);
     if (dec >= 0) return dec > 0;
+    const TauOpen o = tau_open(dx0, dx1, dx2, dv0, dv1, dv2, m[a], m[b], P, P.h, 0, 1);
+    if (o.e >= 0) return o.e > 0;
     ++nfp64;
-    const double tau = tau_fp64(dx0, dx1, dx2, dv0, dv1, dv2, m[a], m[b], P);
+    const double tau = o.tau;
     if (fabs(tau - P.h) < P.near_tol * P.h) {
         const unsigned long long z = atomicAdd(&ctr->near_pairs, 1ull);
         if ((long long)z < near_cap) {

@@ -170,10 +170,10 @@ __global__ void __launch_bounds__(T) k_tau_hook(Level L, TauParams P, DevCounter
 //   edge depth comes from its e, else its FP64 tau, else (an FP32-certified
 //   edge of a fresh mixed split) from certified FP32 decisions at 2h, h,
 //   h/2, ... on the parent's float-float copy, which the first half leaves
-//   untouched, with the FP64 tau from the parent level's state at the first
-//   undecided threshold; near-threshold pairs are logged, and the edges at h
-//   become this split's records (depth carried on, so deeper first halves
-//   never need a float-float copy);
+//   untouched, continued from the parent level's FP64 state at the first
+//   undecided threshold (tau_wide, then the FP64 tau); near-threshold pairs
+//   are logged, and the edges at h become this split's records (depth carried
+//   on, so deeper first halves never need a float-float copy);
 //   k_edges_hook: union-find hooking of this split's records, a compact list
 //   (a fraction of the parent's), so the pointer chasing of the hooks runs
 //   in about one wave (the list holds at least as many records as the
@@ -223,12 +223,18 @@ __global__ void k_edges_filter(EdgeList PE, long long pcount, Level PL, FFView P
                     e = m;
                 } else {
                     const int i = r.a, j = r.b;
-                    tau = tau_fp64(__dsub_rn(PL.x[i], PL.x[j]), __dsub_rn(PL.y[i], PL.y[j]),
-                                   __dsub_rn(PL.z[i], PL.z[j]), __dsub_rn(PL.vx[i], PL.vx[j]),
-                                   __dsub_rn(PL.vy[i], PL.vy[j]), __dsub_rn(PL.vz[i], PL.vz[j]), PL.m[i], PL.m[j], P);
-                    ++my_evals;
-                    const int e64 = first_level_at_or_below(tau, hp, EDGE_E_INF);
-                    e = e64 > m ? e64 : m;
+                    const TauOpen o = tau_open(__dsub_rn(PL.x[i], PL.x[j]), __dsub_rn(PL.y[i], PL.y[j]),
+                                               __dsub_rn(PL.z[i], PL.z[j]), __dsub_rn(PL.vx[i], PL.vx[j]),
+                                               __dsub_rn(PL.vy[i], PL.vy[j]), __dsub_rn(PL.vz[i], PL.vz[j]),
+                                               PL.m[i], PL.m[j], P, hp, m, EDGE_E_INF);
+                    if (o.e >= 0) {
+                        e = o.e;
+                    } else {
+                        tau = o.tau;
+                        ++my_evals;
+                        const int e64 = first_level_at_or_below(tau, hp, EDGE_E_INF);
+                        e = e64 > m ? e64 : m;
+                    }
                 }
             }
             if (tau == tau) log_pair(P, tau, C.gid[a], C.gid[b], ctr, near_ij, near_tau, near_cap);

@@ -82,10 +82,10 @@ __device__ __forceinline__ void k8_drift(double st[7], double dt, bool exact)
 // (undecided tau, Kepler pairs, FP64 kicks): kept out of the lockstep loop
 // so that its hot code stays compact in the instruction cache (a warp of
 // this kernel mostly runs alone on its scheduler and waits on fetches).
-__device__ __noinline__ double tau_fp64_ool(double dx0, double dx1, double dx2, double dv0, double dv1, double dv2,
-                                            double mi, double mj, const TauParams &P)
+__device__ __noinline__ TauOpen tau_open_ool(double dx0, double dx1, double dx2, double dv0, double dv1, double dv2,
+                                             double mi, double mj, const TauParams &P, double h, int m0, int levels)
 {
-    return tau_fp64(dx0, dx1, dx2, dv0, dv1, dv2, mi, mj, P);
+    return tau_open(dx0, dx1, dx2, dv0, dv1, dv2, mi, mj, P, h, m0, levels);
 }
 
 struct K8Acc {
@@ -159,12 +159,12 @@ __device__ __forceinline__ int edge_depth_fp64(double tau, double h, int levels,
 }
 
 // mixed form: certified FP32 decisions from one prep (etah = eta/h) while
-// they settle the threshold; at the first undecided threshold the FP64 tau
-// (tau64(), evaluated once) settles the rest.  used64 reports whether it ran.
+// they settle the threshold; at the first undecided threshold m open(m)
+// (tau_open_ool) settles the rest.  used64 reports whether that took the FP64 tau.
 // The FP32 decisions agree with the FP64 predicate wherever they are taken,
 // so the result is the FP64 predicate's edge depth.
-template <class TauF, class LogF>
-__device__ __forceinline__ int edge_depth_mixed(const TauPrep32 &t, float etah, double h, int levels, TauF tau64,
+template <class OpenF, class LogF>
+__device__ __forceinline__ int edge_depth_mixed(const TauPrep32 &t, float etah, double h, int levels, OpenF open,
                                                 LogF log, bool &used64)
 {
     used64 = false;
@@ -172,8 +172,10 @@ __device__ __forceinline__ int edge_depth_mixed(const TauPrep32 &t, float etah, 
         const int dec = tau_decide_at(t, etah * pow2f(m));
         if (dec > 0) continue;
         if (dec == 0) return m;
+        const TauOpen o = open(m);
+        if (o.e >= 0) return o.e;
         used64 = true;
-        const int e = edge_depth_fp64(tau64(), h, levels, log);
+        const int e = edge_depth_fp64(o.tau, h, levels, log);
         return e > m ? e : m;
     }
     return levels;
@@ -237,7 +239,10 @@ __device__ unsigned pair_path(double A[7], double B[7], double h0, int depth0, i
             bool used64;
             e = edge_depth_mixed(
                 t, Q.etah * pow2f(d), scale2m(h0, d), max(dmax - d + 1, 1),
-                [&]() { return tau_fp64_ool(dx0, dx1, dx2, dv0, dv1, dv2, A[6], B[6], P); },
+                [&](int m) {
+                    return tau_open_ool(dx0, dx1, dx2, dv0, dv1, dv2, A[6], B[6], P, scale2m(h0, d), m,
+                                        max(dmax - d + 1, 1));
+                },
                 [&](double tv, double hm) { near_log(tv, hm, nl.tol, nl.ctr, ga, gb, nl.ij, nl.tau, nl.cap); },
                 used64);
             pc.fp64 += used64 ? 1 : 0;
@@ -324,7 +329,10 @@ __device__ unsigned pair_path_rel(double A[7], double B[7], double h0, int depth
             bool used64;
             e = edge_depth_mixed(
                 t, etah0 * pow2f(d), scale2m(h0, d), max(dmax - d + 1, 1),
-                [&]() { return tau_fp64_ool(r[0], r[1], r[2], u[0], u[1], u[2], ma, mb, P); },
+                [&](int m) {
+                    return tau_open_ool(r[0], r[1], r[2], u[0], u[1], u[2], ma, mb, P, scale2m(h0, d), m,
+                                        max(dmax - d + 1, 1));
+                },
                 [&](double tv, double hm) { near_log(tv, hm, nl.tol, nl.ctr, ga, gb, nl.ij, nl.tau, nl.cap); },
                 used64);
             pc.fp64 += used64 ? 1 : 0;
@@ -466,7 +474,7 @@ __device__ __forceinline__ void small_task(K8Warp &S, const SView V, const int32
     Q.eta = (float)SP.eta_in; Q.eps2 = (float)SP.eps2; Q.G = (float)SP.G;
     Q.hq = 0.f;  // (the pre-test is not used here)
     // eta/h0 in float, once: eta/(h0 2^-k) is this times 2^k exactly
-    const float etah_c = (float)(SP.eta_outside ? SP.eta_in * SP.eta / h0 : SP.eta_in / h0);
+    const float etah_c = mixed_etah(SP.eta_in, SP.eta, SP.eta_outside, h0, SP.G, SP.eps2);
     const bool act = lane < n;
     const int p = act ? mem[lane] : -1;
     double st[7] = {0, 0, 0, 0, 0, 0, 0};
@@ -511,14 +519,14 @@ __device__ __forceinline__ void small_task(K8Warp &S, const SView V, const int32
                 const float etah = etah_c * pow2f(k);
                 const float c11 = 11.f * U32 * U32;
                 const int levels = K8_MAXD - k;
-                // FP64 tau of pair (lane, j), in the pair's fixed order
+                // pair (lane, j) from the FP64 state, in the pair's fixed order
                 // (symmetric bit for bit)
-                auto tau64_of = [&](int j) {
+                auto open_of = [&](int j, int m) {
                     const int lo = lane < j ? lane : j, hi = lane < j ? j : lane;
-                    return tau_fp64_ool(__dsub_rn(S.d[0][lo], S.d[0][hi]), __dsub_rn(S.d[1][lo], S.d[1][hi]),
+                    return tau_open_ool(__dsub_rn(S.d[0][lo], S.d[0][hi]), __dsub_rn(S.d[1][lo], S.d[1][hi]),
                                     __dsub_rn(S.d[2][lo], S.d[2][hi]), __dsub_rn(S.d[3][lo], S.d[3][hi]),
                                     __dsub_rn(S.d[4][lo], S.d[4][hi]), __dsub_rn(S.d[5][lo], S.d[5][hi]),
-                                    S.d[6][lo], S.d[6][hi], P);
+                                    S.d[6][lo], S.d[6][hi], P, h, m, levels);
                 };
                 auto log_of = [&](int j, double tv, double hm) {
                     if (lane < j) near_log(tv, hm, nl.tol, nl.ctr, S.gid[lane], S.gid[j], nl.ij, nl.tau, nl.cap);
@@ -551,7 +559,7 @@ __device__ __forceinline__ void small_task(K8Warp &S, const SView V, const int32
                         if (tau_decide_at(t, etah) != 0) {
                             bool used64;
                             e = edge_depth_mixed(
-                                t, etah, h, levels, [&]() { return tau64_of(j); },
+                                t, etah, h, levels, [&](int m) { return open_of(j, m); },
                                 [&](double tv, double hm) { log_of(j, tv, hm); }, used64);
                             if (used64 && lane < j) ++cn.fp64;
                         }
@@ -969,13 +977,13 @@ __device__ void km_split(KMShared<W> &sh, KMFrame &F, const SView V, const Small
     Q.eta = (float)SP.eta_in; Q.eps2 = (float)SP.eps2; Q.G = (float)SP.G;
     Q.hq = 0.f;
     const float c11 = 11.f * U32 * U32;
-    // the FP64 tau of positions lo < hi, in that order (the other kernels'
+    // positions lo < hi from the FP64 state, in that order (the other kernels'
     // pair order; symmetric bit for bit)
-    auto tau64 = [&](int lo, int hi) {
+    auto open_of = [&](int lo, int hi) {
         const int a = F.sl[lo], b = F.sl[hi];
-        return tau_fp64_ool(__dsub_rn(V.x[a], V.x[b]), __dsub_rn(V.y[a], V.y[b]), __dsub_rn(V.z[a], V.z[b]),
+        return tau_open_ool(__dsub_rn(V.x[a], V.x[b]), __dsub_rn(V.y[a], V.y[b]), __dsub_rn(V.z[a], V.z[b]),
                             __dsub_rn(V.vx[a], V.vx[b]), __dsub_rn(V.vy[a], V.vy[b]),
-                            __dsub_rn(V.vz[a], V.vz[b]), V.m[a], V.m[b], P);
+                            __dsub_rn(V.vz[a], V.vz[b]), V.m[a], V.m[b], P, h, 0, 1);
     };
     bool uf_ok = true;
     auto edge_found = [&](int p, int j) {
@@ -987,7 +995,9 @@ __device__ void km_split(KMShared<W> &sh, KMFrame &F, const SView V, const Small
         }
     };
     auto decide64 = [&](int p, int j) {
-        const double tau = tau64(p, j);
+        const TauOpen o = open_of(p, j);
+        if (o.e >= 0) return o.e > 0;
+        const double tau = o.tau;
         ++cn.fp64;
         near_log(tau, h, nl.tol, nl.ctr, V.gid[F.sl[p]], V.gid[F.sl[j]], nl.ij, nl.tau, nl.cap);
         return tau < h;
@@ -1252,7 +1262,7 @@ __device__ void medium_task(KMShared<W> &sh, const SView V, const int32_t *mem, 
 {
     constexpr int KM_T = W * 32;
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    const float etah0 = (float)(SP.eta_outside ? SP.eta_in * SP.eta / h0 : SP.eta_in / h0);
+    const float etah0 = mixed_etah(SP.eta_in, SP.eta, SP.eta_outside, h0, SP.G, SP.eps2);
     auto frame_at = [&](int k, const int32_t *sl, int n, double h, int depth) {
         KMFrame &F = sh.fr[k];
         char *b = fs + (size_t)k * KM_FRAME_BYTES;

@@ -98,8 +98,28 @@ inline uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
 // certainly false when T~(1-eT)(1-s) >= h (D~ + dD); the slack s = 2e-6
 // covers the FP32 evaluation of the bounds and the FP64 predicate's own
 // rounding.  Any NaN/Inf fails both tests: the pair is undecided.
+//
+// Range.  The model holds while no quantity overflows and none that carries
+// the result loses bits below the normal floats.  So a pair stays undecided
+// unless r^2 >= TAU_TINY, mu >= TAU_MU_MIN and r mu is finite; its flyby term
+// is used from |dv|^2 >= TAU_TINY on; and eta/h is NaN, which leaves every pair
+// undecided, unless the constants lie in the ranges that mixed_etah asks for.
+// Then, with 1/r <= 1e15, s2 <= 1e15 and s1 <= 3.2e18:
+//   an infinite r^2 or |dv|^2 makes its root's product NaN; what else overflows
+//   (rv, mu/v^2) makes dD infinite or NaN, and its term proves nothing;
+//   a term that underflows was below 2^-126 beside a sum above 1e-30, and the
+//   float-float roundings of 2^-149 are far below u r and u |dv|;
+//   T/h, a product left to right, is too small only when the true one is below
+//   1e-19 (D - dD is not: dD covers u D).  It may overflow early: T_ff is then
+//   above a finite D all the same (etah r^2 >= 3.4e38 > 0.75 eta |rv|, whose
+//   double did not overflow), an infinite T_fb proves nothing (tau_decide_at);
+//   below |dv|^2 = TAU_TINY |dv| counts as 1e-15, so that drv holds all of c_v (an
+//   FP32 difference of zero may hide one of that size).
+// With G <= 1e14 TAU_MU_MIN is above tau_mu_floor.  A pair that this leaves undecided is looked
+// at once more in units of its own (tau_wide).
 constexpr float U32 = 5.9604645e-8f;  // 2^-24
 constexpr float SLACK = 2e-6f;
+constexpr float TAU_TINY = 1e-30f, TAU_HUGE = 1e37f, TAU_MU_MIN = 1e-22f;
 
 // eta and eta/h in float (the decision compares T/h with D); c_x = 11 u^2 X
 // and c_v = 11 u^2 V carry the float-float rounding of the differences
@@ -112,6 +132,20 @@ struct MixedTauParams {
 struct MixedTauBounds : MixedTauParams {
     float pb_c2, pb_r3, pb_v;
 };
+
+// eta/h in float: NaN, which settles no pair in any test of this file, when a
+// constant is outside the range that they hold in
+CC_HD float mixed_etah(double eta_in, double eta, int eta_outside, double h, double G, double eps2)
+{
+    const float etah = (float)(eta_outside ? eta_in * eta / h : eta_in / h);
+    const float e = (float)eta_in, g = (float)G, s = (float)eps2;
+    const bool in = etah >= 1e-30f && etah <= 1e30f && e >= 1e-5f && e <= 1e3f && g >= 1e-30f && g <= 1e14f && s <= TAU_HUGE;
+    return in ? etah : nan_32();
+}
+
+// mu from which its float is good to the model's u (a mass below the normal floats
+// is off by up to 2^-150).  The tests that only need mu from above take no less.
+CC_HD float tau_mu_floor(const MixedTauParams &Q) { return 1e-36f * fmaxf(1.f, Q.G); }
 
 // The h-independent part of the decision: everything except T/h.  The
 // decision at a threshold h then costs two products and four comparisons,
@@ -135,10 +169,12 @@ CC_HD TauPrep32 tau_prep_fp32(float dx0, float dx1, float dx2, float dv0, float 
     const float rv = fmaf(dx2, dv2, fmaf(dx1, dv1, dx0 * dv0));
     const float rinv = rsqrt_32(r2);
     const float r = r2 * rinv;
-    const float s1 = rsqrt_32(r * mu);
+    const float rm = r * mu;
+    const float s1 = rsqrt_32(rm);
+    const bool in = r2 >= TAU_TINY && mu >= TAU_MU_MIN && rm <= 3.4e38f;  // (NaN is out)
     const float er = fmaf(c_x, rinv, 2.05f * U32);
-    const float s2 = v2 > 0.f ? rsqrt_32(v2) : 0.f;
-    const float vn = v2 * s2;  // |dv|
+    const float w2 = fmaxf(v2, TAU_TINY), s2 = rsqrt_32(w2);
+    const float vn = w2 * s2;  // |dv|
     const float ev = fmaf(c_v, s2, 2.05f * U32);
     const float drv = (er + ev + 4.f * U32) * (r * vn);
     // free fall: T/h = (eta/h) r2 s1, dT/dt = 1.5 eta rv s1
@@ -146,7 +182,7 @@ CC_HD TauPrep32 tau_prep_fp32(float dx0, float dx1, float dx2, float dv0, float 
     const float Dff = fmaf(-0.5f, fminf(dTff, 1.f), 1.f);
     const float dDff = fmaf(0.5f, fmaf(32.f * U32, fabsf(dTff), 1.5f * Q.eta * s1 * drv), 2.f * U32 * Dff);
     const float eff = fmaf(3.f, er, 40.f * U32);
-    t.r2 = r2;
+    t.r2 = in ? r2 : nan_32();  // out of range: T_ff/h is NaN, T_fb not used
     t.s1 = s1;
     t.r = r;
     t.s2 = s2;
@@ -157,7 +193,7 @@ CC_HD TauPrep32 tau_prep_fp32(float dx0, float dx1, float dx2, float dv0, float 
     // an exactly zero (or unresolved) FP32 velocity difference may hide a
     // tiny nonzero FP64 one, whose flyby term can be small: only a certain
     // free-fall edge decides such a pair
-    t.fb = (v2 > 0.f) && !(vn < 6.f * c_v);
+    t.fb = in && v2 >= TAU_TINY && !(vn < 6.f * c_v);
     // flyby: T/h = (eta/h) r s2, dT/dt = eta rv s2 rinv (1 + mu s2^2 rinv)
     const float g = fmaf(mu * s2 * s2, rinv, 1.f);
     const float k = s2 * rinv * g;
@@ -179,13 +215,107 @@ CC_HD int tau_decide_at(const TauPrep32 &t, float etah)
     const float Tff = etah * t.r2 * t.s1;
     const bool ff_yes = Tff * t.ffA < t.ffLo;
     if (!t.fb) return ff_yes ? 1 : -1;
-    const bool ff_no = Tff * t.ffB >= t.ffHi;
+    const bool ff_no = Tff * t.ffB > t.ffHi;  // (not when both are infinite)
     const float Tfb = etah * t.r * t.s2;
     const bool fb_yes = Tfb * t.fbA < t.fbLo;
-    const bool fb_no = Tfb * t.fbB >= t.fbHi;
+    const bool fb_no = Tfb * t.fbB > t.fbHi;
     if (ff_yes || fb_yes) return 1;
-    if (ff_no && fb_no) return 0;
+    if (ff_no && fb_no && Tfb <= 3.4e38f) return 0;
     return -1;
+}
+
+// Units of a pair's own: powers of two (exact) 2^a for lengths and 2^v for speeds
+// that bring r into [1, 4) and mu and |dv| around it: with q = log2 of mu/(r |dv|^2),
+// whatever the units, |dv|' is near 2^(-q/4) and mu' near 2^(q/2).  a, b, c: the
+// exponents of r, |dv| and mu.
+CC_HD int tau_speed_unit(int a, int b, int c, bool still, int &q)
+{
+    q = still ? 0 : c - a - 2 * b;
+    return still ? (c - a) / 2 : b + q / 4;
+}
+CC_HD int exp_of_f(float x) { return (int)((f2u(x) >> 23) & 0xffu) - 127; }  // x > 0; subnormals: below any other
+CC_HD float two_to_f(int k) { return u2f((uint32_t)(127 + k) << 23); }
+
+// The decision for one pair in units of its own, from float differences (c_x, c_v
+// as in tau_prep_fp32): what the floats hold, whatever the caller's units, is in
+// the range of the model, but for mu/(r |dv|^2) outside 2^+-140.  For the pairs
+// that the tau kernel's certificates leave open; ~30 operations more a pair.
+CC_HD int tau_decide_own(const float d[6], float mu, float c_x, float c_v, const MixedTauParams &Q)
+{
+    const float big_x = fmaxf(fabsf(d[0]), fmaxf(fabsf(d[1]), fabsf(d[2])));
+    const float big_v = fmaxf(fabsf(d[3]), fmaxf(fabsf(d[4]), fabsf(d[5])));
+    const int ax = exp_of_f(big_x), ae = Q.eps2 > 0.f ? (exp_of_f(Q.eps2) + 1) >> 1 : -127, a = ax > ae ? ax : ae;
+    const int b = exp_of_f(big_v), c = exp_of_f(mu);
+    const bool still = big_v == 0.f;
+    int q;
+    const int v = tau_speed_unit(a, b, c, still, q), te = a - v;
+    // (100: the float-float roundings of 2^-149 stay far below u r and u |dv|; an
+    // eps^2 near or below the least float, which mixed_tau_params keeps above zero,
+    // is nothing beside r^2 >= 2^-90)
+    const bool in = a >= -100 && a <= 100 && v >= -100 && v <= 100 && te >= -120 && te <= 120 && q >= -140 &&
+                    q <= 140 && (still || b >= -100) && mu >= tau_mu_floor(Q) && mu <= 3.4e38f &&
+                    (Q.eps2 == 0.f || Q.eps2 >= TAU_TINY || a >= -45);
+    if (!in) return -1;
+    const float X = two_to_f(-a), V = two_to_f(-v);
+    MixedTauParams U = Q;
+    U.etah = Q.etah * two_to_f(te);
+    U.eps2 = Q.eps2 * X * X;
+    const float m = u2f((f2u(mu) & 0x7fffffu) | ((uint32_t)(127 + c - a - 2 * v) << 23));
+    if (!(U.etah >= 1e-30f && U.etah <= 1e30f)) return -1;
+    return tau_decide_at(tau_prep_fp32(d[0] * X, d[1] * X, d[2] * X, d[3] * V, d[4] * V, d[5] * V, m, c_x * X, c_v * V, U),
+                         U.etah);
+}
+
+// The same from a pair's 64-bit differences, for pairs that the decision left
+// open: for the range of the floats, or because the float pairs do not resolve a
+// difference far from the origin (near-threshold pairs stay open as before).  For
+// pairs whose quantities the predicate's own 64-bit operations take without
+// overflow or underflow.
+struct TauWide {
+    TauPrep32 t;
+    float etah;  // eta/h in these units, for the first threshold
+    bool in;     // else every pair is open
+    bool still;  // |dv|^2 is zero in 64 bits: the predicate has no flyby term
+};
+
+// the exponent of a positive finite x; zero and subnormals: below any other
+CC_HD int exp_of(double x) { return (int)((d2u(x) >> 52) & 0x7ffu) - 1023; }
+CC_HD double two_to(int k) { return u2d((uint64_t)(1023 + k) << 52); }
+
+CC_HD TauWide tau_wide(const double dx[3], const double dv[3], double mi, double mj, const TauParams &P, double h)
+{
+    TauWide w;
+    const double mu = P.G * (mi + mj), big_x = fmax(fmax(fabs(dx[0]), fabs(dx[1])), fmax(fabs(dx[2]), sqrt(P.eps2)));
+    const double big_v = fmax(fmax(fabs(dv[0]), fabs(dv[1])), fabs(dv[2]));
+    const int a = exp_of(big_x), c = exp_of(mu), b = exp_of(big_v);
+    w.still = big_v == 0.0;
+    int q;
+    const int vb = tau_speed_unit(a, b, c, w.still, q), te = a - vb;  // the unit of time: 2^te
+    const double e = (P.eta_outside ? P.eta_in * P.eta / h : P.eta_in / h) * two_to(te < -900 ? -900 : te > 900 ? 900 : te);
+    w.in = a >= -250 && a <= 250 && c >= -250 && c <= 250 && (w.still || (b >= -250 && b <= 250)) && q >= -140 && q <= 140 &&
+           e >= 1e-30 && e <= 1e30 && P.eta_in >= 1e-5 && P.eta_in <= 1e3 && mi > 0.0 && mj > 0.0;
+    if (!w.in) return w;
+    const double X = two_to(-a), V = two_to(-vb);
+    MixedTauParams Q;
+    Q.eta = (float)P.eta_in;
+    Q.etah = w.etah = (float)e;
+    Q.eps2 = (float)(P.eps2 * X * X);
+    Q.G = 0.f;
+    Q.hq = 0.f;
+    w.t = tau_prep_fp32((float)(dx[0] * X), (float)(dx[1] * X), (float)(dx[2] * X), (float)(dv[0] * V),
+                        (float)(dv[1] * V), (float)(dv[2] * V), (float)(mu * X * V * V), 0.f, 0.f, Q);
+    return w;
+}
+
+// the decision of tau_decide_at (etah: w.etah 2^m for the threshold h 2^-m)
+CC_HD int tau_decide_wide(const TauWide &w, float etah)
+{
+    if (!w.in) return -1;
+    if (w.still) {
+        const float Tff = etah * w.t.r2 * w.t.s1;
+        return Tff * w.t.ffA < w.t.ffLo ? 1 : Tff * w.t.ffB > w.t.ffHi ? 0 : -1;
+    }
+    return tau_decide_at(w.t, etah);
 }
 
 // A sufficient test for "no edge" that skips the certified evaluation for
@@ -203,7 +333,10 @@ CC_HD int tau_decide_at(const TauPrep32 &t, float etah)
 // analogue are below 1e-4, every FP32 quantity used has relative
 // error below 1e-3 (the error model above: 40u + 3(er + ev) plus the rsqrt
 // budget), so a 2 % margin on each inequality makes the test rigorous; a
-// pair it does not settle goes to the certified decision.
+// pair it does not settle goes to the certified decision.  Out of the range
+// above nothing is certified (r mu may be too large: then T_ff = 0), nor from a
+// T that overflowed, which mu/(r v^2) may have done too.  (A larger mu makes the
+// test stricter: mu from its floor on.)
 CC_HD bool tau_quick_apart(float dx0, float dx1, float dx2, float dv0, float dv1, float dv2,
                                                 float mu, float c_x, float c_v, const MixedTauParams &Q)
 {
@@ -211,17 +344,19 @@ CC_HD bool tau_quick_apart(float dx0, float dx1, float dx2, float dv0, float dv1
     const float v2 = fmaf(dv2, dv2, fmaf(dv1, dv1, dv0 * dv0));
     const float rinv = rsqrt_ftz(r2);
     const float r = r2 * rinv;
-    const float s1 = rsqrt_ftz(r * mu);
+    const float m = fmaxf(mu, tau_mu_floor(Q)), rm = r * m;
+    const float s1 = rsqrt_ftz(rm);
     const float s2 = rsqrt_ftz(v2);   // inf for v2 = 0: rejected below
     const float vn = v2 * s2;         // |dv|
     const float Tff = Q.etah * r2 * s1;                  // T_ff / h
     const float q = Q.hq * vn * rinv;                    // h |dv| / r
     const float Tfb = Q.etah * r * s2;                   // T_fb / h
-    const float g = mu * rinv * s2 * s2;                 // mu / (r v^2)
+    const float g = m * rinv * s2 * s2;                  // mu / (r v^2)
     const float M = 1.02f;
     // (the bounds below leave 3.5u for a relative part of c_x/r, c_v/|dv|;
     // all conditions are evaluated: no short-circuit branches)
-    const bool ok = (c_x * rinv <= 0.99e-4f) & (v2 > 0.f) & (c_v * s2 <= 0.99e-4f) & (0.75f * M * q < 1.f) &
+    const bool ok = (fminf(r2, v2) >= TAU_TINY) & (rm >= 2e-38f) & (fmaxf(r2, v2) <= TAU_HUGE) &
+                    (fmaxf(Tff, Tfb) <= 3.4e38f) & (c_x * rinv <= 0.99e-4f) & (v2 > 0.f) & (c_v * s2 <= 0.99e-4f) & (0.75f * M * q < 1.f) &
                     (Tff * fmaf(-0.75f * M, q, 1.f) >= M) & (Tfb >= M * fmaf(0.5f * Q.eta, 1.f + g, 1.f));
     return ok;
 }
@@ -267,21 +402,22 @@ CC_HD bool tau_groups_apart(const GroupBox &A, const GroupBox &B, const MixedTau
         d2 = fmaf(g, g, d2);
         w2 = fmaf(w, w, w2);
     }
-    const float d = sqrtf(d2), vmax = sqrtf(w2);
-    const float mu = (A.gm + B.gm) * 1.0001f;
-    if (!(d > 0.f) || !(mu > 0.f)) return false;
+    const float d = sqrtf(d2), vmax = fmaxf(sqrtf(w2), 1e-18f);  // (squares below the floats: at most that)
+    const float mu = fmaxf((A.gm + B.gm) * 1.0001f, tau_mu_floor(Q));
+    if (!(d2 >= TAU_TINY) || !(d2 <= TAU_HUGE)) return false;
     // free fall at (d, vmax, mu_max)
     const float X = Q.etah * d * sqrtf(d / mu);
     const float q = Q.hq * vmax / d;
-    if (!(X * (1.f - 0.75f * M * q) >= M)) return false;
-    // flyby: roots of a v^2 - b v + c with the margin M on f >= 1
-    const float a = M * (2.f + Q.eta) * d, b = 2.f * Q.etah * d2, c = M * Q.eta * mu;
-    const float disc = b * b - 4.f * a * c;
-    if (!(disc > 0.f)) return false;
-    const float vp = (b + sqrtf(disc)) / (2.f * a);
-    const float vm = c / (a * vp);  // the product of the roots is c/a
+    if (!(X * (1.f - 0.75f * M * q) >= M) || !(X <= TAU_HUGE)) return false;
+    // flyby: the roots of v^2 - 2 b v + c with the margin M on f >= 1 (b is a
+    // speed: its square is in range where the speeds' are)
+    const float e = Q.etah * d2, b = e / (M * (2.f + Q.eta) * d), c = Q.eta * mu / ((2.f + Q.eta) * d);
+    const float disc = b * b - c;
+    if (!(e >= TAU_TINY) || !(disc >= TAU_TINY) || !(disc <= TAU_HUGE)) return false;
+    const float vp = b + sqrtf(disc);
+    const float vm = c / vp;
     if (!(vmax <= vp * 0.9999f)) return false;
-    const float vt = vm * 1.0001f + 4.f * pad_v;
+    const float vt = fmaxf(vm * 1.0001f + 4.f * pad_v, 1e-15f);
     vthr2 = vt * vt;
     return true;
 }
@@ -304,13 +440,14 @@ CC_HD bool tau_groups_apart(const GroupBox &A, const GroupBox &B, const MixedTau
 // c^2 w >= 0: that is (3) with r_min^2 - c^2 v_thr^2 to spare (r_min is
 // raised until it is not negative), and it implies (1).  Returns false when
 // the bounds cannot be used (the caller then leaves every pair open); the
-// caller has seen that all |x|, |v| are below TAU_WILD, so no sum overflows.
+// caller has seen that all |x|, |v| are below TAU_WILD, so no sum overflows
+// (and r3 > 1e-33 with eta >= 1e-5 keeps V mu a normal float).
 constexpr float TAU_WILD = 1e15f;
 // whether a body's high parts and G m are inside what the bounds allow for
 // (NaN is not)
 CC_HD bool tau_in_box(const float s[6], float gm)
 {
-    bool in = gm > 0.f && gm < 1e30f;
+    bool in = gm >= 0.f && gm < 1e30f;
     for (int k = 0; k < 6; ++k) in = in && fabsf(s[k]) < TAU_WILD;
     return in;
 }
@@ -322,7 +459,7 @@ struct PairBounds {
 CC_HD bool tau_pair_bounds(float amax, float vabs, float mu_max, const MixedTauBounds &Q,
                                                 PairBounds &b)
 {
-    const float mu = mu_max * 1.0001f;
+    const float mu = fmaxf(mu_max * 1.0001f, tau_mu_floor(Q));
     const float r3 = mu * Q.pb_r3;
     // r_min by exp2(log2/3): the approximations' error is far inside 5e-4
     float rmin = 1.0005f * exp2f(log2_est(r3) * (1.f / 3.f));
@@ -331,7 +468,7 @@ CC_HD bool tau_pair_bounds(float amax, float vabs, float mu_max, const MixedTauB
     const float w2 = vt * vt, p2 = fmaxf(rmin * rmin, 1.0001f * Q.pb_c2 * w2);
     b.p0 = Q.eps2 - p2;
     b.w0 = -w2;
-    return Q.pb_c2 >= 0.f && r3 > 1e-36f && r3 < 1e36f && w2 < 1e30f && p2 < 1e30f;
+    return Q.pb_c2 >= 0.f && r3 > 1e-33f && r3 < 1e36f && w2 < 1e30f && p2 < 1e30f;
 }
 
 // those sums for two columns of a row at a time (the packed differences of
@@ -355,8 +492,8 @@ inline MixedTauBounds mixed_tau_params(const TauParams &P)
     const double etah = P.eta_outside ? P.eta_in * P.eta / P.h : P.eta_in / P.h;
     const double hq = P.eta_outside ? P.h / P.eta : P.h;  // h/eta_in in the units of T: eta_in/etah
     Q.eta = (float)P.eta_in;
-    Q.etah = (float)etah;
-    Q.eps2 = (float)P.eps2;
+    Q.etah = mixed_etah(P.eta_in, P.eta, P.eta_outside, P.h, P.G, P.eps2);
+    Q.eps2 = P.eps2 > 0.0 ? fmaxf((float)P.eps2, 1e-37f) : 0.f;
     Q.G = (float)P.G;
     Q.hq = (float)hq;
     // D: a 3 % tighter (3) at the usual eta; more where eta is not small
@@ -367,14 +504,10 @@ inline MixedTauBounds mixed_tau_params(const TauParams &P)
     Q.pb_r3 = (float)(T * T * 1.0001);
     Q.pb_v = (float)(M * P.eta_in / (2.0 * etah * D) * 1.0001);
     // (q >= 4/(3M) has no free-fall bound; constants outside the float range)
-    if (!(0.75 * M * q < 0.95) || !(Q.pb_c2 < 1e30f) || !(Q.pb_r3 < 1e36f) || !(Q.pb_v < 1e36f)) Q.pb_c2 = -1.f;
+    if (!(Q.etah > 0.f) || !(0.75 * M * q < 0.95) || !(Q.pb_c2 > 1e-36f) || !(Q.pb_c2 < 1e30f) || !(Q.pb_r3 < 1e36f) ||
+        !(Q.pb_v < 1e36f))
+        Q.pb_c2 = -1.f;
     return Q;
-}
-
-CC_HD int tau_decide_fp32(float dx0, float dx1, float dx2, float dv0, float dv1, float dv2,
-                                               float mu, float c_x, float c_v, const MixedTauParams &Q)
-{
-    return tau_decide_at(tau_prep_fp32(dx0, dx1, dx2, dv0, dv1, dv2, mu, c_x, c_v, Q), Q.etah);
 }
 
 }  // namespace cc

@@ -66,6 +66,20 @@ static int decide(const Body &a, const Body &b, const MixedTauParams &Q, int m)
                                       c11 * fmaxf(big(a, 3), big(b, 3)), Q);
     return tau_decide_at(t, Q.etah * (float)std::ldexp(1.0, m));
 }
+static int own(const Body &a, const Body &b, const MixedTauParams &Q)
+{
+    const float c11 = 11.f * U32 * U32;
+    float d[6];
+    for (int k = 0; k < 6; ++k) d[k] = diff(a.s[k], b.s[k]);
+    return tau_decide_own(d, gm_of(a, Q) + gm_of(b, Q), c11 * fmaxf(big(a, 0), big(b, 0)),
+                          c11 * fmaxf(big(a, 3), big(b, 3)), Q);
+}
+static TauWide wide(const Body &a, const Body &b, const TauParams &P)
+{
+    double dx[3], dv[3];
+    for (int k = 0; k < 3; ++k) { dx[k] = a.s[k] - b.s[k]; dv[k] = a.s[3 + k] - b.s[3 + k]; }
+    return tau_wide(dx, dv, a.m, b.m, P, P.h);
+}
 static bool quick(const Body &a, const Body &b, const MixedTauParams &Q)
 {
     float d[6];
@@ -93,7 +107,7 @@ static GroupBox box_of(const Body *b, int n, const MixedTauParams &Q, bool &in)
     }
     return B;
 }
-static long bad = 0, settled = 0, asked = 0, apart = 0, pairs_apart = 0, speeds = 0;
+static long bad = 0, settled = 0, asked = 0, widely = 0, owns = 0, apart = 0, pairs_apart = 0, speeds = 0;
 static void wrong(const char *what, const Body &a, const Body &b, double tau, double h, const TauParams &P)
 {
     if (++bad > 8) return;
@@ -107,13 +121,14 @@ static void wrong(const char *what, const Body &a, const Body &b, double tau, do
 }
 
 // argv: trials, outside, eta, G, L, M, V, eps, scatter (decades by which each
-// trial moves its own length, mass, speed and G)
+// trial moves its own length, mass, speed and G), drift (a speed in units of V
+// that all bodies have in common)
 int main(int, char **argv)
 {
     const long n = atol(argv[1]);
     const int outside = atoi(argv[2]);
     const double eta = atof(argv[3]), G0 = atof(argv[4]), L0 = atof(argv[5]), M0 = atof(argv[6]), V0 = atof(argv[7]);
-    const double eps = atof(argv[8]), sc = atof(argv[9]);
+    const double eps = atof(argv[8]), sc = atof(argv[9]), drift = atof(argv[10]);
     for (long it = 0; it < n; ++it) {
         auto dec = [&]() { return std::pow(10.0, uni(-sc, sc)); };
         TauParams P{};
@@ -139,11 +154,12 @@ int main(int, char **argv)
                 q.s[k] = (k < 3 ? L : V) * (c[k] + off);
             }
             q.m = M * std::exp(uni(-3, 3));
+            for (int k = 3; k < 6; ++k) q.s[k] += V * drift;
             if (it % 5 == 0) for (int k = 3; k < 6; ++k) q.s[k] = V * U;  // at rest together
         }
         // thresholds: next to one pair's tau, and far from it
         const double t0 = tau64(a[0], b[0], P);
-        const double f[8] = {1.0 + 1e-5, 1.0 - 1e-5, 1.01, 0.97, 0.5, 2.0, std::exp(uni(-14, 14)), std::exp(uni(-40, 40))};
+        const double f[10] = {1.0 + 5e-7, 1.0 - 5e-7, 1.0 + 1e-5, 1.0 - 1e-5, 1.01, 0.97, 0.5, 2.0, std::exp(uni(-14, 14)), std::exp(uni(-40, 40))};
         for (double q : f) {
             P.h = t0 * q;
             if (!(P.h > 1e-290) || !(P.h < 1e290)) continue;
@@ -152,11 +168,20 @@ int main(int, char **argv)
                 for (int j = 0; j < 8; ++j) {
                     if (i && j) continue;  // one row, one column
                     const double t = tau64(a[i], b[j], P);
+                    const TauWide w = wide(a[i], b[j], P);
+                    const int o = own(a[i], b[j], Q);
+                    owns += o >= 0;
+                    if (o >= 0 && (std::fabs(t - P.h) < 1e-6 * P.h || o != (int)(t < P.h))) wrong("own", a[i], b[j], t, P.h, P);
                     for (int m = 0; m < 60; m = 2 * m + 1) {
-                        const int e = decide(a[i], b[j], Q, m);
+                        const double hm = std::ldexp(P.h, -m);
+                        const int e = decide(a[i], b[j], Q, m), f = tau_decide_wide(w, w.etah * (float)std::ldexp(1.0, m));
                         ++asked;
                         settled += e >= 0;
-                        if (e >= 0 && e != (int)(t < std::ldexp(P.h, -m))) wrong("decision", a[i], b[j], t, std::ldexp(P.h, -m), P);
+                        widely += f >= 0;
+                        // (within 1e-6 of the threshold a pair stays open: the log of near pairs sees it)
+                        const bool near = std::fabs(t - hm) < 1e-6 * hm;
+                        if (e >= 0 && (near || e != (int)(t < hm))) wrong("decision", a[i], b[j], t, hm, P);
+                        if (f >= 0 && (near || f != (int)(t < hm))) wrong("wide", a[i], b[j], t, hm, P);
                     }
                     if (quick(a[i], b[j], Q)) {
                         ++apart;
@@ -199,8 +224,8 @@ int main(int, char **argv)
             }
         }
     }
-    printf("settled %ld of %ld, apart: quick %ld, pair %ld, speed %ld; wrong %ld\n", settled, asked, apart, pairs_apart,
-           speeds, bad);
+    printf("settled %ld of %ld, apart: quick %ld, pair %ld, speed %ld; wide %ld own %ld; wrong %ld\n", settled, asked, apart,
+           pairs_apart, speeds, widely, owns, bad);
     return bad != 0;
 }
 '''
@@ -214,13 +239,14 @@ def harness(tmp_path_factory):
                     os.path.join(ROOT, "paper_1407_7105_gb300", "csrc"), str(d / "t.cpp"), "-o", str(d / "t")],
                    check=True)
 
-    def run(n, outside=0, eta=0.03, G=1.0, L=1.0, M=1e-4, V=1.0, eps=0.0, scatter=0.0):
-        r = subprocess.run([str(d / "t"), *map(repr, (n, outside, eta, G, L, M, V, eps, scatter))], capture_output=True,
-                           text=True)
+    def run(n, outside=0, eta=0.03, G=1.0, L=1.0, M=1e-4, V=1.0, eps=0.0, scatter=0.0, drift=0.0):
+        r = subprocess.run([str(d / "t"), *map(repr, (n, outside, eta, G, L, M, V, eps, scatter, drift))],
+                           capture_output=True, text=True)
         assert r.returncode == 0, r.stdout
         w = r.stdout.split()
         return {"settled": int(w[1]) / int(w[3].rstrip(",")), "quick": int(w[6].rstrip(",")),
-                "pair": int(w[8].rstrip(",")), "speed": int(w[10].rstrip(";"))}
+                "pair": int(w[8].rstrip(",")), "speed": int(w[10].rstrip(";")),
+                "wide": int(w[12]) / int(w[3].rstrip(",")), "own": int(w[14].rstrip(";")) * 6 / int(w[3].rstrip(","))}
 
     return run
 
@@ -232,3 +258,29 @@ def test_nbody_units(harness, outside, eta, eps):
     got = harness(3000, outside=outside, eta=eta, eps=eps)
     # (and they do settle: most decisions, and some of each certificate)
     assert got["settled"] > 0.7 and got["quick"] and got["pair"] and got["speed"], got
+
+
+@pytest.mark.parametrize("G,L,M,V", [(6.674e-8, 1.5e13, 2e33, 3e6),     # CGS, two Suns an astronomical unit apart
+                                     (6.674e-11, 1.5e11, 2e30, 3e4),    # SI, the same
+                                     (6.674e-11, 1.5e13, 8e36, 2e6),    # SI, around a body of 4e6 Suns
+                                     (6.674e-11, 1e17, 2e32, 1e3),      # SI, 100 Suns at 3 pc
+                                     (1.0, 1e-20, 1.0, 1.0), (1.0, 1e-14, 1.0, 1e7), (1.0, 1.0, 1e-40, 1e-20),
+                                     (1e35, 1.0, 1e-38, 0.1), (4e-44, 1.0, 2e30, 2e-7)])
+def test_any_units(harness, G, L, M, V):
+    """Where a product leaves the floats' range (r mu in CGS, r^2 of tiny lengths)
+    the pair is settled in units of its own, or by the 64-bit predicate."""
+    assert harness(2000, G=G, L=L, M=M, V=V)["wide"] > (0.3 if L == 1e-20 else 0.6)
+
+
+@pytest.mark.parametrize("outside", [0, 1])
+@pytest.mark.parametrize("scatter", [4, 8, 15, 20, 30, 45])
+def test_scattered_scales(harness, scatter, outside):
+    """Every trial its own length, mass, speed and G, up to 10^(+-scatter)."""
+    harness(4000, M=1.0, outside=outside, eps=0.01 * (scatter == 15), scatter=float(scatter))
+
+
+@pytest.mark.parametrize("drift", [1e6, 1e9, 1e11, 1e12, 1e13])
+def test_common_speed(harness, drift):
+    """Bodies that fly together so fast that the float pairs no longer resolve
+    their relative speeds: a difference of zero may hide one that matters."""
+    harness(8000, drift=drift, M=1.0)
