@@ -127,10 +127,10 @@ struct MixedTauParams {
     float eta, etah, eps2, G;
     float hq;  // eta/etah (h, or h/eta when eta multiplies the min): the pre-test's q = hq |dv|/r
 };
-// the tau kernel's: with tau_pair_bounds' constants (c^2, T^2, V of its bounds;
-// pb_c2 < 0: they are off)
+// the tau kernel's: with tau_pair_bounds' constants (c^2, log2 T^2 and log2 V of
+// its bounds; pb_c2 < 0: they are off)
 struct MixedTauBounds : MixedTauParams {
-    float pb_c2, pb_r3, pb_v;
+    float pb_c2, pb_lt, pb_lv;
 };
 
 // eta/h in float: NaN, which settles no pair in any test of this file, when a
@@ -441,13 +441,13 @@ CC_HD bool tau_groups_apart(const GroupBox &A, const GroupBox &B, const MixedTau
 // raised until it is not negative), and it implies (1).  Returns false when
 // the bounds cannot be used (the caller then leaves every pair open); the
 // caller has seen that all |x|, |v| are below TAU_WILD, so no sum overflows
-// (and r3 > 1e-33 with eta >= 1e-5 keeps V mu a normal float).
-constexpr float TAU_WILD = 1e15f;
+// (3 (2 TAU_WILD)^2 < 3.4e38: parsecs in SI and CGS units are inside).
+constexpr float TAU_WILD = 5e18f;
 // whether a body's high parts and G m are inside what the bounds allow for
 // (NaN is not)
 CC_HD bool tau_in_box(const float s[6], float gm)
 {
-    bool in = gm >= 0.f && gm < 1e30f;
+    bool in = gm >= 0.f && gm < 1e36f;
     for (int k = 0; k < 6; ++k) in = in && fabsf(s[k]) < TAU_WILD;
     return in;
 }
@@ -459,16 +459,17 @@ struct PairBounds {
 CC_HD bool tau_pair_bounds(float amax, float vabs, float mu_max, const MixedTauBounds &Q,
                                                 PairBounds &b)
 {
-    const float mu = fmaxf(mu_max * 1.0001f, tau_mu_floor(Q));
-    const float r3 = mu * Q.pb_r3;
-    // r_min by exp2(log2/3): the approximations' error is far inside 5e-4
-    float rmin = 1.0005f * exp2f(log2_est(r3) * (1.f / 3.f));
+    // r_min and v_thr by exp2 of sums of logarithms, which no unit takes out of
+    // the floats' range; their error (below 1e-4) is far inside the 5e-4
+    const float lm = log2_est(fmaxf(mu_max * 1.0001f, tau_mu_floor(Q)));
+    float rmin = 1.0005f * exp2f((lm + Q.pb_lt) * (1.f / 3.f));
     rmin = fmaxf(rmin, fmaxf(1.02e3f * 7.1f * U32 * amax, 1e-15f));
-    float vt = fmaxf(1.0001f * Q.pb_v * mu / (rmin * rmin), fmaxf(1.02e3f * 7.1f * U32 * vabs, 1e-15f));
+    float vt = 1.0005f * exp2f(lm + Q.pb_lv - 2.f * log2_est(rmin));
+    vt = fmaxf(vt, fmaxf(1.02e3f * 7.1f * U32 * vabs, 1e-15f));
     const float w2 = vt * vt, p2 = fmaxf(rmin * rmin, 1.0001f * Q.pb_c2 * w2);
     b.p0 = Q.eps2 - p2;
     b.w0 = -w2;
-    return Q.pb_c2 >= 0.f && r3 > 1e-33f && r3 < 1e36f && w2 < 1e30f && p2 < 1e30f;
+    return Q.pb_c2 >= 0.f && w2 < TAU_HUGE && p2 < TAU_HUGE;
 }
 
 // those sums for two columns of a row at a time (the packed differences of
@@ -501,12 +502,10 @@ inline MixedTauBounds mixed_tau_params(const TauParams &P)
     const double c = M * (2.0 + P.eta_in) / (2.0 * etah * (1.0 - D));
     const double q = hq / c, T = M / (etah * (1.0 - 0.75 * M * q));
     Q.pb_c2 = (float)(c * c * 1.0001);
-    Q.pb_r3 = (float)(T * T * 1.0001);
-    Q.pb_v = (float)(M * P.eta_in / (2.0 * etah * D) * 1.0001);
+    Q.pb_lt = (float)(2.0 * log2(T));
+    Q.pb_lv = (float)log2(M * P.eta_in / (2.0 * etah * D));
     // (q >= 4/(3M) has no free-fall bound; constants outside the float range)
-    if (!(Q.etah > 0.f) || !(0.75 * M * q < 0.95) || !(Q.pb_c2 > 1e-36f) || !(Q.pb_c2 < 1e30f) || !(Q.pb_r3 < 1e36f) ||
-        !(Q.pb_v < 1e36f))
-        Q.pb_c2 = -1.f;
+    if (!(Q.etah > 0.f) || !(0.75 * M * q < 0.95) || !(Q.pb_c2 > 1e-36f) || !(Q.pb_c2 < 1e30f)) Q.pb_c2 = -1.f;
     return Q;
 }
 
