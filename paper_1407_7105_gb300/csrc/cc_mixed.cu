@@ -248,7 +248,9 @@ __device__ __forceinline__ bool box_add(GroupBox &B, const float s[6], float gm)
         B.vlo[k] = fminf(B.vlo[k], s[3 + k]);
         B.vhi[k] = fmaxf(B.vhi[k], s[3 + k]);
     }
-    B.gm = fmaxf(B.gm, gm);
+    // (a negative mass, which only a caller's own arrays can hold, has no largest
+    // mu: no test of the group then takes its pairs)
+    B.gm = gm >= 0.f ? fmaxf(B.gm, gm) : CUDART_INF_F;
     return !tau_in_box(s, gm);
 }
 
@@ -312,7 +314,9 @@ __device__ __forceinline__ int tau_decide_pair(const Level &L, const FFView &F, 
             d[c] = (jh - ih) + (jl - il);
             big[c / 3] = fmaxf(big[c / 3], fmaxf(fabsf(ih), fabsf(jh)));
         }
-        return tau_decide_own(d, Q.G * fl32(L.m[i]) + Q.G * fl32(L.m[j]), c11 * big[0], c11 * big[1], Q);
+        // (with a negative mass the sum can cancel, and has no relative error bound)
+        const float gi = Q.G * fl32(L.m[i]), gj = Q.G * fl32(L.m[j]);
+        return tau_decide_own(d, gi >= 0.f && gj >= 0.f ? gi + gj : CUDART_NAN_F, c11 * big[0], c11 * big[1], Q);
     } else {
         const float4 a0 = F.pq[2 * i], a1 = F.pq[2 * i + 1], b0 = F.vq[2 * i], b1 = F.vq[2 * i + 1];
         const float4 p0 = F.pq[2 * j], p1 = F.pq[2 * j + 1], v0 = F.vq[2 * j], v1 = F.vq[2 * j + 1];
