@@ -584,6 +584,7 @@ static int ensure_level(cc_ctx *c, LevelAlloc &a, int need, int nsets)
 // twice the last count when a split overflowed it (up to EDGE_CAP_MAX); an
 // incomplete list only means the next first-half split evaluates tau itself.
 constexpr long long EDGE_CAP_MAX = 1ll << 22;
+static long long edge_cap_max(const cc_ctx *c) { return c->p.edge_rec_max > 0 ? (long long)c->p.edge_rec_max : EDGE_CAP_MAX; }
 
 // the edge-record count of a level, in its split summary block
 static unsigned long long *edge_count_of(const LevelAlloc &a) { return (unsigned long long *)(a.d_ncomp + 2); }
@@ -591,7 +592,7 @@ static unsigned long long *edge_count_of(const LevelAlloc &a) { return (unsigned
 static int ensure_edges(cc_ctx *c, LevelAlloc &a, long long at_least = 0)
 {
     a.E.count = edge_count_of(a);
-    const long long cap_max = c->p.edge_rec_max > 0 ? (long long)c->p.edge_rec_max : EDGE_CAP_MAX;
+    const long long cap_max = edge_cap_max(c);
     long long want = std::max<long long>(std::max<long long>(4096, 4ll * a.cap), at_least);
     if (a.ecount > a.E.cap) want = std::max(want, 2 * a.ecount);
     want = std::min(std::max(want, at_least), std::max(cap_max, at_least));
@@ -1849,7 +1850,7 @@ int cc_timestep_graph(cc_ctx *c, const int32_t *set, int64_t n_set, double h, in
     // needs the FP64 tau of every pair: one pass to count, one to write.
     const bool certified = c->p.near_tol <= GRAPH_NEAR_MAX;
     DevCounters h1;
-    auto pass = [&](bool rec) -> int {
+    auto pass = [&](const EdgeList &E) -> int {
         CC_TRY(reset_call_counters(c));
         if (certified) {
             int bin;
@@ -1858,10 +1859,10 @@ int cc_timestep_graph(cc_ctx *c, const int32_t *set, int64_t n_set, double h, in
             if (u.tau_blocks[var] > 0x7fffffff) return fail(c, CC_E_ARG, "set too large for the tile grid");
             Level L = u.L;
             L.tile_off = u.tau_off[var];
-            launch_prep_ff(u.L, u.F, c->p.G, true, c->stream, true, rec ? u.E.count : nullptr);
+            launch_prep_ff(u.L, u.F, c->p.G, true, c->stream, true, E.count);
             const int ev = ev_begin(c, 0, nullptr, timed ? TK_TAUMIX : -1, bin, var, (double)u.pairs);
             launch_tau_mixed(L, u.F, (int)u.tau_blocks[var], P, var, c->d_ctr, c->d_near_ij, c->d_near_tau,
-                             c->near_cap, rec ? u.E : EdgeList{nullptr, nullptr, 0}, c->stream);
+                             c->near_cap, E, c->stream);
             ev_end(c, ev);
         } else {
             launch_init_parent(u.L, nullptr, c->stream);
@@ -1873,8 +1874,12 @@ int cc_timestep_graph(cc_ctx *c, const int32_t *set, int64_t n_set, double h, in
         return CC_OK;
     };
     const bool rec = certified && edges_out;
-    if (rec) CC_TRY(ensure_edges(c, u));
-    CC_TRY(pass(rec));
+    EdgeList E{nullptr, nullptr, 0};
+    if (rec) {
+        CC_TRY(ensure_edges(c, u));
+        E = u.E;
+    }
+    CC_TRY(pass(E));
     const long long ne = (long long)h1.edges;
     if (n_edges) *n_edges = ne;
     if (n_near) *n_near = (long long)h1.near_pairs;
@@ -1885,18 +1890,27 @@ int cc_timestep_graph(cc_ctx *c, const int32_t *set, int64_t n_set, double h, in
     CC_CUDA(c, cudaMemsetAsync(&c->d_ctr->tau_fp64, 0, sizeof(unsigned long long), c->stream));
     CC_TRY(check_device_error(c));
     if (edges_out && ne > 0) {
-        if (rec && ne > u.E.cap) {  // more edges than records: once more, with room for all
-            CC_TRY(ensure_edges(c, u, ne));
-            CC_TRY(pass(true));
-            CC_CUDA(c, cudaMemsetAsync(&c->d_ctr->tau_fp64, 0, sizeof(unsigned long long), c->stream));
-        }
         // the edges as id pairs, sorted lexicographically
-        const size_t need = (size_t)ne * 8 + edge_sort_scratch_bytes(ne) + (size_t)n_set * 16 + 1024;
+        const size_t scratch = std::max(edge_sort_scratch_bytes(ne), (size_t)ne * sizeof(EdgeRec));
+        const size_t need = (size_t)ne * 8 + scratch + (size_t)n_set * 16 + 1024;
         CC_TRY(ensure_tmp(c, need));
         int32_t *de = (int32_t *)((char *)c->tmp + (size_t)n_set * 16);
         void *ss = (void *)(de + 2 * ne);
+        if (rec && ne > E.cap) {
+            // more edges than records: once more, into a longer list for this
+            // and the next call while a level may keep that many, else where
+            // the sort will work (a dense graph's would take as much again)
+            if (ne <= edge_cap_max(c)) {
+                u.ecount = ne;
+                CC_TRY(ensure_edges(c, u));
+            }
+            E = ne <= u.E.cap ? u.E : EdgeList{(EdgeRec *)ss, u.E.count, ne};
+            CC_TRY(pass(E));
+            CC_CUDA(c, cudaMemsetAsync(&c->d_ctr->tau_fp64, 0, sizeof(unsigned long long), c->stream));
+            CC_TRY(check_device_error(c));  // (a pass that gave up leaves records unwritten)
+        }
         if (rec) {
-            launch_ok_rec_pairs(u.E.rec, ne, u.L.gid, de, c->stream);
+            launch_ok_rec_pairs(E.rec, ne, u.L.gid, de, c->stream);
         } else {
             CC_TRY(reset_call_counters(c));
             launch_init_parent(u.L, nullptr, c->stream);
