@@ -298,14 +298,16 @@ __device__ __forceinline__ void tau_load_hi(const Level &L, const FFView &F, con
     }
 }
 
-// the certified decision of one pair from its float-float differences
-template <bool RAW>
+// the certified decision of one pair from its float-float differences; OWN: in
+// units of the pair's own
+template <bool RAW, bool OWN>
 __device__ __forceinline__ int tau_decide_pair(const Level &L, const FFView &F, const MixedTauParams &Q, int i, int j)
 {
     constexpr float c11 = 11.f * U32 * U32;
+    float d[6], mu, cx, cv;
     if constexpr (RAW) {
         const double *src[6] = {L.x, L.y, L.z, L.vx, L.vy, L.vz};
-        float d[6], big[2] = {0.f, 0.f};
+        float big[2] = {0.f, 0.f};
 #pragma unroll
         for (int c = 0; c < 6; ++c) {
             float ih, il, jh, jl;
@@ -316,14 +318,24 @@ __device__ __forceinline__ int tau_decide_pair(const Level &L, const FFView &F, 
         }
         // (with a negative mass the sum can cancel, and has no relative error bound)
         const float gi = Q.G * fl32(L.m[i]), gj = Q.G * fl32(L.m[j]);
-        return tau_decide_own(d, gi >= 0.f && gj >= 0.f ? gi + gj : CUDART_NAN_F, c11 * big[0], c11 * big[1], Q);
+        mu = gi >= 0.f && gj >= 0.f ? gi + gj : CUDART_NAN_F;
+        cx = c11 * big[0];
+        cv = c11 * big[1];
     } else {
         const float4 a0 = F.pq[2 * i], a1 = F.pq[2 * i + 1], b0 = F.vq[2 * i], b1 = F.vq[2 * i + 1];
         const float4 p0 = F.pq[2 * j], p1 = F.pq[2 * j + 1], v0 = F.vq[2 * j], v1 = F.vq[2 * j + 1];
-        const float d[6] = {(p0.x - a0.x) + (p1.x - a1.x), (p0.y - a0.y) + (p1.y - a1.y), (p0.z - a0.z) + (p1.z - a1.z),
-                            (v0.x - b0.x) + (v1.x - b1.x), (v0.y - b0.y) + (v1.y - b1.y), (v0.z - b0.z) + (v1.z - b1.z)};
-        return tau_decide_own(d, a0.w + p0.w, c11 * F.maxes[0], c11 * F.maxes[1], Q);
+        d[0] = (p0.x - a0.x) + (p1.x - a1.x);
+        d[1] = (p0.y - a0.y) + (p1.y - a1.y);
+        d[2] = (p0.z - a0.z) + (p1.z - a1.z);
+        d[3] = (v0.x - b0.x) + (v1.x - b1.x);
+        d[4] = (v0.y - b0.y) + (v1.y - b1.y);
+        d[5] = (v0.z - b0.z) + (v1.z - b1.z);
+        mu = a0.w + p0.w;
+        cx = c11 * F.maxes[0];
+        cv = c11 * F.maxes[1];
     }
+    if constexpr (OWN) return tau_decide_own(d, mu, cx, cv, Q);
+    else return tau_decide_at(tau_prep_fp32(d[0], d[1], d[2], d[3], d[4], d[5], mu, cx, cv, Q), Q.etah);
 }
 
 // an edge of each lane with `edge`: the local union, and a place in the warp's list
@@ -356,18 +368,23 @@ __device__ __noinline__ uint2 tau_settle_batch(MixedTauSmem<T, S, R> &sm, int w,
     const bool has = lane < cnt;
     const unsigned ent = has ? sm.q[w][lane] : 0u;
     int dec = 0;
-    if (has) dec = tau_decide_pair<RAW>(L, F, Q, ibase + (int)(ent >> 8), j0 + (int)(ent & 255u));
+    // (RAW: the float pairs again in the open batch would spill)
+    if (has) dec = tau_decide_pair<RAW, RAW>(L, F, Q, ibase + (int)(ent >> 8), j0 + (int)(ent & 255u));
     const unsigned ub = __ballot_sync(0xffffffffu, dec < 0);
     return make_uint2(tau_edges(sm, w, dec > 0, ent, CUDART_NAN, ne, joff, ctr, E), ub);
 }
 
-// The undecided ones of them (lanes ub) by the exact FP64 predicate (logged when
-// near the threshold).  Returns (lanes whose pair is an edge, FP64 evaluations of
-// this lane's pair).  Apart from the batch above, which is the common one.
-template <int T, int S, int R>
+// The undecided ones of them (lanes ub): the decision in the pair's own units (in
+// units far from 1 the batch above leaves every pair open), else the exact FP64
+// predicate (logged when near the threshold).  Returns (lanes whose pair is an
+// edge, FP64 evaluations of this lane's pair).  Apart from the batch above, which
+// is the common one: own units for all of its pairs took 3 % of a level by the unit
+// calls (40009 bodies, 1.73 against 1.67 ms).
+template <int T, int S, int R, bool RAW>
 __device__ __noinline__ uint2 tau_settle_open(MixedTauSmem<T, S, R> &sm, int w, unsigned ub, int ne, int ibase, int j0,
-                                              int joff, const Level &L, const TauParams &P, DevCounters *ctr,
-                                              int32_t *near_ij, double *near_tau, long long near_cap, const EdgeList &E)
+                                              int joff, const Level &L, const FFView &F, const TauParams &P,
+                                              const MixedTauParams &Q, DevCounters *ctr, int32_t *near_ij,
+                                              double *near_tau, long long near_cap, const EdgeList &E)
 {
     const int lane = threadIdx.x & 31;
     const unsigned ent = (ub >> lane) & 1u ? sm.q[w][lane] : 0u;
@@ -376,20 +393,25 @@ __device__ __noinline__ uint2 tau_settle_open(MixedTauSmem<T, S, R> &sm, int w, 
     double tau = CUDART_NAN;
     if ((ub >> lane) & 1u) {
         const int gi = ibase + (int)(ent >> 8), gj = j0 + (int)(ent & 255u);
-        tau = tau_fp64(__dsub_rn(L.x[gi], L.x[gj]), __dsub_rn(L.y[gi], L.y[gj]), __dsub_rn(L.z[gi], L.z[gj]),
-                       __dsub_rn(L.vx[gi], L.vx[gj]), __dsub_rn(L.vy[gi], L.vy[gj]), __dsub_rn(L.vz[gi], L.vz[gj]),
-                       L.m[gi], L.m[gj], P);
-        nfp64 = 1u;
-        if (fabs(tau - P.h) < P.near_tol * P.h) {
-            const unsigned long long q = atomicAdd(&ctr->near_pairs, 1ull);
-            if ((long long)q < near_cap) {
-                const int pi = L.gid[gi], pj = L.gid[gj];
-                near_ij[2 * q] = pi < pj ? pi : pj;
-                near_ij[2 * q + 1] = pi < pj ? pj : pi;
-                near_tau[q] = tau;
+        int dec = -1;
+        if constexpr (!RAW) dec = tau_decide_pair<false, true>(L, F, Q, gi, gj);
+        edge = dec > 0;
+        if (dec < 0) {
+            tau = tau_fp64(__dsub_rn(L.x[gi], L.x[gj]), __dsub_rn(L.y[gi], L.y[gj]), __dsub_rn(L.z[gi], L.z[gj]),
+                           __dsub_rn(L.vx[gi], L.vx[gj]), __dsub_rn(L.vy[gi], L.vy[gj]), __dsub_rn(L.vz[gi], L.vz[gj]),
+                           L.m[gi], L.m[gj], P);
+            nfp64 = 1u;
+            if (fabs(tau - P.h) < P.near_tol * P.h) {
+                const unsigned long long q = atomicAdd(&ctr->near_pairs, 1ull);
+                if ((long long)q < near_cap) {
+                    const int pi = L.gid[gi], pj = L.gid[gj];
+                    near_ij[2 * q] = pi < pj ? pi : pj;
+                    near_ij[2 * q + 1] = pi < pj ? pj : pi;
+                    near_tau[q] = tau;
+                }
             }
+            edge = tau < P.h;
         }
-        edge = tau < P.h;
     }
     return make_uint2(tau_edges(sm, w, edge, ent, tau, ne, joff, ctr, E), nfp64);
 }
@@ -572,8 +594,8 @@ __global__ void __launch_bounds__(T *S / R, 768 * R / (T * S))
         const uint2 c = tau_settle_batch<T, S, R, RAW>(sm, w, cnt, ne, ibase, j0, joff, L, F, Q, ctr, E);
         listed(c.x);
         if (c.y != 0u) {
-            const uint2 d = tau_settle_open<T, S, R>(sm, w, c.y, ne, ibase, j0, joff, L, P, ctr, near_ij, near_tau,
-                                                     near_cap, E);
+            const uint2 d = tau_settle_open<T, S, R, RAW>(sm, w, c.y, ne, ibase, j0, joff, L, F, P, Q, ctr, near_ij,
+                                                          near_tau, near_cap, E);
             my_fp64 += d.y;
             listed(d.x);
         }

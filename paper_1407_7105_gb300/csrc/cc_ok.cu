@@ -34,6 +34,13 @@ __host__ __device__ inline MixedTauParams ok_q(const TauParams &P)
     return Q;
 }
 
+// (out of line: its registers stay out of the lists' kernels)
+static __device__ __noinline__ TauOpen ok_open(double dx0, double dx1, double dx2, double dv0, double dv1, double dv2,
+                                               double ma, double mb, const TauParams &P)
+{
+    return tau_open(dx0, dx1, dx2, dv0, dv1, dv2, ma, mb, P, P.h, 0, 1);
+}
+
 // tau(a,b) < P.h from the rounded FP64 differences (a < b): certified FP32, also
 // in the pair's own units, else the FP64 tau (logged when within near_tol of the pivot; ++nfp64)
 __device__ __forceinline__ bool ok_fast(const double *x, const double *y, const double *z, const double *vx,
@@ -48,7 +55,7 @@ __device__ __forceinline__ bool ok_fast(const double *x, const double *y, const 
                                       Q.G * (fl32(m[a]) + fl32(m[b])), 0.f, 0.f, Q);
     const int dec = tau_decide_at(t, Q.etah);
     if (dec >= 0) return dec > 0;
-    const TauOpen o = tau_open(dx0, dx1, dx2, dv0, dv1, dv2, m[a], m[b], P, P.h, 0, 1);
+    const TauOpen o = ok_open(dx0, dx1, dx2, dv0, dv1, dv2, m[a], m[b], P);
     if (o.e >= 0) return o.e > 0;
     ++nfp64;
     const double tau = o.tau;
