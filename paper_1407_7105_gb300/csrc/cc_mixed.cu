@@ -150,7 +150,8 @@ void launch_prep_kick(const Level &L, const FFView &F, const int32_t *order, con
 // pair (tau_pair_bounds: no square root; 13 FP32 operations against ~35 and
 // three reciprocal square roots for tau_quick_apart), formed for two columns
 // at a time with the packed FP32 instructions (add/fma .f32x2: one issue slot
-// for two pairs), so a pair costs ~10 issue slots; the comparisons' outcomes
+// for two pairs), so a pair costs ~10 issue slots (~12 in cold groups, whose speed
+// bound is each pair's own: TAU_FAR); the comparisons' outcomes
 // are the sign bits of two sums, shifted into a 32-column mask per lane, so
 // there is no vote and no branch per column.  Pairs left open are queued per
 // warp and settled 32 at a time by the certified decision.
@@ -164,6 +165,17 @@ void launch_prep_kick(const Level &L, const FFView &F, const int32_t *order, con
 // RAW: the set is a caller's FP64 arrays (L.x .. L.m, L.total bodies, no
 // float-float copy): columns and rows are rounded as they are loaded.
 constexpr int TAU_JG = 8;  // columns per group of the group certificates
+// The pairs' own speed bounds (tau_pair_far, TAU_FAR: three packed operations more
+// for two pairs) from v_thr = span/16 on, the widest relative speed per component of
+// the two groups: where v_thr leaves a few pairs in a hundred open, settling them
+// takes longer than the better bound.  Measured, tau kernel, with v_thr alone / the
+// column test of before it / now: 16384-body spheres at h = 1/1024, virial ratio 0.5
+// 0.122 / 0.283 / 0.122 ms, 0.02 0.421 / 0.267 / 0.107, 0.01 0.794 / 0.267 / 0.105, 0.001
+// 0.425 / 0.267 / 0.105; 40009 bodies, 0.005 4.64 / 1.51 / 0.48; 32768-body fractal with a
+// mass spectrum, 0.3 0.755 / 1.021 / 0.352.  span/4 and span/8 were slower in all of
+// these (0.173 and 0.109 at 0.02), span/32 and span/64 within 2 %, but for hot spheres
+// (40009 bodies, 0.5: 0.49 and 0.52 against 0.48).
+constexpr float TAU_FAR_SPAN = 1.f / 256.f;
 
 template <int T, int S, int R>
 struct __align__(16) MixedTauSmem {
@@ -175,10 +187,11 @@ struct __align__(16) MixedTauSmem {
     double tau[W][128];
     GroupBox jb[T / TAU_JG];                    // boxes of the j-tile's TAU_JG-column groups
     float4 gq[W][T / S / TAU_JG];               // per warp and column group: p0, w0, what to do (TauKind), mu
+    float2 gf[W][T / S / TAU_JG];               // and a, k (TAU_FAR)
     uint64_t bar;
 };
 
-enum TauKind : int { TAU_BOUNDS = 0, TAU_SPEED = 1, TAU_OPEN = 2 };
+enum TauKind : int { TAU_BOUNDS = 0, TAU_SPEED = 1, TAU_OPEN = 2, TAU_FAR = 3 };
 
 // min / max over each aligned segment of W lanes (a whole warp: one
 // instruction)
@@ -571,6 +584,16 @@ __global__ void __launch_bounds__(T *S / R, 768 * R / (T * S))
                 g.x = b.p0;
                 g.y = b.w0;
                 g.z = __int_as_float(TAU_BOUNDS);
+                // v_thr beside the groups' speeds
+                const float span = tau_speed_span(A, B);
+                PairFar f;
+                if (TAU_FAR_SPAN * span * span < -b.w0 &&
+                    tau_pair_far(A.amax, A.vabs, fmaxf(A.amax, B.amax), span, A.gm + B.gm, Q, f)) {
+                    g.x = f.p0;
+                    g.y = f.w0;
+                    g.z = __int_as_float(TAU_FAR);
+                    sm.gf[w][lane] = make_float2(f.a, f.k);
+                }
             }
         }
         sm.gq[w][lane] = g;
@@ -627,6 +650,21 @@ __global__ void __launch_bounds__(T *S / R, 768 * R / (T * S))
                         m[r] = __funnelshift_l((uint32_t)(oo >> 32), m[r], 1);
                     }
                 }
+            } else if (kind == TAU_FAR) {
+                const float2 gf = sm.gf[w][(cb - kb) / TAU_JG + g];
+                const uint64_t p0 = pack2(gc.x, gc.x), w0 = pack2(gc.y, gc.y), fa = pack2(gf.x, gf.x), fk = pack2(gf.y, gf.y);
+#pragma unroll
+                for (int u = 0; u < TAU_JG / 2; ++u) {
+                    const ulonglong2 a = J[3 * u], b = J[3 * u + 1], c = J[3 * u + 2];
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        const uint64_t dx = add2(a.x, nx[r][0]), dy = add2(a.y, nx[r][1]), dz = add2(b.x, nx[r][2]);
+                        const uint64_t du = add2(b.y, nx[r][3]), dv = add2(c.x, nx[r][4]), dw = add2(c.y, nx[r][5]);
+                        const uint64_t oo = tau_far_open(dx, dy, dz, du, dv, dw, p0, w0, nc2, fa, fk);
+                        m[r] = __funnelshift_l((uint32_t)oo, m[r], 1);
+                        m[r] = __funnelshift_l((uint32_t)(oo >> 32), m[r], 1);
+                    }
+                }
             } else if (kind == TAU_SPEED) {
                 const uint64_t w0 = pack2(gc.y, gc.y);
 #pragma unroll
@@ -657,9 +695,10 @@ __global__ void __launch_bounds__(T *S / R, 768 * R / (T * S))
         }
         if (!__any_sync(0xffffffffu, open != 0)) continue;
         if (__reduce_add_sync(0xffffffffu, (unsigned)open) > 32u * 32u * R / 2u) {
-            // slow bodies everywhere (a cold system: v < v_thr at separations
-            // far above r_min): the full certificate column by column is
-            // cheaper than settling them all
+            // most pairs open (groups outside the bounds' range): the full
+            // certificate column by column is cheaper than settling them all.
+            // (From a quarter, an eighth or a sixteenth of the pairs on it is
+            // wasted where they are edges: 16384 bodies, h = 1/64, 1.03 -> 1.20-1.23 ms)
             for (int c = 0; c < min(32, k1 - cb); ++c) {
                 const int k = cb + c;
                 const float *h = reinterpret_cast<const float *>(sm.hp) + (k >> 1) * 12 + (k & 1);

@@ -486,6 +486,54 @@ CC_HD uint64_t tau_pair_open(uint64_t dx, uint64_t dy, uint64_t dz, uint64_t du,
     return fma2(ww, nc2, pp) | ww;
 }
 
+// The same with (2) taken at each pair's own separation: v >= V mu_max/r^2 as
+// (a p)^2 w >= a^2 (V mu_max)^2 with p = r~^2 - r_min^2 and w = v~^2 - v_fl^2, v_fl the
+// least speed that the high parts resolve (1.02e3 c_v).  p <= r^2 and w <= v^2, so it
+// implies (2) with the margin of V, and w >= 0; (3) and (1) as before, with v_fl in
+// v_thr's place.  In a cold system v_thr, which is V mu_max/r_min^2, is above most
+// speeds at separations far above r_min.  a, a power of two, keeps a p below 2^50 and
+// (a p)^2 w below 2^100 whatever the units; a product that underflows leaves its
+// pair open.  Returns false when the threshold is out of the floats' range.
+struct PairFar {
+    float p0, w0, a, k;  // eps^2 - r_min^2, -v_fl^2, a, -a^2 (V mu_max)^2
+};
+
+// xmax: both groups' largest |x_hi| component; wmax: their widest relative speed per
+// component (of the high parts)
+CC_HD bool tau_pair_far(float amax, float vabs, float xmax, float wmax, float mu_max, const MixedTauBounds &Q, PairFar &f)
+{
+    // (3.6 = log2 12: p <= 12 xmax^2 + eps^2, w <= 12 wmax^2)
+    const float lm = log2_est(fmaxf(mu_max * 1.0001f, tau_mu_floor(Q)));
+    float rmin = 1.0005f * exp2f((lm + Q.pb_lt) * (1.f / 3.f));
+    rmin = fmaxf(rmin, fmaxf(1.02e3f * 7.1f * U32 * amax, 1e-15f));
+    const float vf = fmaxf(1.02e3f * 7.1f * U32 * vabs, 1e-15f), w2 = vf * vf;
+    const float p2 = fmaxf(rmin * rmin, 1.0001f * Q.pb_c2 * w2);
+    const float lp = fmaxf(2.f * log2_est(xmax) + 3.6f, log2_est(Q.eps2)) + 1.f, lw = 2.f * log2_est(wmax) + 3.6f;
+    const float la = floorf(fminf(50.f, 50.f - 0.5f * lw) - lp), lk = 2.f * (lm + Q.pb_lv + la);
+    f.p0 = Q.eps2 - p2;
+    f.w0 = -w2;
+    f.a = exp2f(la);
+    f.k = -1.002f * exp2f(lk);
+    return Q.pb_c2 >= 0.f && p2 < TAU_HUGE && w2 < TAU_HUGE && fabsf(la) <= 120.f && lk >= fmaxf(lw, 0.f) - 110.f &&
+           lk <= 110.f;
+}
+CC_HD uint64_t tau_far_open(uint64_t dx, uint64_t dy, uint64_t dz, uint64_t du, uint64_t dv, uint64_t dw, uint64_t p0,
+                            uint64_t w0, uint64_t nc2, uint64_t a, uint64_t k)
+{
+    const uint64_t pp = fma2(dz, dz, fma2(dy, dy, fma2(dx, dx, p0)));
+    const uint64_t ww = tau_speed_open(du, dv, dw, w0), t = mul2(pp, a);
+    return fma2(ww, nc2, pp) | fma2(mul2(t, t), ww, k);
+}
+
+// the widest relative speed between two groups, per component from their boxes
+CC_HD float tau_speed_span(const GroupBox &A, const GroupBox &B)
+{
+    float w = 0.f;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) w = fmaxf(w, fmaxf(B.vhi[k] - A.vlo[k], A.vhi[k] - B.vlo[k]));
+    return w;
+}
+
 // the FP32 constants of a split at threshold P.h
 inline MixedTauBounds mixed_tau_params(const TauParams &P)
 {

@@ -107,7 +107,7 @@ static GroupBox box_of(const Body *b, int n, const MixedTauParams &Q, bool &in)
     }
     return B;
 }
-static long bad = 0, settled = 0, asked = 0, widely = 0, owns = 0, apart = 0, pairs_apart = 0, speeds = 0;
+static long bad = 0, settled = 0, asked = 0, widely = 0, owns = 0, apart = 0, pairs_apart = 0, speeds = 0, fars = 0;
 static void wrong(const char *what, const Body &a, const Body &b, double tau, double h, const TauParams &P)
 {
     if (++bad > 8) return;
@@ -222,10 +222,26 @@ int main(int, char **argv)
                         if (tau64(p, r, P) < P.h) wrong("pair", p, r, tau64(p, r, P), P.h, P);
                     }
             }
+            PairFar fr;
+            if (tau_pair_far(A.amax, A.vabs, fmaxf(A.amax, B.amax), tau_speed_span(A, B), A.gm + B.gm, Q, fr)) {
+                for (auto &p : a)
+                    for (auto &r : b) {
+                        uint64_t e[6];
+                        for (int k = 0; k < 6; ++k) {
+                            const float x = hi_of(r.s[k]) - hi_of(p.s[k]);
+                            e[k] = pack2(x, x);
+                        }
+                        if (tau_far_open(e[0], e[1], e[2], e[3], e[4], e[5], pack2(fr.p0, fr.p0), pack2(fr.w0, fr.w0),
+                                         pack2(-Q.pb_c2, -Q.pb_c2), pack2(fr.a, fr.a), pack2(fr.k, fr.k)) >> 63)
+                            continue;
+                        ++fars;
+                        if (tau64(p, r, P) < P.h) wrong("far", p, r, tau64(p, r, P), P.h, P);
+                    }
+            }
         }
     }
-    printf("settled %ld of %ld, apart: quick %ld, pair %ld, speed %ld; wide %ld own %ld; wrong %ld\n", settled, asked, apart,
-           pairs_apart, speeds, widely, owns, bad);
+    printf("settled %ld of %ld, apart: quick %ld, pair %ld, speed %ld; wide %ld own %ld; wrong %ld far %ld\n", settled, asked, apart,
+           pairs_apart, speeds, widely, owns, bad, fars);
     return bad != 0;
 }
 '''
@@ -246,7 +262,7 @@ def harness(tmp_path_factory):
         w = r.stdout.split()
         return {"settled": int(w[1]) / int(w[3].rstrip(",")), "quick": int(w[6].rstrip(",")),
                 "pair": int(w[8].rstrip(",")), "speed": int(w[10].rstrip(";")),
-                "wide": int(w[12]) / int(w[3].rstrip(",")), "own": int(w[14].rstrip(";")) * 6 / int(w[3].rstrip(","))}
+                "wide": int(w[12]) / int(w[3].rstrip(",")), "own": int(w[14].rstrip(";")) * 6 / int(w[3].rstrip(",")), "far": int(w[18])}
 
     return run
 
@@ -258,6 +274,8 @@ def test_nbody_units(harness, outside, eta, eps):
     got = harness(3000, outside=outside, eta=eta, eps=eps)
     # (and they do settle: most decisions, and some of each certificate)
     assert got["settled"] > 0.7 and got["quick"] and got["pair"] and got["speed"], got
+    # (at each pair's own separation the speed's bound certifies most of what the common one does, and more)
+    assert got["far"] > got["pair"], got
 
 
 @pytest.mark.parametrize("G,L,M,V", [(6.674e-8, 1.5e13, 2e33, 3e6),     # CGS, two Suns an astronomical unit apart
@@ -271,6 +289,8 @@ def test_any_units(harness, G, L, M, V):
     """Where a product leaves the floats' range (r mu in CGS, r^2 of tiny lengths)
     the pair is settled in units of its own, or by the 64-bit predicate."""
     got = harness(2000, G=G, L=L, M=M, V=V)
+    if G in (6.674e-8, 6.674e-11):
+        assert got["far"] > got["pair"], got
     if M == 1e-300:  # (mu outside the floats, and of 64 bits' use only as zero)
         assert got["pair"] and got["speed"]
     else:
