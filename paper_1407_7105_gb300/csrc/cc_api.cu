@@ -438,10 +438,14 @@ static int tune_pick(cc_ctx *c, int tkind, const long long *blocks, long long wo
 // of them, the tuner's choice below.  Measured per 1e6 pairs, 256 against the
 // best tuned shape: 2.1e9 pairs 0.38 / 0.40-0.48 us, 8.0e8 0.79 / 0.92, 2.5e8
 // 0.62 / 0.87; the 16384-body level (1.34e8 pairs in 14 tiles per SM, its
-// edges in the tiles on the diagonal) 1.39 / 0.82.
+// edges in the tiles on the diagonal) 1.39 / 0.82.  And at least TAU_WIDE_PAIRS
+// pairs a tile: of a small set's tiles most rows are empty.  4400 systems of 3 bodies
+// 33 / 20 us a launch, of 64 51 / 31, of 128 82 / 68, of 200 and 256 150 and 180 by both,
+// 1500 of 300 (15000 pairs a tile) 110 / 99, of 400 (26600) 141 / 156, of 512 181 / 199.
+constexpr long long TAU_WIDE_PAIRS = 20000;
 static int tau_pick(cc_ctx *c, const LevelAlloc &a, int *bin, bool *timed)
 {
-    if (a.tau_blocks[TAU_VAR_WIDE] >= 24ll * c->nsm) {
+    if (a.tau_blocks[TAU_VAR_WIDE] >= 24ll * c->nsm && a.pairs >= TAU_WIDE_PAIRS * a.tau_blocks[TAU_VAR_WIDE]) {
         *bin = 0;
         *timed = false;
         return TAU_VAR_WIDE;
