@@ -155,7 +155,7 @@ int cc_default_params(cc_params *p);
  * stream: a cudaStream_t (NULL = default stream).  Device memory grows with
  * the recursion: each depth's level buffers at first use, and for the FP64
  * kicks (the FP64 form; the mixed form below h_fp64) of levels with at least
- * 2^18 pairs and no centre-of-mass approximation, the pair forces of every
+ * 2^21 pairs and no centre-of-mass approximation, the pair forces of every
  * set (3 n^2 doubles per set; 6.4 GB for a 16384-body set), kept up to 24 GB
  * for the context's lifetime; when that allocation fails, or a level needs
  * more, the kick computes the forces in place (same results, no error).

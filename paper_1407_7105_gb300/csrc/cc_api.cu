@@ -936,11 +936,14 @@ static int com_prepare(cc_ctx *c, LevelAlloc &a)
 // 16384-body set needs 6.4 GB, a 28000-body one 18.8 GB; larger levels
 // compute the forces in the kick)
 constexpr size_t PF_BUDGET = (size_t)24 << 30;
-// levels with fewer pairs kick with the forces computed in place: the ~24
-// FP64 operations a precomputed pair saves do not pay for the second launch
-// and the offsets' upload (Plummer 256 and 1024: 20-35 % slower per step
-// with the matrices at every level)
-constexpr long long PF_MIN_PAIRS = 1LL << 18;
+// levels with fewer pairs kick with the forces computed in place: each pair twice,
+// but in one launch whose rows fill the chip sooner than the triangle's 128-wide
+// tiles, and without the offsets' upload.  Kick with the matrices / in place, ms, one
+// set of 256 bodies 0.094 / 0.022, 724 0.118 / 0.052, 1024 0.130 / 0.067, 1448 0.158 /
+// 0.124, 2048 (2^21 pairs) 0.181 / 0.169, 4096 0.408 / 0.552; 2e6 pairs in 60 sets of 256
+// 0.150 / 0.127, in 16 of 512 0.158 / 0.131, in 250 of 128 0.116 / 0.129, in 1000 of 64
+// 0.117 / 0.141; 4.2e6 in two of 2048 0.226 / 0.280.  (The same bits.)
+constexpr long long PF_MIN_PAIRS = 1LL << 21;
 
 static int ensure_kpart(cc_ctx *c, int chunks, int fcap)
 {

@@ -5,7 +5,7 @@
 //   * a first half's edges from its parent's records;
 //   * the kick K_{h,V_ij} between members of different components
 //     (Eqs. kickij, kickji; Sec. 2.2 K_{h, V_R + V_CC + V_CR}) in FP64: rows
-//     in place (k_kick64), or from 2^18 pairs each pair's force once
+//     in place (k_kick64), or from 2^21 pairs each pair's force once
 //     (k_pair_forces) and the rows summed after it (k_kick_rows);
 //   * the energy diagnostic H (Eq. Hamiltonian).
 // j-tiles are staged in shared memory by TMA bulk copies (cp.async.bulk)
