@@ -215,6 +215,42 @@ __device__ __forceinline__ void stumpff_f(float z, float &c2, float &c3)
     }
 }
 
+// The universal Kepler equation's left side (less its t = sqrt(mu) dt); it grows
+// with chi, its derivative being the separation.
+__device__ __forceinline__ double kepler_eq(double chi, double alpha, double a1, double a2, double r0n, double t)
+{
+    const double x2 = chi * chi;
+    double c2, c3;
+    stumpff(alpha * x2, c2, c3);
+    return a1 * x2 * c2 + a2 * x2 * chi * c3 + r0n * chi - t;
+}
+
+// Its root between two neighbouring doubles by bisection, for the orbits that the
+// iteration of kepler_universal does not bring to its criterion: from a start far
+// from the root near a tight pericentre (1 - e below 1e-3) it creeps, at a few
+// thousandths of the way a step, and where the derivative is small it runs round a
+// cycle of doubles about the root.  2.5e-7 of the solves of a cluster of binaries,
+// one state of 32768 bodies in a hundred.  An equation that overflows (or is NaN)
+// counts as beyond the root.
+static __device__ __noinline__ bool kepler_bisect(double alpha, double a1, double a2, double r0n, double t, double &chi)
+{
+    const double s = t < 0.0 ? -1.0 : 1.0;
+    double lo = 0.0, hi = s * fmin(fabs(t) / r0n, 1e300);
+    for (int it = 0; s * kepler_eq(hi, alpha, a1, a2, r0n, t) < 0.0; ++it) {
+        if (it == 2000) return false;
+        lo = hi;
+        hi *= 2.0;
+    }
+    for (int it = 0; it < 2000; ++it) {
+        const double mid = lo + 0.5 * (hi - lo);
+        if (mid == lo || mid == hi) break;
+        if (s * kepler_eq(mid, alpha, a1, a2, r0n, t) < 0.0) lo = mid; else hi = mid;
+    }
+    const double fl = fabs(kepler_eq(lo, alpha, a1, a2, r0n, t)), fh = fabs(kepler_eq(hi, alpha, a1, a2, r0n, t));
+    chi = fl < fh ? lo : hi;
+    return isfinite(fmin(fl, fh));
+}
+
 // Advance the relative orbit (r0, v0) under mu by dt; returns false when
 // the iteration does not converge.  The Laguerre-Conway iteration runs in
 // FP32 first (a GB300 FP64 instruction costs the pipe ~64 cycles, an FP32
@@ -284,6 +320,7 @@ __device__ __forceinline__ bool kepler_universal(const double r0[3], const doubl
     }
     double c2 = 0.5, c3 = 1.0 / 6.0, F1 = r0n;
     bool conv = false;
+    long long kept64 = -1;  // (a NaN's bits; as in FP32, a repeated chi shows a cycle)
     // Laguerre-Conway iteration (order n = 5) on the universal Kepler equation
     for (int it = 0; it < 200; ++it) {
         const double x2 = chi * chi, z = alpha * x2;
@@ -299,11 +336,15 @@ __device__ __forceinline__ bool kepler_universal(const double r0[3], const doubl
             conv = true;
             break;
         }
+        const long long b = __double_as_longlong(chi);
+        if (b == kept64) break;
+        if ((it & (it + 1)) == 0) kept64 = b;
     }
-    if (!conv) return false;
-    // one Newton polish at the converged point
-    bool moved;
-    {
+    bool moved = true;
+    if (!conv) {
+        if (!kepler_bisect(alpha, a1, a2, r0n, smu * dt, chi)) return false;
+    } else {
+        // one Newton polish at the converged point
         const double x2 = chi * chi, z = alpha * x2;
         stumpff(z, c2, c3);
         const double F = a1 * x2 * c2 + a2 * x2 * chi * c3 + r0n * chi - smu * dt;
