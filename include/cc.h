@@ -248,11 +248,12 @@ int cc_timing(cc_ctx *ctx, cc_timing_t *out);
 
 /* One cell of the launch-shape autotuner: a kernel and a size bin (the
  * launch's pair count in [2^bin, 2^(bin+1))).  Variant v of the kernel is
- * the launch shape (shape[v], slices[v]): for the tau kernels the tile edge
- * (64, 128) and the threads per tile row (its columns split in slices; the
- * largest levels run 256-wide tiles by a fixed rule and have no cell); for
- * the FP64 kick the tile edge (32, 64, 128), slices 1; for the mixed kick
- * the j-chunk in tiles of 128 and the column slices of each tile. */
+ * the launch shape (shape[v], slices[v]): for the certified tau kernel the
+ * tile edge (64, 128) and the threads per tile row (its columns split in
+ * slices; the largest levels run 256-wide tiles by a fixed rule and have no
+ * cell); for the mixed kick
+ * the j-chunk in tiles of 128 and the column slices of each tile.
+ * The FP64 kernels run in one shape and have no cells. */
 typedef struct {
     int32_t kernel;            /* CC_TUNE_TAU_FP64 .. CC_TUNE_KICK_MIXED           */
     int32_t bin;

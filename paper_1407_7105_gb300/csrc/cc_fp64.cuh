@@ -263,12 +263,11 @@ CC_HD float div_const_f(float x)
 }
 
 #ifdef __CUDACC__
-// a + b and a b as fused multiply-adds with a one and a minus zero that the
-// compiler cannot see: the same bits (a times one is exact, a sum with -0
-// keeps every value and sign), and a DFMA holds the pipe 64 cycles a warp
-// where a DADD or DMUL holds it 77 (each measured alone on it)
+// a + b as a fused multiply-add with a one that the compiler cannot see: the
+// same bits (a times one is exact), and a DFMA holds the pipe 64 cycles a warp
+// where a DADD or DMUL holds it 77 (each measured alone on it; a product is
+// __fma_rn with a minus zero, whose sum keeps every value and sign)
 __device__ __forceinline__ double add_fma(double a, double b, double one) { return __fma_rn(a, one, b); }
-__device__ __forceinline__ double mul_fma(double a, double b, double nzero) { return __fma_rn(a, b, nzero); }
 
 // rn(1 / rn(r2 rn(sqrt r2))) by the IEEE instructions: what rinv3_rn is, and
 // the way out where it does not apply

@@ -836,13 +836,14 @@ void launch_tau_raw(const double *m, const double *x3, const double *v3, int n, 
 // PACKED = false is the same operations a column at a time, for levels below
 // MK_PACKED_MIN pairs.  A column rounds alike in both, but the launch shapes do
 // not sum alike (a chunk is a partial sum), the tuner chooses between them by
-// their times, and packed arithmetic favours the long chunk by 5 to 10 %.  From
-// 2^29 pairs on chunk 4 wins by 6 to 17 % either way (chunk 4 against 1, a
-// column at a time 0.83-0.94, packed 0.79-0.93).  Below, the two lie within a few
-// per cent (32768 bodies, 2^24-pair levels: 1.03-1.06, packed 0.94-1.01), and a
-// different choice would move the last bits of a kick, which a hard binary
-// magnifies by 1e4 and more before the step is over (1.5e-8 of the velocities).
-// There the packed form would save ~20 us of a 2.8 ms step (16384 bodies).
+// their times, and packed arithmetic favours the long chunk by 3 to 8 %: the
+// choice turns with it where the two are close, and another choice moves the last
+// bits of a kick, which a hard binary magnifies by 1e4 and more before the step is
+// over (1.5e-8 of the velocities).  Chunk 4 against 1, time per pair, a column at a
+// time / packed: 2^25 pairs 1.055 / 0.988, 2^26 0.990 / 0.988, 2^27 0.958 / 0.947, 2^28
+// 0.952 / 0.933, 2^28.9 0.932 / 0.921, from 2^29 on 0.83-0.94 / 0.79-0.93.  What the line
+// costs below it: a kick of every pair of 8192 bodies takes 78 us where the packed
+// form would take 68, 16384 262 and 213, 32000 946 and 770.
 constexpr int MK_T = 128;
 constexpr int MK_CHUNK_MAX = 4;  // j-tiles per chunk (tuned per size bin)
 static_assert(MK_VAR_CHUNK[0] <= MK_CHUNK_MAX && MK_VAR_CHUNK[1] <= MK_CHUNK_MAX && MK_VAR_CHUNK[2] <= MK_CHUNK_MAX,

@@ -639,8 +639,9 @@ __global__ void __launch_bounds__(PF_THREADS, 6) k_pair_forces(Level L, double G
 // (coalesced 256-byte pieces, 48 columns ahead) and overwrites the left-out
 // terms with zero; they meet once per KW columns at a barrier of their own.
 // Four pairs a block, so every scheduler gets the same number.  24 bytes a
-// pair, 4.7 TB/s at the additions' rate.  A 16384-body step: 8.5 ms when the
-// tiles were staged by 256 threads for 96 to add, 7.9 ms so.
+// pair, 4.7 TB/s at the additions' rate.  The 15 launches of a 16384-body
+// step: 8.5 ms when the tiles were staged by 256 threads for 96 to add, 7.7 ms so
+// (ncu; the step 19.1 ms).
 constexpr int KW = 16;                      // columns a stage
 constexpr int KR_PAIRS = 4, KR_STAGES = 4;  // 16 KB a pair
 constexpr int KR_SMEM = KR_PAIRS * KR_STAGES * KW * 32 * 8;
