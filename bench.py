@@ -47,11 +47,10 @@ KICK_FLOPS = 25  # one pair force applied to both bodies (Eqs. kickij/kickji): t
                  # mixed form's row kick evaluates each pair from both sides, which is not credited (the
                  # FP64 kick evaluates each unordered pair once, k_pair_forces, and sums rows, k_kick_rows)
 # DRAM bytes (read + write) per launch of the pair kernels, averaged over the
-# launches of one step in an ncu capture (dram__bytes_read.sum +
-# dram__bytes_write.sum): profiles/launches_plummer16384_mixed.md (mixed form)
-# and profiles/k_tau_hook_k_kick64_plummer16384_fp64.md (FP64 form; the FP64
-# kick's two kernels per kick call: profiles/launches_plummer16384_fp64.md)
-KERNEL_TRAFFIC = {"k_kick_mixed": 391e3, "k_tau_mixed": 850e3, "k_pair_forces+k_kick_rows": 3.07e9, "k_tau_hook": 616e3}
+# launches of one step in an ncu capture of these kernels (dram__bytes_read.sum +
+# dram__bytes_write.sum; the FP64 kick's two kernels per kick call):
+# profiles/pair_kernels_plummer16384.md
+KERNEL_TRAFFIC = {"k_kick_mixed": 371e3, "k_tau_mixed": 733e3, "k_pair_forces+k_kick_rows": 3.11e9}
 
 
 WORKLOADS = {
@@ -485,7 +484,7 @@ def run_gpu(args, rank, world):
     roof = {"bound": "alu", "kernel": kname, "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
             "frac": (achieved / peak) if achieved else None, "traffic": KERNEL_TRAFFIC.get(kname),
             "traffic_note": ("bytes per kick call (both kernels)" if "+" in kname else "bytes per launch")
-                            + " from an ncu capture of the same kernel (profiles/)",
+                            + " from an ncu capture of the same kernel (profiles/pair_kernels_plummer16384.md)",
             "peak_source": ("FP32" if fp32 else "FP64") + " FMA throughput measured by cc_probe_peaks on this GPU "
                            "(MEASURED_PEAKS.json has no FP32/FP64 figure)",
             "algorithmic_flops_per_pair": TAU_FLOPS if kname.startswith("k_tau") else KICK_FLOPS,
